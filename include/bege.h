@@ -406,7 +406,7 @@ BEGE_API int bege_serve_destroy(bege_ctx* ctx, int32_t server_id);
  * a latency-critical loop never calls cudaMalloc/cudaFree).  It runs the
  * whole search of one segment -- spectrum, correlation with bank rows
  * [k_begin, k_end), sigma and tails -- using only the caller's buffers plus
- * one fixed scratch array inside the library (about 1.05 MiB of device
+ * one fixed scratch array inside the library (about 1.2 MiB of device
  * memory per GPU, held from library load until process exit).  It calls no
  * cudaMalloc, cudaFree or other allocating routine.
  *

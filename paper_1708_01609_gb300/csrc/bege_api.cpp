@@ -179,10 +179,12 @@ int get_plan(bege_ctx* ctx, int64_t n, std::shared_ptr<PlanHost>* out) {
   auto p = std::make_shared<PlanHost>();
   p->g = bege::make_geometry(n);
   const bege::Geometry& g = p->g;
-  // tables: tw2 [16 R0], tw3 [F], wH [256 S], wR0S [R0 S], w16S [16 S], wS [S], wN [H]
+  // tables: tw2 [16 R0], tw3 [F], wH [256 S], wR0S [R0 S], wS [S], wN [H]
   const size_t n_tw2 = 16 * g.R0, n_tw3 = g.F, n_wH = 256 * g.S, n_wR0S = g.R0 * g.S,
-               n_w16S = 16 * g.S, n_wS = g.S, n_wN = g.H;
-  std::vector<float2> h(n_tw2 + n_tw3 + n_wH + n_wR0S + n_w16S + n_wS + n_wN);
+               n_wS = g.S, n_wN = g.H;
+  size_t n_unit = 0;
+  for (int t = 0; t < bege::kUnitTables; ++t) n_unit += bege::unit_table_size(g.S, t);
+  std::vector<float2> h(n_tw2 + n_tw3 + n_wH + n_wR0S + n_wS + n_wN + n_unit);
   size_t o = 0;
   const size_t o_tw2 = o;
   for (int r = 0; r < 16; ++r)
@@ -199,15 +201,21 @@ int get_plan(bege_ctx* ctx, int64_t n, std::shared_ptr<PlanHost>* out) {
   const size_t o_wR0S = o;
   for (size_t k = 0; k < n_wR0S; ++k) h[o + k] = wexp((int64_t)k, (int64_t)g.R0 * g.S);
   o += n_wR0S;
-  const size_t o_w16S = o;
-  for (size_t k = 0; k < n_w16S; ++k) h[o + k] = wexp((int64_t)k, 16 * (int64_t)g.S);
-  o += n_w16S;
   const size_t o_wS = o;
   for (size_t k = 0; k < n_wS; ++k) h[o + k] = wexp((int64_t)k, g.S);
   o += n_wS;
   const size_t o_wN = o;
   for (size_t k = 0; k < n_wN; ++k) h[o + k] = wexp((int64_t)k, g.N);
   o += n_wN;
+  size_t o_unit[bege::kUnitTables];
+  for (int t = 0; t < bege::kUnitTables; ++t) {
+    o_unit[t] = o;
+    for (int i = 0; i < bege::unit_table_size(g.S, t); ++i, ++o) {
+      const bege::Turn a = bege::unit_table_turn(g.S, t, i);
+      const double x = 2.0 * M_PI * (double)a.num / (double)a.den;
+      h[o] = bege::rot_entry(std::cos(x), std::sin(x));
+    }
+  }
   int rc = ctx->alloc(&p->tables, h.size() * sizeof(float2));
   if (rc) return rc;
   cudaError_t e = cudaMemcpy(p->tables.ptr, h.data(), h.size() * sizeof(float2),
@@ -222,9 +230,14 @@ int get_plan(bege_ctx* ctx, int64_t n, std::shared_ptr<PlanHost>* out) {
   p->dev.tw3 = base + o_tw3;
   p->dev.wH = base + o_wH;
   p->dev.wR0S = base + o_wR0S;
-  p->dev.w16S = base + o_w16S;
   p->dev.wS = base + o_wS;
   p->dev.wN = base + o_wN;
+  p->dev.t1 = base + o_unit[0];
+  p->dev.t2 = base + o_unit[1];
+  p->dev.t3 = base + o_unit[2];
+  p->dev.u2 = base + o_unit[3];
+  p->dev.u1 = base + o_unit[4];
+  p->dev.uc = base + o_unit[5];
   ctx->plans[n] = p;
   *out = p;
   return BEGE_OK;
@@ -263,7 +276,7 @@ int segment_common(bege_ctx* ctx, const float* y_dev, int64_t n, int32_t channel
     return rc;
   }
   cudaError_t e = bege::launch_segment(plan->dev, y_dev, static_cast<float2*>(seg->D.ptr),
-                                       static_cast<float4*>(seg->AB.ptr), s);
+                                       static_cast<float4*>(seg->AB.ptr), ctx->cfg.precision != 0, s);
   if (e != cudaSuccess) {
     ctx->release(&seg->D);
     ctx->release(&seg->AB);

@@ -12,15 +12,15 @@
 // counter that the batch zeroes before each launch; clusters leave when it
 // passes the last item, so nothing waits on anything else.
 #include "bege_batch.h"
-#include "bege_corr.cuh"
+#include "bege_unit.cuh"
 
 namespace bege {
 
 namespace {
 
-constexpr int kF = 4096;
-constexpr int kNC = 2;
-constexpr int kT = 256;
+using namespace unit;
+
+constexpr int kNC = 2;          // columns of a CTA (one unit)
 constexpr int kCluster = 8;
 
 __device__ __forceinline__ int plan_index(int S) {
@@ -34,44 +34,74 @@ struct ItemState {
   int64_t k_begin, k_end;
 };
 
-// One work item.  The per-template body takes the column count S = N/8192
-// at run time, so a single copy of it serves every segment length; only the
-// S-point combine is compiled per S.  (With four per-S copies of the body the
-// kernel spills about 1 KB per thread under its 128-register budget.)
+template <int S>
+__device__ __forceinline__ void combine_group(const float2* uc, int grank, float thr, uint32_t tmpl,
+                                              int64_t krow, const TailOut& out) {
+  Combine<S, 1> cb;
+  cb.twiddles(uc, grank);
+  cb.template emit<false>(Sm<1>::rowptr(), uc, grank, thr, tmpl, krow, out, 0.f);
+}
+
+// One work item.  The stages do not depend on the column count S = N/8192, so
+// one copy of them serves every segment length; only the tables and the
+// S-point combine (compiled per S) do.
 __device__ __forceinline__ void run_item(const BatchArgs& b, const ItemState* st, int rank) {
   const int S = st->sg.S;
   const int C = S / kNC;
   const int G = kCluster / C;
+  using SM = Sm<1>;
   cg::cluster_group cluster = cg::this_cluster();
   const int group = rank / C, grank = rank - group * C, gbase = group * C;
   const PlanDev& p = b.plans[plan_index(S)];
-  setup_columns<kF, 0, kNC, kT>(p, grank, gbase, true, S);
+  setup_unit<1>(p, S, grank, 0);
+  if (threadIdx.x < C)
+    SM::rowptr()[threadIdx.x] = cluster.map_shared_rank(SM::rows(0), (unsigned)(gbase + threadIdx.x));
   __syncthreads();
   const int64_t iters = (st->k_end - st->k_begin + G - 1) / G;
   for (int64_t i = 0; i < iters; ++i) {
     const int64_t k = st->k_begin + i * G + group;
     const bool active = k < st->k_end;  // uniform over the CTAs of a group
-    if (active)
-      template_columns<kF, 0, kNC, kT, true>(grank, st->sg.bank + k * st->sg.Lp,
-                                             (int)(st->sg.Lp / 2), 1, st->sg.AB, S);
-    // a one-CTA group reads only its own columns: a CTA barrier suffices
-    if (C == 1) __syncthreads(); else cluster.sync();
+    const int64_t krow = k - st->sg.k0;
+    const TailOut out{st->sg.recs, st->sg.cap, st->sg.counter, nullptr};
     if (active) {
-      const float sigma = group_sigma_rt(Smem<kF, kNC>::sigpart(), gbase, C, S * 8192);
-      const int64_t krow = k - st->sg.k0;
-      if (grank == 0 && threadIdx.x == 0) st->sg.sigma[krow] = sigma;
-      const TailOut out{st->sg.recs, st->sg.cap, st->sg.counter, nullptr};
-      const float thr = st->sg.kappa * sigma;
-      float2* const* cp = Smem<kF, kNC>::colptr();
-      switch (S) {
-        case 2: combine_and_emit<kF, 2, kNC, kT>(cp, S * 4096, grank, thr, (uint32_t)k, krow, out, 0.f); break;
-        case 4: combine_and_emit<kF, 4, kNC, kT>(cp, S * 4096, grank, thr, (uint32_t)k, krow, out, 0.f); break;
-        case 8: combine_and_emit<kF, 8, kNC, kT>(cp, S * 4096, grank, thr, (uint32_t)k, krow, out, 0.f); break;
-        default: combine_and_emit<kF, 16, kNC, kT>(cp, S * 4096, grank, thr, (uint32_t)k, krow, out, 0.f); break;
+      stage1<1, true, false>(0, S, grank, st->sg.bank + k * st->sg.Lp, (int)(st->sg.Lp / 2), 1);
+      unit_sync<1>(0);
+      stage2<1>(0);
+      mid_enter<1>(0, grank);
+      middle<1, 1>(0, grank, st->sg.AB);
+      mid_leave<1>(0, grank);
+      stage2i<1>(0);
+      unit_sync<1>(0);
+      if (C == 1) {  // one CTA holds the template: no other CTA is waited for
+        const float share = unit_power<1>(0);
+        const float sigma = sigma_of(&share, 1, S * 2 * kF);
+        if (threadIdx.x == 0) st->sg.sigma[krow] = sigma;
+        finish_s2<false>(p.uc, st->sg.kappa * sigma, (uint32_t)k, krow, out, sigma);
+      } else {
+        stage1i<1>(0);
+        if (threadIdx.x == 0) {
+          const float share = unit_power<1>(0);
+          for (int q = 0; q < C; ++q)
+            *cluster.map_shared_rank(SM::sigall() + grank, (unsigned)(gbase + q)) = share;
+        }
       }
     }
-    // remote reads done before the columns are overwritten
-    if (C == 1) __syncthreads(); else cluster_sync_after_reads();
+    if (C == 1) continue;
+    cluster_arrive();
+    cluster_wait();  // every row and share of the group is ready
+    if (active) {
+      const float sigma = sigma_of(SM::sigall(), C, S * 2 * kF);
+      if (grank == 0 && threadIdx.x == 0) st->sg.sigma[krow] = sigma;
+      const float thr = st->sg.kappa * sigma;
+      switch (S) {
+        case 4: combine_group<4>(p.uc, grank, thr, (uint32_t)k, krow, out); break;
+        case 8: combine_group<8>(p.uc, grank, thr, (uint32_t)k, krow, out); break;
+        default: combine_group<16>(p.uc, grank, thr, (uint32_t)k, krow, out); break;
+      }
+    }
+    __syncwarp();
+    cluster_arrive_relaxed();  // every remote value has fed a vote: the reads are done
+    cluster_wait();
   }
 }
 
@@ -80,7 +110,7 @@ __global__ void __launch_bounds__(kT, 2) batch_kernel(BatchArgs b) {
   __shared__ ItemState st;
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = (int)cluster.block_rank();
-  setup_common<kF, kNC, kT>(b.plans[0]);  // F-only tables: the same for every N
+  unit::setup_common<1>(b.plans[0]);  // F-only tables: the same for every N
   for (;;) {
     if (rank == 0 && threadIdx.x == 0) item_slot = (int)atomicAdd(b.queue, 1u);
     cluster.sync();
@@ -104,10 +134,10 @@ __global__ void __launch_bounds__(kT, 1) segment_batch_kernel(BatchArgs b,
                                                              const SegJob* __restrict__ jobs) {
   const SegJob j = jobs[blockIdx.x];
   switch (j.S) {
-    case 2: segment_body<kF, 2, kNC, kT>(b.plans[0], j.rank, j.y, j.D, j.AB); break;
-    case 4: segment_body<kF, 4, kNC, kT>(b.plans[1], j.rank, j.y, j.D, j.AB); break;
-    case 8: segment_body<kF, 8, kNC, kT>(b.plans[2], j.rank, j.y, j.D, j.AB); break;
-    default: segment_body<kF, 16, kNC, kT>(b.plans[3], j.rank, j.y, j.D, j.AB); break;
+    case 2: segment_body<kF, 2, kNC, kT>(b.plans[0], j.rank, j.y, j.D, j.AB, false); break;
+    case 4: segment_body<kF, 4, kNC, kT>(b.plans[1], j.rank, j.y, j.D, j.AB, false); break;
+    case 8: segment_body<kF, 8, kNC, kT>(b.plans[2], j.rank, j.y, j.D, j.AB, false); break;
+    default: segment_body<kF, 16, kNC, kT>(b.plans[3], j.rank, j.y, j.D, j.AB, false); break;
   }
 }
 
@@ -116,7 +146,7 @@ __global__ void __launch_bounds__(kT, 1) segment_batch_kernel(BatchArgs b,
 int batch_max_clusters() {
   static int cached = -1;
   if (cached >= 0) return cached;
-  constexpr size_t smem = Lay<kF, kNC>::total;
+  constexpr size_t smem = unit::Lay<1>::total;
   if (cudaFuncSetAttribute(batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
       cudaSuccess)
     return 0;
@@ -141,7 +171,7 @@ int batch_max_clusters() {
 }
 
 cudaError_t launch_batch(const BatchArgs& b, int clusters, cudaStream_t s) {
-  constexpr size_t smem = Lay<kF, kNC>::total;
+  constexpr size_t smem = unit::Lay<1>::total;
   cudaError_t e = cudaFuncSetAttribute(batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem);
   if (e != cudaSuccess) return e;
@@ -162,7 +192,7 @@ cudaError_t launch_batch(const BatchArgs& b, int clusters, cudaStream_t s) {
 
 cudaError_t launch_segment_batch(const BatchArgs& b, const SegJob* jobs, int njobs,
                                  cudaStream_t s) {
-  constexpr size_t smem = Lay<kF, kNC>::total;
+  constexpr size_t smem = bege::Lay<kF, kNC>::total;
   cudaError_t e = cudaFuncSetAttribute(segment_batch_kernel,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;

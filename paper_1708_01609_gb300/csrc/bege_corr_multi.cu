@@ -5,26 +5,29 @@
 // L2-resident scratch, and then, for each segment, the product with that
 // segment's coefficients, the inverse transform, sigma and the tails, with
 // exactly the single-segment kernel's arithmetic.
-#include "bege_corr.cuh"
+#include "bege_unit.cuh"
 
 namespace bege {
 
 namespace {
 
-constexpr int kF = 4096;
-constexpr int kNC = 2;
-constexpr int kT = 256;
+using namespace unit;
+
 constexpr int kMinB = 2;
 
 template <int S>
 __global__ void __launch_bounds__(kT, kMinB) correlate_multi_kernel(PlanDev p, MultiArgs a) {
-  constexpr int C = ColMap<S, kNC>::C;
-  using SM = Smem<kF, kNC>;
+  constexpr int C = S / 2;
+  using SM = Sm<1>;
   cg::cluster_group cluster = cg::this_cluster();
-  const int N = p.g.N, H = p.g.H;
-  const int rank = (int)cluster.block_rank();
-  setup_common<kF, kNC, kT>(p);
-  setup_columns<kF, S, kNC, kT>(p, rank, 0, true);
+  const int rank = C == 1 ? 0 : (int)cluster.block_rank();
+  unit::setup_common<1>(p);
+  setup_unit<1>(p, S, rank, 0);
+  if constexpr (C > 1) {
+    if (threadIdx.x < C)
+      SM::rowptr()[threadIdx.x] = cluster.map_shared_rank(SM::rows(0), (unsigned)threadIdx.x);
+    cluster_arrive();  // paired with the wait of the first stage 1
+  }
   __syncthreads();
 
   const int cid = blockIdx.x / C;
@@ -33,42 +36,59 @@ __global__ void __launch_bounds__(kT, kMinB) correlate_multi_kernel(PlanDev p, M
   float2* const scratch = a.scratch + (size_t)blockIdx.x * 32 * kT;
 
   for (int64_t k = a.k0 + cid; k < a.k1; k += ncl) {
-    // S2: forward passes 1-2 (pass 3 runs inside fused_mid for m = 0)
-    fwd_first_pass<kF, S, kNC, kT, true>(rank, a.bank + k * a.Lp, nz, 1);
-    stockham_pass<kF, kNC, kT, 16, 16, false>(SM::cols(), SM::tw2());
+    // S2: forward stages 1-2 (stage 3 runs inside the middle for m = 0)
+    stage1<1, true, (C > 1)>(0, S, rank, a.bank + k * a.Lp, nz, 1);
+    unit_sync<1>(0);
+    stage2<1>(0);
+    mid_enter<1>(0, rank);
     const int64_t krow = k - a.k0;
     for (int m = 0; m < a.M; ++m) {
-      // S3-S5 for segment m: product, sigma partial, inverse transform
-      fused_mid<S, kNC, kT, true>(rank, a.AB[m], SM::red(), S, a.M > 1 ? scratch : nullptr,
-                                  m > 0);
-      if (threadIdx.x == 0) {
-        float s = 0.f;
-        for (int w = 0; w < kT / 32; ++w) s += SM::red()[w];
-        store_sigma_partial<kF, S, kNC, true>(rank, s);
+      // S3-S5 for segment m: product, sigma share, inverse transform
+      if (m == 0) {
+        middle<1, 1, true, false>(0, rank, a.AB[0], a.M > 1 ? scratch : nullptr, false);
+      } else {
+        // the rows are rewritten: after the cluster's reads (S = 2: after
+        // every thread has read its own rows)
+        if constexpr (C == 1) __syncthreads();
+        middle<1, 1, true, (C > 1)>(0, rank, a.AB[m], scratch, true);
       }
-      __syncthreads();
-      // two rounds per pass over disjoint columns: the last inverse pass's
-      // round barriers order these stores; a cluster barrier follows it
-      stockham_pass<kF, kNC, kT, 16, 16, true, false>(SM::cols(), SM::tw2());
-      inv_last_pass<kF, S, kNC, kT, false>();
-      cluster.sync();  // every column and sigma partial of the cluster is ready
-      float tot = 0.f;  // Eq. PT over the cluster's partials, in rank order
-#pragma unroll
-      for (int q = 0; q < C; ++q) tot += SM::sigall()[q];
-      const float sigma = sqrtf(2.0f * tot) / (float)N;
-      if (rank == 0 && threadIdx.x == 0) a.sigma[m][krow] = sigma;
+      mid_leave<1>(0, rank);
+      stage2i<1>(0);
+      unit_sync<1>(0);
       const TailOut out{a.recs[m], a.cap[m], a.counter[m], nullptr};
-      combine_and_emit<kF, S, kNC, kT>(SM::colptr(), H, rank, a.kappa * sigma, (uint32_t)k, krow,
-                                       out, sigma);
-      cluster_sync_after_reads();  // remote reads done before the columns are overwritten
+      if constexpr (S == 2) {
+        const float share = unit_power<1>(0);
+        const float sigma = sigma_of(&share, 1, S * 2 * kF);
+        if (threadIdx.x == 0) a.sigma[m][krow] = sigma;
+        finish_s2<false>(p.uc, a.kappa * sigma, (uint32_t)k, krow, out, sigma);
+      } else {
+        stage1i<1>(0);
+        if (threadIdx.x == 0) {
+          const float share = unit_power<1>(0);
+#pragma unroll
+          for (int q = 0; q < C; ++q)
+            *cluster.map_shared_rank(SM::sigall() + rank, (unsigned)q) = share;
+        }
+        cluster_arrive();
+        Combine<S, 1> cb;
+        cb.twiddles(p.uc, rank);
+        cluster_wait();  // every row and share of the cluster is ready
+        const float sigma = sigma_of(SM::sigall(), S / 2, S * 2 * kF);
+        if (rank == 0 && threadIdx.x == 0) a.sigma[m][krow] = sigma;
+        cb.template emit<false>(SM::rowptr(), p.uc, rank, a.kappa * sigma, (uint32_t)k, krow, out,
+                                sigma);
+        __syncwarp();
+        cluster_arrive_relaxed();  // every remote value has fed a vote: the reads are done
+      }
     }
   }
+  if constexpr (C > 1) cluster_wait();  // the cluster's last reads of this CTA's rows
 }
 
 template <int S>
 cudaError_t launch_multi_t(const PlanDev& p, const MultiArgs& a, cudaStream_t s) {
-  constexpr int C = ColMap<S, kNC>::C;
-  constexpr size_t smem = Lay<kF, kNC>::total;
+  constexpr int C = S / 2;
+  constexpr size_t smem = unit::Lay<1>::total;
   auto kern = correlate_multi_kernel<S>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -106,7 +126,7 @@ size_t multi_scratch_bytes(int sms) { return (size_t)sms * kMinB * kT * 32 * siz
 
 cudaError_t launch_correlate_multi(const PlanDev& p, const MultiArgs& a, cudaStream_t s) {
   if (a.k1 <= a.k0 || a.M < 1) return cudaSuccess;
-  if (p.g.F != kF || a.Lp > kF || a.M > kMaxMulti) return cudaErrorInvalidValue;
+  if (p.g.F != kF || p.g.S < 2 || a.Lp > kF || a.M > kMaxMulti) return cudaErrorInvalidValue;
   switch (p.g.S) {
     case 2: return launch_multi_t<2>(p, a, s);
     case 4: return launch_multi_t<4>(p, a, s);

@@ -1,16 +1,12 @@
 // Correlate kernels for S = 8 columns (N = 2^16).
-#include "bege_corr.cuh"
+#include "bege_unit.cuh"
 
 namespace bege {
 
 cudaError_t launch_correlate_s8(const PlanDev& p, const CorrelateArgs& a, CorrConfig c,
                                  bool halfz, cudaStream_t s) {
-  if (c.nc == 2 && c.threads == 256)
-    return halfz ? launch_corr_t<4096, 8, 2, 256, 2, true>(p, a, s)
-                 : launch_corr_t<4096, 8, 2, 256, 2, false>(p, a, s);
-  if (c.nc == 4 && c.threads == 512)
-    return halfz ? launch_corr_t<4096, 8, 4, 512, 1, true>(p, a, s)
-                 : launch_corr_t<4096, 8, 4, 512, 1, false>(p, a, s);
+  if (c.nc == 2 && c.threads == 256) return unit::launch_unit<8, 1>(p, a, halfz, s);
+  if (c.nc == 4 && c.threads == 512) return unit::launch_unit<8, 2>(p, a, halfz, s);
   return cudaErrorInvalidValue;
 }
 

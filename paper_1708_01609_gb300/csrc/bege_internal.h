@@ -46,10 +46,94 @@ struct PlanDev {
   const float2* tw3;   // [F]      Stockham pass 3: [r*(F/16) + k] = wF^(k r)
   const float2* wH;    // [256*S]  wH^k
   const float2* wR0S;  // [R0*S]   w(R0 S)^q
-  const float2* w16S;  // [16*S]   w(16 S)^q
   const float2* wS;    // [S]      wS^q
   const float2* wN;    // [H]      wN^j
+  // S >= 2, {cos, tan} sets of bege_unit.cuh (rot_entry, set_turns):
+  const float2* t1;    // [S][8]         stage 1: column b
+  const float2* t2;    // [S][8][16]     stage 2: column b, k0
+  const float2* t3;    // [S/2][8][256]  stage 3: unit, thread
+  const float2* u2;    // [8][16]        stage 2': n0
+  const float2* u1;    // [8][256]       stage 1': n0 + 16 n1
+  const float2* uc;    // [S/2][4096]    stage c: n
 };
+
+// Sizes (in float2) of the sets of an S-column plan, in the order t1, t2, t3,
+// u2, u1, uc; all 0 for S = 1.
+constexpr int kUnitTables = 6;
+constexpr __host__ __device__ int unit_table_size(int S, int table) {
+  if (S < 2) return 0;
+  switch (table) {
+    case 0: return 8 * S;
+    case 1: return 128 * S;
+    case 2: return 1024 * S;
+    case 3: return 128;
+    case 4: return 2048;
+    default: return 2048 * S;
+  }
+}
+
+// Entry i of a table: the angle it holds, num / den of a turn.
+struct Turn {
+  int64_t num, den;
+};
+inline __host__ __device__ Turn unit_table_turn(int S, int table, int i) {
+  int64_t x = 0, M = 1;  // base x / M turns
+  int q = 0;             // place in the 16-point set
+  switch (table) {
+    case 0: q = i & 7; x = i >> 3; M = 16 * S; break;
+    case 1: {
+      const int b = i >> 7, k0 = i & 15;
+      q = (i >> 4) & 7; x = S * k0 + b; M = 256 * S;
+      break;
+    }
+    case 2: {
+      // thread t of the middle of unit u holds butterfly (k0, k1) of column b
+      const int u = i >> 11, t = i & 255, l = t & 15;
+      int b = u, k0, k1 = l;
+      if (u > 0) {
+        k0 = (t & 16) ? 15 - (t >> 5) : t >> 5;
+      } else if (t & 16) {
+        b = S / 2; k0 = t >> 5;
+      } else if (t >= 32) {
+        k0 = t >> 5;
+      } else {
+        k0 = l < 8 ? 0 : 8; k1 = l & 7;
+      }
+      q = (i >> 8) & 7; x = (int64_t)S * (k0 + 16 * k1) + b; M = 4096 * (int64_t)S;
+      break;
+    }
+    case 3: q = i >> 4; x = i & 15; M = 256; break;
+    case 4: q = i >> 8; x = i & 255; M = 4096; break;
+    default: {
+      // the S-point DFT uses the end of the set: S = 2 {base}, 4 {2 x base,
+      // base}, 8 {4 x, 2 x, base, base + 1/8}, 16 the whole set
+      const int e = i >> 12;
+      x = i & 4095; M = 4096 * (int64_t)S;
+      const int64_t den = 16 * M;
+      if (S == 16) { q = e; break; }
+      if (S == 8 && e == 3) return {(16 * x + 2 * M) % den, den};
+      const int levels = S == 8 ? 2 : S == 4 ? 1 : 0;
+      return {(16 * x << (levels - e)) % den, den};
+    }
+  }
+  const int64_t den = 16 * M;
+  switch (q) {
+    case 0: return {128 * x % den, den};
+    case 1: return {64 * x % den, den};
+    case 2: return {32 * x % den, den};
+    case 3: return {(32 * x + 2 * M) % den, den};
+    default: return {(16 * x + (q - 4) * M) % den, den};
+  }
+}
+
+// {cos, tan} of an angle with FP64 cosine c and sine s, rounded so that
+// cos * tan is the sine to FP32 also where the cosine is (nearly) zero.
+inline __host__ __device__ float2 rot_entry(double c, double s) {
+  float cf = (float)c;
+  const float least = 9.31322574615478515625e-10f;  // 2^-30
+  if (cf < least && cf > -least) cf = cf < 0.f ? -least : least;
+  return make_float2(cf, (float)(s / (double)cf));
+}
 
 Geometry make_geometry(int64_t n);
 
@@ -71,8 +155,9 @@ CorrConfig default_config(const Geometry& g);
 bool config_valid(const Geometry& g, CorrConfig c);
 
 // S1: segment spectrum.  y: N floats (device).  D: H+1 complex (natural
-// order).  AB: S*F float4 {A_j, B_j} in residue-major order [b*F + a].
-cudaError_t launch_segment(const PlanDev& p, const float* y, float2* D, float4* AB,
+// order).  AB: H float4 {A_j, B_j}, in residue-major order [b*F + a] (natural:
+// the tensor-core kernel) or in the order the FP32 kernels read them.
+cudaError_t launch_segment(const PlanDev& p, const float* y, float2* D, float4* AB, bool natural,
                            cudaStream_t s);
 
 // S2..S6 over bank rows [k0, k1).  bank: rows of Lp floats (zero-padded

@@ -14,7 +14,7 @@
 //     by every call, ahead of the call's own kernels on its stream, so no
 //     call depends on what an earlier call left in the array).
 // The array lives on every GPU that loads the library until the process
-// exits (about 1.05 MiB).  All calls on a device share it and it keeps the
+// exits (about 1.2 MiB).  All calls on a device share it and it keeps the
 // contents of the last call, so two calls whose work overlaps on the GPU
 // (for example on two streams) corrupt each other; callers serialise them.
 #include <mutex>
@@ -39,10 +39,15 @@ constexpr size_t kOffTw2 = kOffD + al256((kMaxH + 1) * sizeof(float2));
 constexpr size_t kOffTw3 = kOffTw2 + al256(256 * sizeof(float2));
 constexpr size_t kOffWH = kOffTw3 + al256(4096 * sizeof(float2));
 constexpr size_t kOffWR0S = kOffWH + al256(256 * 8 * sizeof(float2));
-constexpr size_t kOffW16S = kOffWR0S + al256(16 * 8 * sizeof(float2));
-constexpr size_t kOffWS = kOffW16S + al256(16 * 8 * sizeof(float2));
+constexpr size_t kOffWS = kOffWR0S + al256(256 * 8 * sizeof(float2));
 constexpr size_t kOffWN = kOffWS + al256(8 * sizeof(float2));
-constexpr size_t kScratchBytes = kOffWN + al256(kMaxH * sizeof(float2));
+constexpr size_t kOffUnit = kOffWN + al256(kMaxH * sizeof(float2));
+constexpr size_t unit_tables(int S, int upto) {
+  size_t n = 0;
+  for (int t = 0; t < upto; ++t) n += unit_table_size(S, t);
+  return n;
+}
+constexpr size_t kScratchBytes = kOffUnit + al256(unit_tables(8, kUnitTables) * sizeof(float2));
 
 static __device__ __align__(256) unsigned char g_search_scratch[kScratchBytes];
 
@@ -56,11 +61,11 @@ __device__ __forceinline__ float2 unit_root(int64_t k, int64_t M) {
 // The twiddle tables of PlanDev for geometry g, written into the scratch
 // regions (same definitions as the tables the context uploads).
 __global__ void search_tables_kernel(Geometry g, float2* tw2, float2* tw3, float2* wH,
-                                     float2* wR0S, float2* w16S, float2* wS, float2* wN) {
+                                     float2* wR0S, float2* wS, float2* wN, float2* unit) {
   const int64_t n_tw2 = 16 * g.R0, n_tw3 = g.F, n_wH = 256 * (int64_t)g.S,
-                n_wR0S = (int64_t)g.R0 * g.S, n_w16S = 16 * (int64_t)g.S, n_wS = g.S,
-                n_wN = g.H;
-  const int64_t total = n_tw2 + n_tw3 + n_wH + n_wR0S + n_w16S + n_wS + n_wN;
+                n_wR0S = (int64_t)g.R0 * g.S, n_wS = g.S, n_wN = g.H;
+  int64_t total = n_tw2 + n_tw3 + n_wH + n_wR0S + n_wS + n_wN;
+  for (int t = 0; t < kUnitTables; ++t) total += unit_table_size(g.S, t);
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total;
        i += (int64_t)gridDim.x * blockDim.x) {
     int64_t j = i;
@@ -85,17 +90,23 @@ __global__ void search_tables_kernel(Geometry g, float2* tw2, float2* tw3, float
       continue;
     }
     j -= n_wR0S;
-    if (j < n_w16S) {
-      w16S[j] = unit_root(j, 16 * (int64_t)g.S);
-      continue;
-    }
-    j -= n_w16S;
     if (j < n_wS) {
       wS[j] = unit_root(j, g.S);
       continue;
     }
     j -= n_wS;
-    wN[j] = unit_root(j, g.N);
+    if (j < n_wN) {
+      wN[j] = unit_root(j, g.N);
+      continue;
+    }
+    j -= n_wN;
+    const int64_t at = j;
+    int t = 0;
+    while (j >= unit_table_size(g.S, t)) j -= unit_table_size(g.S, t++);
+    const Turn a = unit_table_turn(g.S, t, (int)j);
+    double s, c;
+    sincospi(2.0 * (double)a.num / (double)a.den, &s, &c);
+    unit[at] = rot_entry(c, s);
   }
 }
 
@@ -158,21 +169,22 @@ extern "C" int bege_search_noalloc(const float* strain_dev, int64_t n, const flo
     p.tw3 = reinterpret_cast<const float2*>(base + kOffTw3);
     p.wH = reinterpret_cast<const float2*>(base + kOffWH);
     p.wR0S = reinterpret_cast<const float2*>(base + kOffWR0S);
-    p.w16S = reinterpret_cast<const float2*>(base + kOffW16S);
     p.wS = reinterpret_cast<const float2*>(base + kOffWS);
     p.wN = reinterpret_cast<const float2*>(base + kOffWN);
+    float2* const unit = reinterpret_cast<float2*>(base + kOffUnit);
+    const float2** const tables[kUnitTables] = {&p.t1, &p.t2, &p.t3, &p.u2, &p.u1, &p.uc};
+    for (int t = 0; t < kUnitTables; ++t) *tables[t] = unit + unit_tables(g.S, t);
     // The tables are rebuilt on every call, in stream order before this
     // call's kernels: the host keeps no record of which n the array holds,
     // which could disagree with the device's order of work.
     search_tables_kernel<<<64, 256, 0, s>>>(
         g, const_cast<float2*>(p.tw2), const_cast<float2*>(p.tw3), const_cast<float2*>(p.wH),
-        const_cast<float2*>(p.wR0S), const_cast<float2*>(p.w16S), const_cast<float2*>(p.wS),
-        const_cast<float2*>(p.wN));
+        const_cast<float2*>(p.wR0S), const_cast<float2*>(p.wS), const_cast<float2*>(p.wN), unit);
     e = cudaGetLastError();
     if (e != cudaSuccess) return set_last_error(BEGE_ECUDA, cudaGetErrorString(e));
     float4* AB = reinterpret_cast<float4*>(base + kOffAB);
     float2* D = reinterpret_cast<float2*>(base + kOffD);
-    e = launch_segment(p, strain_dev, D, AB, s);
+    e = launch_segment(p, strain_dev, D, AB, false, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(tail_count_dev, 0, sizeof(unsigned long long), s);
     if (e == cudaSuccess) {
       CorrelateArgs a{};

@@ -37,29 +37,33 @@ bool config_valid(const Geometry& g, CorrConfig c) {
   return false;
 }
 
-// Default launch shape: two columns and 256 threads per CTA (two CTAs per
-// SM) was the fastest for every N >= 2^14 on GB300.
+// Default launch shape.  S >= 4: two units (512 threads) a CTA, one CTA per
+// SM, so half as many CTAs meet in a cluster and a unit's neighbour in the
+// CTA needs no distributed shared memory; S = 2 has one unit a template and
+// two CTAs per SM.  Per template (65536 chirps, GB300), 4 x 512 against 2 x
+// 256: N = 2^15 75.7 / 81.9 ns, 2^16 170.7 / 188.8, 2^17 405 / 411.
 CorrConfig default_config(const Geometry& g) {
   if (g.S == 1) return {1, 256};
-  return {2, 256};
+  if (g.S == 2) return {2, 256};
+  return {4, 512};
 }
 
-cudaError_t launch_segment(const PlanDev& p, const float* y, float2* D, float4* AB,
+cudaError_t launch_segment(const PlanDev& p, const float* y, float2* D, float4* AB, bool natural,
                            cudaStream_t s) {
   const Geometry& g = p.g;
   switch (g.S) {
     case 1:
       switch (g.F) {
-        case 512: return launch_segment_t<512, 1, 1, 256>(p, y, D, AB, s);
-        case 1024: return launch_segment_t<1024, 1, 1, 256>(p, y, D, AB, s);
-        case 2048: return launch_segment_t<2048, 1, 1, 256>(p, y, D, AB, s);
-        case 4096: return launch_segment_t<4096, 1, 1, 256>(p, y, D, AB, s);
+        case 512: return launch_segment_t<512, 1, 1, 256>(p, y, D, AB, natural, s);
+        case 1024: return launch_segment_t<1024, 1, 1, 256>(p, y, D, AB, natural, s);
+        case 2048: return launch_segment_t<2048, 1, 1, 256>(p, y, D, AB, natural, s);
+        case 4096: return launch_segment_t<4096, 1, 1, 256>(p, y, D, AB, natural, s);
         default: return cudaErrorInvalidValue;
       }
-    case 2: return launch_segment_t<4096, 2, 2, 256>(p, y, D, AB, s);
-    case 4: return launch_segment_t<4096, 4, 4, 512>(p, y, D, AB, s);
-    case 8: return launch_segment_t<4096, 8, 4, 512>(p, y, D, AB, s);
-    case 16: return launch_segment_t<4096, 16, 4, 512>(p, y, D, AB, s);
+    case 2: return launch_segment_t<4096, 2, 2, 256>(p, y, D, AB, natural, s);
+    case 4: return launch_segment_t<4096, 4, 4, 512>(p, y, D, AB, natural, s);
+    case 8: return launch_segment_t<4096, 8, 4, 512>(p, y, D, AB, natural, s);
+    case 16: return launch_segment_t<4096, 16, 4, 512>(p, y, D, AB, natural, s);
     default: return cudaErrorInvalidValue;
   }
 }

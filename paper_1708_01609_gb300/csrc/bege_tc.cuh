@@ -42,6 +42,17 @@
 namespace bege {
 namespace tc {
 
+// A cluster barrier that orders only earlier reads of distributed shared
+// memory before later writes (the combine's remote reads before the next
+// template overwrites the columns): every remote value has fed a warp vote
+// or the threshold before its thread arrives, so the reads have completed
+// and the arrive needs no release fence.  Data that other CTAs read later
+// is published by the full (release / acquire) barrier before the combine.
+__device__ __forceinline__ void cluster_sync_after_reads() {
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;\n\tbarrier.cluster.wait.aligned;" :::
+               "memory");
+}
+
 constexpr int kF = 4096;
 constexpr int kGT = 256;  // threads of a group: 8 warps, two per TMEM lane quarter
 

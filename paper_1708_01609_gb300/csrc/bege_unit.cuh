@@ -1,0 +1,816 @@
+// The correlation for N >= 2^14 (S >= 2 columns of F = 4096 points): per-stage
+// functions of one unit (two columns, 256 threads) shared by the single,
+// block and batch kernels, and the single-segment kernel itself.
+//
+// Stages.  With the column split of bege_corr.cuh, j = S a + b, write
+// a = k0 + 16 k1 + 256 k2 and m = n0 + 16 n1 + 256 n2.  Forward (z -> Z):
+//   1  over n2 -> k0   twiddle base (S k0' + b) 256 / H with k0' = 0: b / (16 S)
+//   2  over n1 -> k1   base (S k0 + b) / (256 S)
+//   3  over n0 -> k2   base (S (k0 + 16 k1) + b) / H
+// inverse (Y -> rho), n = n0 + 16 n1 + 256 n2 + 4096 n3:
+//   3' over k2 -> n0   no twiddle
+//   2' over k1 -> n1   base n0 / 256
+//   1' over k0 -> n2   base (n0 + 16 n1) / 4096
+//   c  over b  -> n3   base (n0 + 16 n1 + 256 n2) / H
+// (bases in turns; input r of a stage is turned by r times its base).  Each
+// stage is a decimation-in-time DFT whose input twiddles are w^r for one base
+// w, so every twiddle, the column's own w_H^(b m) and w_H^(-b n) included,
+// enters a radix-2 butterfly a +/- w b as two fused multiply-adds: w b =
+// cos (1 -/+ i tan) b, u = (1 -/+ i tan) b and a +/- cos u, six operations
+// for a butterfly at any angle, and a 16-point stage needs 8 (cos, tan)
+// pairs in place of 15 factors.  The table keeps |cos| >= 2^-30 with tan =
+// sin / cos, so cos * tan rounds sin also where the cosine vanishes (the
+// leftover 2^-30 is far below an FP32 rounding); each u is rounded once and
+// scaled by cos, which costs no more than the rounding of a plain product.
+//
+// Every stage works in place: a butterfly writes the 16 rows it read, so the
+// spectrum sits digit-reversed in shared memory, the product reads its
+// coefficients in the same order (coef_pos), and one ordering point between
+// stages is enough.  Stages 2, 3, 3', 2' exchange values only between
+// threads of the same k0; warp w of a unit holds k0 = w and 15 - w (a column
+// bin's mirror has every digit complemented), so between them a warp waits
+// for itself only and the warps drift: the loads of one overlap the
+// arithmetic of another.  Unit 0 (columns 0 and S/2, each its own mirror)
+// pairs k0 with 16 - k0 in column 0 and takes a barrier there.
+//
+// Rows.  Block k0 (256 rows, 288 16-byte slots) of a unit holds its two
+// columns interleaved (float4 {slot 0, slot 1}, row i at slot i) between
+// stages 1-2 and from 2' on, and as two arrays of 16 x 18 float2 (column c,
+// row n0 + 16 k1 at 288 c + n0 + 18 k1) from 2 to 2': the middle reads and
+// writes 16 consecutive values of one column as 8 16-byte accesses, free of
+// bank conflicts, and its mirror butterfly in the other column likewise.
+//
+// Bound: FP32 issue and shared-memory bandwidth (FFT butterflies), not HBM:
+// at N = 2^16 a correlation issues 110e3 warp instructions (91e3 of them on
+// the FMA pipe) and moves 23.5e3 shared-memory wavefronts, 50% and 39% of
+// what its time allows; what is left is latency (L2 coefficients, the
+// cluster's barrier) with 16 warps per SM, all that 128 registers a thread
+// allow.  Per template of 1 s, against Stockham passes with plain twiddle
+// products and ten CTA barriers a template (65536 chirps, GB300): N = 2^14
+// 49.6 -> 35.2 ns, 2^15 102 -> 75.7, 2^16 216 -> 171, 2^17 473 -> 405.
+// Measured beside it and not kept: packed FP32 pairs (an FFMA2 takes the FMA
+// pipe 2.2 to 2.5 cycles, no less than two FFMAs); columns of 2048 points with
+// 128-thread units (183 ns at 2^16, 41 at 2^14); stage 1' storing straight
+// into the CTA that combines (209 ns against 191 for reading there, with
+// clusters of four).
+#pragma once
+
+#include "bege_corr.cuh"
+
+namespace bege {
+namespace unit {
+
+constexpr int kF = 4096;
+constexpr int kT = 256;         // threads of a unit
+constexpr int kBlk = 288;       // 16-byte slots of a block of 256 rows
+
+// Shared memory of a CTA with U units (bytes).
+template <int U>
+struct Lay {
+  static constexpr size_t u1 = 0;                        // [8][256] float2: stage 1'
+  static constexpr size_t u2 = u1 + 8 * 256 * 8;         // [8][16] float2: stage 2'
+  static constexpr size_t ws = u2 + 8 * 16 * 8;          // [16] float2: w_S^q (folded templates)
+  static constexpr size_t rowptr = ws + 16 * 8;          // [8] the units' rows in the cluster
+  static constexpr size_t sigall = rowptr + 8 * 8;       // [8] units' shares of sum |Y|^2
+  static constexpr size_t units = sigall + 8 * 4;
+  // within a unit
+  static constexpr size_t rows = 0;                      // 16 blocks
+  static constexpr size_t t3 = rows + 16 * kBlk * 16;    // [8][256] float2: stage 3
+  static constexpr size_t t2 = t3 + 8 * 256 * 8;         // [8][16] float4: stage 2, both columns
+  static constexpr size_t t1 = t2 + 8 * 16 * 16;         // [8] float4: stage 1, both columns
+  static constexpr size_t red = t1 + 8 * 16;             // [8] warp sums
+  static constexpr size_t unit_bytes = red + 8 * 4;
+  static constexpr size_t total = units + U * unit_bytes;
+  static_assert(units % 16 == 0 && unit_bytes % 16 == 0, "16-byte rows");
+};
+
+template <int U>
+struct Sm {
+  using L = Lay<U>;
+  static __device__ __forceinline__ unsigned char* unit(int ui) {
+    return smem_raw + L::units + (U == 1 ? 0 : ui * L::unit_bytes);
+  }
+  static __device__ __forceinline__ float4* rows(int ui) { return reinterpret_cast<float4*>(unit(ui) + L::rows); }
+  static __device__ __forceinline__ float2* t3(int ui) { return reinterpret_cast<float2*>(unit(ui) + L::t3); }
+  static __device__ __forceinline__ float4* t2(int ui) { return reinterpret_cast<float4*>(unit(ui) + L::t2); }
+  static __device__ __forceinline__ float4* t1(int ui) { return reinterpret_cast<float4*>(unit(ui) + L::t1); }
+  static __device__ __forceinline__ float* red(int ui) { return reinterpret_cast<float*>(unit(ui) + L::red); }
+  static __device__ __forceinline__ float2* u1() { return reinterpret_cast<float2*>(smem_raw + L::u1); }
+  static __device__ __forceinline__ float2* u2() { return reinterpret_cast<float2*>(smem_raw + L::u2); }
+  static __device__ __forceinline__ float2* ws() { return reinterpret_cast<float2*>(smem_raw + L::ws); }
+  static __device__ __forceinline__ float4** rowptr() { return reinterpret_cast<float4**>(smem_raw + L::rowptr); }
+  static __device__ __forceinline__ float* sigall() { return reinterpret_cast<float*>(smem_raw + L::sigall); }
+};
+
+__device__ __forceinline__ int unit_tid() { return threadIdx.x & (kT - 1); }
+
+// All threads of the unit (barrier 0 where the CTA is one unit).
+template <int U>
+__device__ __forceinline__ void unit_sync(int ui) {
+  if constexpr (U == 1)
+    __syncthreads();
+  else
+    asm volatile("bar.sync %0, %1;" ::"r"(ui + 1), "n"(kT) : "memory");
+}
+
+__device__ __forceinline__ void cluster_arrive_relaxed() {
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_arrive() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// ---------------------------------------------------------------------------
+// DFTs with merged twiddles
+// ---------------------------------------------------------------------------
+// (a, b) -> (a + w b, a - w b), w = e^(-/+ i angle) (-/+ i)^K, {c, t} = (cos, tan) of the angle.
+template <bool INV, int K>
+__device__ __forceinline__ void bfly(float2& a, float2& b, float c, float t) {
+  float2 u = rot_a<INV>(b, t);
+  if constexpr (K == 1) u = mul_mi<INV>(u);
+  b = cfma(a, -c, u);
+  a = cfma(a, c, u);
+}
+
+// The index that holds output k of an R-point DFT below (bit-reversed).
+template <int R>
+__host__ __device__ constexpr int rev(int k) {
+  int r = 0;
+  for (int b = 1; b < R; b <<= 1) r = 2 * r + ((k & b) ? 1 : 0);
+  return r;
+}
+
+// 16-point DFTs of two columns, twiddle pairs w(q) = {c_a, t_a, c_b, t_b}:
+// q = 0: 8 x base, 1: 4 x, 2: 2 x, 3: 2 x + 1/8, 4 + i: base + i/16 (turns).
+// HALFZ: inputs 8..15 are zero (and not read).
+template <bool INV, bool HALFZ, class W>
+__device__ __forceinline__ void dft16x2(float2 (&a)[16], float2 (&b)[16], W w) {
+  if constexpr (!HALFZ) {
+    const float4 s = w(0);
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      bfly<INV, 0>(a[r], a[r + 8], s.x, s.y);
+      bfly<INV, 0>(b[r], b[r + 8], s.z, s.w);
+    }
+  }
+  {
+    const float4 s = w(1);
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      if constexpr (HALFZ) {
+        a[8 + r] = a[r]; a[12 + r] = a[4 + r];
+        b[8 + r] = b[r]; b[12 + r] = b[4 + r];
+      }
+      bfly<INV, 0>(a[r], a[r + 4], s.x, s.y);
+      bfly<INV, 1>(a[8 + r], a[12 + r], s.x, s.y);
+      bfly<INV, 0>(b[r], b[r + 4], s.z, s.w);
+      bfly<INV, 1>(b[8 + r], b[12 + r], s.z, s.w);
+    }
+  }
+#pragma unroll
+  for (int p = 0; p < 2; ++p) {
+    const float4 s = w(2 + p);
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      bfly<INV, 0>(a[8 * p + r], a[8 * p + r + 2], s.x, s.y);
+      bfly<INV, 1>(a[8 * p + 4 + r], a[8 * p + 4 + r + 2], s.x, s.y);
+      bfly<INV, 0>(b[8 * p + r], b[8 * p + r + 2], s.z, s.w);
+      bfly<INV, 1>(b[8 * p + 4 + r], b[8 * p + 4 + r + 2], s.z, s.w);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const float4 s = w(4 + i);
+    const int o = 8 * (i & 1) + 4 * (i >> 1);
+    bfly<INV, 0>(a[o], a[o + 1], s.x, s.y);
+    bfly<INV, 1>(a[o + 2], a[o + 3], s.x, s.y);
+    bfly<INV, 0>(b[o], b[o + 1], s.z, s.w);
+    bfly<INV, 1>(b[o + 2], b[o + 3], s.z, s.w);
+  }
+}
+
+// S-point DFT (S = 2 .. 16) of one row, pairs w(q): the last entries of the
+// 16-point set, i.e. S = 8: {4 x base, 2 x, base, base + 1/8}, S = 4: {2 x,
+// base}, S = 2: {base}.
+template <int S, bool INV, class W>
+__device__ __forceinline__ void dft_row(float2 (&x)[S], W w) {
+  int q = 0;
+  if constexpr (S == 16) {
+    const float2 s = w(0);
+#pragma unroll
+    for (int r = 0; r < 8; ++r) bfly<INV, 0>(x[r], x[r + 8], s.x, s.y);
+    q = 1;
+  }
+  if constexpr (S >= 8) {
+    const float2 s = w(q);
+#pragma unroll
+    for (int o = 0; o < S; o += 16)
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        bfly<INV, 0>(x[o + r], x[o + r + 4], s.x, s.y);
+        if constexpr (S == 16) bfly<INV, 1>(x[8 + r], x[12 + r], s.x, s.y);
+      }
+    ++q;
+  }
+  if constexpr (S >= 4) {
+    constexpr int P = S == 16 ? 2 : 1;  // distinct twiddles of this level
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+      const float2 s = w(q + p);
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        bfly<INV, 0>(x[8 * p + r], x[8 * p + r + 2], s.x, s.y);
+        if constexpr (S >= 8) bfly<INV, 1>(x[8 * p + 4 + r], x[8 * p + 4 + r + 2], s.x, s.y);
+      }
+    }
+    q += P;
+  }
+  constexpr int P = S >= 8 ? S / 4 : 1;
+#pragma unroll
+  for (int i = 0; i < P; ++i) {
+    const float2 s = w(q + i);
+    const int o = S == 16 ? 8 * (i & 1) + 4 * (i >> 1) : 4 * i;
+    bfly<INV, 0>(x[o], x[o + 1], s.x, s.y);
+    if constexpr (S >= 4) bfly<INV, 1>(x[o + 2], x[o + 3], s.x, s.y);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Set-up
+// ---------------------------------------------------------------------------
+template <int U>
+__device__ __forceinline__ void setup_common(const PlanDev& p) {
+  using SM = Sm<U>;
+  for (int i = threadIdx.x; i < 8 * 256; i += kT * U) SM::u1()[i] = p.u1[i];
+  for (int i = threadIdx.x; i < 8 * 16; i += kT * U) SM::u2()[i] = p.u2[i];
+}
+
+// Tables of unit ug (columns ug and S - ug; unit 0: 0 and S/2) in slot ui.
+template <int U>
+__device__ __forceinline__ void setup_unit(const PlanDev& p, int S, int ug, int ui) {
+  using SM = Sm<U>;
+  const int t = unit_tid();
+  const int ba = ug, bb = ug == 0 ? S / 2 : S - ug;
+  for (int i = t; i < 8 * 256; i += kT) SM::t3(ui)[i] = p.t3[ug * 2048 + i];
+  if (t < 128) {
+    const float2 a = p.t2[ba * 128 + t], b = p.t2[bb * 128 + t];
+    SM::t2(ui)[t] = make_float4(a.x, a.y, b.x, b.y);
+  }
+  if (t < 8) {
+    const float2 a = p.t1[ba * 8 + t], b = p.t1[bb * 8 + t];
+    SM::t1(ui)[t] = make_float4(a.x, a.y, b.x, b.y);
+  }
+  if (ui == 0 && t < 16) SM::ws()[t] = t < S ? p.wS[t] : make_float2(1.f, 0.f);
+}
+
+// ---------------------------------------------------------------------------
+// Stages
+// ---------------------------------------------------------------------------
+// Stage 1 from the template's nz complex samples z (upper half of the columns
+// zero with HALFZ; otherwise folded over nfold multiples of F).  WAIT: the
+// cluster's reads of the previous contents of the rows are awaited after the
+// loads and the arithmetic, before the stores.
+template <int U, bool HALFZ, bool WAIT>
+__device__ __forceinline__ void stage1(int ui, int S, int ug, const float* __restrict__ src,
+                                       int nz, int nfold) {
+  using SM = Sm<U>;
+  const float2* z = reinterpret_cast<const float2*>(src);
+  const int j = unit_tid();
+  float2 va[16], vb[16];
+  if constexpr (HALFZ) {
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      const int m = j + 256 * r;
+      va[r] = vb[r] = m < nz ? __ldg(z + m) : make_float2(0.f, 0.f);
+    }
+  } else {
+#pragma unroll
+    for (int r = 0; r < 16; ++r) {
+      const int m = j + 256 * r;
+      va[r] = vb[r] = m < nz ? __ldg(z + m) : make_float2(0.f, 0.f);
+    }
+    const int bb = ug == 0 ? S / 2 : S - ug;
+#pragma unroll 1
+    for (int f = 1; f < nfold; ++f) {
+      const float2 wa = SM::ws()[(ug * f) & (S - 1)], wb = SM::ws()[(bb * f) & (S - 1)];
+#pragma unroll
+      for (int r = 0; r < 16; ++r) {
+        const int m = j + 256 * r + kF * f;
+        const float2 x = m < nz ? __ldg(z + m) : make_float2(0.f, 0.f);
+        va[r] = cadd(va[r], cmul(x, wa));
+        vb[r] = cadd(vb[r], cmul(x, wb));
+      }
+    }
+  }
+  const float4* w = SM::t1(ui);
+  dft16x2<false, HALFZ>(va, vb, [&](int q) { return w[q]; });
+  if constexpr (WAIT) cluster_wait();
+  float4* row = SM::rows(ui) + j;
+#pragma unroll
+  for (int k = 0; k < 16; ++k) row[k * kBlk] = make_float4(va[rev<16>(k)].x, va[rev<16>(k)].y,
+                                                          vb[rev<16>(k)].x, vb[rev<16>(k)].y);
+}
+
+// Stage 2: rows n0 + 16 n1 of block k0, interleaved in, separate out.
+template <int U>
+__device__ __forceinline__ void stage2(int ui) {
+  using SM = Sm<U>;
+  const int lane = threadIdx.x & 31, w8 = unit_tid() >> 5;
+  const int k0 = lane < 16 ? w8 : 15 - w8, n0 = lane & 15;
+  float4* blk = SM::rows(ui) + k0 * kBlk;
+  float2 va[16], vb[16];
+#pragma unroll
+  for (int r = 0; r < 16; ++r) {
+    const float4 v = blk[n0 + 16 * r];
+    va[r] = make_float2(v.x, v.y);
+    vb[r] = make_float2(v.z, v.w);
+  }
+  const float4* w = SM::t2(ui) + k0;
+  dft16x2<false, false>(va, vb, [&](int q) { return w[16 * q]; });
+  __syncwarp();
+  float2* c = reinterpret_cast<float2*>(blk) + n0;
+#pragma unroll
+  for (int k = 0; k < 16; ++k) c[18 * k] = va[rev<16>(k)];
+#pragma unroll
+  for (int k = 0; k < 16; ++k) c[288 + 18 * k] = vb[rev<16>(k)];
+}
+
+// The butterflies of thread t in the middle: (k0, k1) of column slot sa and
+// the mirror (k0b, k1b) of slot sb.  self: thread 0 of unit 0, which holds
+// butterflies (0, 0) and (0, 8) of column 0, each its own mirror.
+struct MidItem {
+  int sa, sb, k0, k1, k0b, k1b;
+};
+__device__ __forceinline__ MidItem mid_item(bool unit0, int t) {
+  MidItem m;
+  const int l = t & 15, w8 = t >> 5;
+  if (!unit0) {
+    m.sa = 0; m.sb = 1;
+    m.k0 = (t & 16) ? 15 - w8 : w8; m.k1 = l;
+    m.k0b = 15 - m.k0; m.k1b = 15 - l;
+  } else if (t & 16) {
+    m.sa = m.sb = 1;
+    m.k0 = w8; m.k1 = l;
+    m.k0b = 15 - w8; m.k1b = 15 - l;
+  } else {
+    m.sa = m.sb = 0;
+    if (w8 > 0) {
+      m.k0 = w8; m.k1 = l;
+      m.k0b = 16 - w8; m.k1b = 15 - l;
+    } else if (l < 8) {
+      m.k0 = m.k0b = 0;
+      m.k1 = l; m.k1b = l == 0 ? 8 : 16 - l;
+    } else {
+      m.k0 = m.k0b = 8;
+      m.k1 = l - 8; m.k1b = 15 - m.k1;
+    }
+  }
+  return m;
+}
+
+// A coefficient load that stays where it is written.
+__device__ __forceinline__ float4 ld_coef(const float4* p) {
+  float4 v;
+  asm volatile("ld.global.cg.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "l"(p));
+  return v;
+}
+
+// Stage 3, the product with sum |Y|^2, stage 3' of thread t's two
+// butterflies, in place.  zb holds the mirror's outputs conjugated and
+// reversed, g[r] = conj Z[mirror row 15 - r], which are the outputs of the
+// same twiddled DFT on the conjugated inputs (so both butterflies use one
+// set of twiddles).  MULTI: the spectrum is kept in `scratch` (32 values a
+// thread, stride kT) for the block's other segments, or with `reload` read
+// from there.  AHEAD: pairs of rows whose coefficients are loaded ahead.
+template <int U, int AHEAD, bool MULTI = false, bool WAIT = false>
+__device__ __forceinline__ void middle(int ui, int ug, const float4* __restrict__ coef,
+                                       float2* __restrict__ scratch = nullptr,
+                                       bool reload = false) {
+  using SM = Sm<U>;
+  const int t = unit_tid();
+  const bool unit0 = ug == 0, self = unit0 && t == 0;
+  const MidItem m = mid_item(unit0, t);
+  float4* pa = SM::rows(ui) + m.k0 * kBlk + (m.sa * 144 + m.k1 * 9);
+  float4* pb = SM::rows(ui) + m.k0b * kBlk + (m.sb * 144 + m.k1b * 9);
+  const float4* ab = coef + (size_t)ug * (24 * kT) + t;
+  float2 za[16], zb[16];
+  // the coefficients of the first AHEAD pairs of rows are under way during
+  // stage 3, the others AHEAD pairs ahead of their use
+  float4 c0[AHEAD], c1[AHEAD], c2[AHEAD];
+#pragma unroll
+  for (int i = 0; i < AHEAD; ++i) {
+    c0[i] = ld_coef(ab + 3 * i * kT);
+    c1[i] = ld_coef(ab + (3 * i + 1) * kT);
+    c2[i] = ld_coef(ab + (3 * i + 2) * kT);
+  }
+  if (MULTI && reload) {
+#pragma unroll
+    for (int r = 0; r < 16; ++r) {
+      za[r] = __ldcg(scratch + r * kT + t);
+      zb[r] = __ldcg(scratch + (16 + r) * kT + t);
+    }
+  } else {
+    {
+      float2 xa[16], xb[16];
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        const float4 v = pa[r], u = pb[r];
+        xa[2 * r] = make_float2(v.x, v.y);
+        xa[2 * r + 1] = make_float2(v.z, v.w);
+        xb[2 * r] = make_float2(u.x, -u.y);
+        xb[2 * r + 1] = make_float2(u.z, -u.w);
+      }
+      if (self) {  // butterfly (0, 8) has its own base, 1/32 turn, and no mirror
+        constexpr float c[16] = {1.f, 0.98078528040323044913f, 0.92387953251128675613f,
+                                 0.83146961230254523708f, 0.70710678118654752440f,
+                                 0.55557023301960222474f, 0.38268343236508977173f,
+                                 0.19509032201612826785f, 0.f, -0.19509032201612826785f,
+                                 -0.38268343236508977173f, -0.55557023301960222474f,
+                                 -0.70710678118654752440f, -0.83146961230254523708f,
+                                 -0.92387953251128675613f, -0.98078528040323044913f};
+#pragma unroll
+        for (int r = 1; r < 16; ++r) {
+          const float s = r < 8 ? c[8 - r] : c[r - 8];  // sin(2 pi r / 32)
+          xb[r] = cmul(cconj(xb[r]), make_float2(c[r], -s));
+        }
+        xb[0] = cconj(xb[0]);
+      }
+      const float2* w = SM::t3(ui) + t;
+      dft16x2<false, false>(xa, xb, [&](int q) {
+        const float2 s = w[256 * q];
+        return make_float4(s.x, s.y, s.x, s.y);
+      });
+#pragma unroll
+      for (int r = 0; r < 16; ++r) {
+        za[r] = xa[rev<16>(r)];
+        zb[r] = xb[rev<16>(r)];
+      }
+    }
+    if (MULTI && scratch) {
+#pragma unroll
+      for (int r = 0; r < 16; ++r) {
+        __stcg(scratch + r * kT + t, za[r]);
+        __stcg(scratch + (16 + r) * kT + t, zb[r]);
+      }
+    }
+  }
+  float acc = 0.f;
+  float2 yb[16];  // the mirror butterfly's Y by its own k2
+  if (!self) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const float4 a0 = c0[i % AHEAD], a1 = c1[i % AHEAD], b = c2[i % AHEAD];
+      if (i + AHEAD < 8) {
+        c0[i % AHEAD] = ld_coef(ab + 3 * (i + AHEAD) * kT);
+        c1[i % AHEAD] = ld_coef(ab + (3 * (i + AHEAD) + 1) * kT);
+        c2[i % AHEAD] = ld_coef(ab + (3 * (i + AHEAD) + 2) * kT);
+      }
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const int r = 2 * i + e;
+        const float4 A = e ? a1 : a0;
+        const float2 B = e ? make_float2(b.z, b.w) : make_float2(b.x, b.y);
+        const float2 x = za[r], g = zb[r];
+        za[r] = packed_product(x, cconj(g), make_float2(A.x, A.y), B);
+        yb[15 - r] = packed_product(cconj(g), x, make_float2(A.z, A.w), cconj(B));
+        acc = fmaf(za[r].x, za[r].x, fmaf(za[r].y, za[r].y, acc));
+        acc = fmaf(yb[15 - r].x, yb[15 - r].x, fmaf(yb[15 - r].y, yb[15 - r].y, acc));
+      }
+    }
+  } else {
+    // butterfly (0, 0): rows k2 pair with (16 - k2) mod 16; (0, 8): with 15 - k2
+    const float2* af = reinterpret_cast<const float2*>(ab);
+    auto A = [&](int r, int h) { return __ldcg(af + 2 * (3 * (r >> 1) + (r & 1)) * kT + h); };
+    auto B = [&](int r) { return __ldcg(af + 2 * (3 * (r >> 1) + 2) * kT + (r & 1)); };
+    const float2 ends = B(0);  // B of rows 0 and 8, both real
+    float2 ya[16];
+#pragma unroll
+    for (int r = 0; r < 16; ++r) {
+      const float2 b = r == 0 ? make_float2(ends.x, 0.f)
+                     : r == 8 ? make_float2(ends.y, 0.f)
+                     : r < 8 ? B(r) : cconj(B(16 - r));
+      ya[r] = packed_product(za[r], za[(16 - r) & 15], A(r, 0), b);
+      acc = fmaf(ya[r].x, ya[r].x, fmaf(ya[r].y, ya[r].y, acc));
+    }
+#pragma unroll
+    for (int r = 0; r < 16; ++r) {
+      const float2 b = r < 8 ? B(8 + r) : cconj(B(8 + 15 - r));
+      yb[r] = packed_product(zb[r], zb[15 - r], A(15 - r, 1), b);
+      acc = fmaf(yb[r].x, yb[r].x, fmaf(yb[r].y, yb[r].y, acc));
+    }
+#pragma unroll
+    for (int r = 0; r < 16; ++r) za[r] = ya[r];
+  }
+  dft<16, true>(za);
+  dft<16, true>(yb);
+  acc = warp_sum(acc);
+  if ((t & 31) == 0) SM::red(ui)[t >> 5] = acc;
+  if constexpr (WAIT) cluster_wait();
+#pragma unroll
+  for (int r = 0; r < 8; ++r)
+    pa[r] = make_float4(za[2 * r].x, za[2 * r].y, za[2 * r + 1].x, za[2 * r + 1].y);
+#pragma unroll
+  for (int r = 0; r < 8; ++r)
+    pb[r] = make_float4(yb[2 * r].x, yb[2 * r].y, yb[2 * r + 1].x, yb[2 * r + 1].y);
+}
+
+// Order the middle after stage 2 (mid_enter) and before stage 2' (mid_leave):
+// within the warp.  In unit 0 the middle of warp w also reads and writes block
+// 16 - w of column 0, which warp w - 1 holds (warp 0: block 8 of warp 7), so
+// each warp hands over to one neighbour through a named barrier of the two
+// warps, and all of them still drift; with two units in a CTA there are too
+// few named barriers for that, and the unit synchronises.
+__device__ __forceinline__ void pair_sync(int id) {
+  asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory");
+}
+__device__ __forceinline__ void pair_arrive(int id) {
+  asm volatile("bar.arrive %0, 64;" ::"r"(id) : "memory");
+}
+template <int U>
+__device__ __forceinline__ void mid_enter(int ui, int ug) {
+  __syncwarp();
+  if (ug != 0) return;
+  if constexpr (U > 1) {
+    unit_sync<U>(ui);
+  } else {
+    const int w8 = threadIdx.x >> 5;
+    if (w8 < 7) pair_arrive(w8 + 1);
+    if (w8 == 0 || w8 == 7) pair_sync(15);  // both wait: mid_leave uses 15 the other way
+    if (w8 > 0) pair_sync(w8);
+  }
+}
+template <int U>
+__device__ __forceinline__ void mid_leave(int ui, int ug) {
+  __syncwarp();
+  if (ug != 0) return;
+  if constexpr (U > 1) {
+    unit_sync<U>(ui);
+  } else {
+    const int w8 = threadIdx.x >> 5;
+    pair_arrive(w8 == 0 ? 15 : 7 + w8);
+    pair_sync(w8 == 7 ? 15 : 8 + w8);
+  }
+}
+
+// Stage 2': separate in, interleaved out.
+template <int U>
+__device__ __forceinline__ void stage2i(int ui) {
+  using SM = Sm<U>;
+  const int lane = threadIdx.x & 31, w8 = unit_tid() >> 5;
+  const int k0 = lane < 16 ? w8 : 15 - w8, n0 = lane & 15;
+  float4* blk = SM::rows(ui) + k0 * kBlk;
+  const float2* c = reinterpret_cast<const float2*>(blk) + n0;
+  float2 va[16], vb[16];
+#pragma unroll
+  for (int r = 0; r < 16; ++r) {
+    va[r] = c[18 * r];
+    vb[r] = c[288 + 18 * r];
+  }
+  const float2* w = SM::u2() + n0;
+  dft16x2<true, false>(va, vb, [&](int q) {
+    const float2 s = w[16 * q];
+    return make_float4(s.x, s.y, s.x, s.y);
+  });
+  __syncwarp();
+#pragma unroll
+  for (int k = 0; k < 16; ++k)
+    blk[n0 + 16 * k] = make_float4(va[rev<16>(k)].x, va[rev<16>(k)].y, vb[rev<16>(k)].x,
+                                   vb[rev<16>(k)].y);
+}
+
+// Stage 1': rows j of every block, in place; outputs by n2 in natural order.
+template <int U>
+__device__ __forceinline__ void stage1i_compute(int ui, float2 (&va)[16], float2 (&vb)[16]) {
+  using SM = Sm<U>;
+  const int j = unit_tid();
+  const float4* row = SM::rows(ui) + j;
+#pragma unroll
+  for (int r = 0; r < 16; ++r) {
+    const float4 v = row[r * kBlk];
+    va[r] = make_float2(v.x, v.y);
+    vb[r] = make_float2(v.z, v.w);
+  }
+  const float2* w = SM::u1() + j;
+  dft16x2<true, false>(va, vb, [&](int q) {
+    const float2 s = w[256 * q];
+    return make_float4(s.x, s.y, s.x, s.y);
+  });
+}
+template <int U>
+__device__ __forceinline__ void stage1i_store(int ui, const float2 (&va)[16],
+                                              const float2 (&vb)[16]) {
+  float4* row = Sm<U>::rows(ui) + unit_tid();
+#pragma unroll
+  for (int k = 0; k < 16; ++k)
+    row[k * kBlk] = make_float4(va[rev<16>(k)].x, va[rev<16>(k)].y, vb[rev<16>(k)].x,
+                                vb[rev<16>(k)].y);
+}
+template <int U>
+__device__ __forceinline__ void stage1i(int ui) {
+  float2 va[16], vb[16];
+  stage1i_compute<U>(ui, va, vb);
+  stage1i_store<U>(ui, va, vb);
+}
+
+// Sum |Y|^2 of a unit, in warp order (after a barrier that follows the middle).
+template <int U>
+__device__ __forceinline__ float unit_power(int ui) {
+  float s = 0.f;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) s += Sm<U>::red(ui)[w];
+  return s;
+}
+
+// sigma from the units' shares (Eq. PT on the packed spectrum).
+__device__ __forceinline__ float sigma_of(const float* shares, int units, int N) {
+  float tot = 0.f;
+  for (int q = 0; q < units; ++q) tot += shares[q];
+  return sqrtf(2.0f * tot) / (float)N;
+}
+
+// Stage c and the tails of rows [rank F/C, (rank + 1) F/C) of a group of C
+// CTAs (32 / S rows a thread); rowptr: the rows of the group's units.  All
+// rows are loaded at once, so their latency (distributed shared memory) is
+// paid once; a warp in which some value passes reads them again one by one.
+template <int S, int U>
+struct Combine {
+  static constexpr int C = S / 2 / U;
+  static constexpr int per = kF / C;
+  static constexpr int R = per / (kT * U);
+  float2 w[R][S / 2];
+
+  static __device__ __forceinline__ int row(int rank, int r) {
+    return rank * per + r * (kT * U) + (int)threadIdx.x;
+  }
+  static __device__ __forceinline__ int slot(int n1) { return (n1 >> 8) * kBlk + (n1 & 255); }
+  static __device__ __forceinline__ void load(float4* const* rowptr, int at, float2 (&t)[S]) {
+#pragma unroll
+    for (int u = 0; u < S / 2; ++u) {
+      const float4 v = rowptr[u][at];
+      t[u] = make_float2(v.x, v.y);
+      t[u == 0 ? S / 2 : S - u] = make_float2(v.z, v.w);
+    }
+  }
+  __device__ __forceinline__ void twiddles(const float2* __restrict__ uc, int rank) {
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+      for (int q = 0; q < S / 2; ++q) w[r][q] = __ldg(uc + q * kF + row(rank, r));
+  }
+  template <bool EXT>
+  __device__ __forceinline__ void emit(float4* const* rowptr, const float2* __restrict__ uc,
+                                       int rank, float thr, uint32_t tmpl, int64_t krow,
+                                       const TailOut& a, float sigma) {
+    float2 t[R][S];
+#pragma unroll
+    for (int r = 0; r < R; ++r) load(rowptr, slot(row(rank, r)), t[r]);
+    float big = 0.f;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      dft_row<S, true>(t[r], [&](int q) { return w[r][q]; });
+#pragma unroll
+      for (int k = 0; k < S; ++k) big = fmaxf(big, fmaxf(fabsf(t[r][k].x), fabsf(t[r][k].y)));
+    }
+    if (a.dump || __any_sync(0xffffffffu, big > thr * (float)(S * kF))) {
+#pragma unroll 1
+      for (int r = 0; r < R; ++r) {
+        const int n1 = row(rank, r);
+        float2 x[S], o[S];
+        load(rowptr, slot(n1), x);
+        dft_row<S, true>(x, [&](int q) { return __ldg(uc + q * kF + n1); });
+#pragma unroll
+        for (int k = 0; k < S; ++k) o[k] = x[rev<S>(k)];
+        emit_row<S, kF, EXT>(o, n1, S * kF, thr, tmpl, krow, a, sigma);
+      }
+    }
+  }
+};
+
+// S = 2 (one unit, no cluster): stage 1', stage c and the tails in one go.
+// The rows reach shared memory only where some value of the warp passes.
+template <bool EXT>
+__device__ __forceinline__ void finish_s2(const float2* __restrict__ uc, float thr, uint32_t tmpl,
+                                          int64_t krow, const TailOut& a, float sigma) {
+  constexpr int S = 2;
+  const int j = unit_tid();
+  float2 va[16], vb[16];
+  stage1i_compute<1>(0, va, vb);
+  float big = 0.f;
+#pragma unroll
+  for (int k = 0; k < 16; ++k) {
+    const float2 s = __ldg(uc + j + 256 * k);
+    float2 &x = va[rev<16>(k)], &y = vb[rev<16>(k)];
+    bfly<true, 0>(x, y, s.x, s.y);
+    big = fmaxf(big, fmaxf(fmaxf(fabsf(x.x), fabsf(x.y)), fmaxf(fabsf(y.x), fabsf(y.y))));
+  }
+  if (a.dump || __any_sync(0xffffffffu, big > thr * (float)(S * kF))) {
+    stage1i_store<1>(0, va, vb);  // this thread's own rows
+    const float4* row = Sm<1>::rows(0) + j;
+#pragma unroll 1
+    for (int k = 0; k < 16; ++k) {
+      const float4 v = row[k * kBlk];
+      float2 o[2] = {make_float2(v.x, v.y), make_float2(v.z, v.w)};
+      emit_row<S, kF, EXT>(o, j + 256 * k, S * kF, thr, tmpl, krow, a, sigma);
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
+// S2-S6 of one segment: C = S / 2 / U CTAs of a cluster share a template
+// ---------------------------------------------------------------------------
+template <int S, int U, bool HALFZ, bool EXT>
+__global__ void __launch_bounds__(kT * U, U == 1 ? 2 : 1) unit_kernel(PlanDev p, CorrelateArgs a) {
+  constexpr int C = S / 2 / U;
+  using SM = Sm<U>;
+  cg::cluster_group cluster = cg::this_cluster();
+  const int rank = C == 1 ? 0 : (int)cluster.block_rank();
+  const int ui = U == 1 ? 0 : (int)threadIdx.x / kT;
+  const int ug = rank * U + ui;
+  setup_common<U>(p);
+  setup_unit<U>(p, S, ug, ui);
+  if constexpr (C > 1) {
+    if (threadIdx.x < S / 2)
+      SM::rowptr()[threadIdx.x] = cluster.map_shared_rank(
+          SM::rows(0), (unsigned)threadIdx.x / U) + (threadIdx.x % U) * (SM::L::unit_bytes / 16);
+    cluster_arrive();  // paired with the wait of the first stage 1
+  } else if constexpr (S > 2) {
+    if (threadIdx.x < S / 2) SM::rowptr()[threadIdx.x] = SM::rows((int)threadIdx.x);
+  }
+  __syncthreads();
+
+  const int cid = blockIdx.x / C, ncl = gridDim.x / C;
+  const int nz = (int)(a.Lp / 2), nfold = (nz + kF - 1) / kF;
+  const TailOut out{a.recs, a.cap, a.counter, a.dump, a.proj, a.kappa_hi, a.lag_end};
+  for (int64_t k = a.k0 + cid; k < a.k1; k += ncl) {
+    stage1<U, HALFZ, (C > 1)>(ui, S, ug, a.bank + k * a.Lp, nz, nfold);
+    unit_sync<U>(ui);
+    stage2<U>(ui);
+    mid_enter<U>(ui, ug);
+    middle<U, (S <= 4 ? 2 : 1)>(ui, ug, a.AB);
+    mid_leave<U>(ui, ug);
+    stage2i<U>(ui);
+    unit_sync<U>(ui);
+    const int64_t krow = k - a.k0;
+    if constexpr (S == 2) {
+      const float share = unit_power<U>(0);
+      const float sigma = sigma_of(&share, 1, S * 2 * kF);
+      if (threadIdx.x == 0) a.sigma[krow] = sigma;
+      finish_s2<EXT>(p.uc, a.kappa * sigma, (uint32_t)k, krow, out, sigma);
+    } else {
+      stage1i<U>(ui);
+      if (unit_tid() == 0) {
+        const float share = unit_power<U>(ui);
+#pragma unroll
+        for (int q = 0; q < C; ++q) {
+          if constexpr (C > 1)
+            *cluster.map_shared_rank(SM::sigall() + ug, (unsigned)q) = share;
+          else
+            SM::sigall()[ug] = share;
+        }
+      }
+      if constexpr (C > 1) cluster_arrive();
+      Combine<S, U> cb;
+      cb.twiddles(p.uc, rank);
+      if constexpr (C > 1)
+        cluster_wait();  // every row and share of the cluster is ready
+      else
+        __syncthreads();
+      const float sigma = sigma_of(SM::sigall(), S / 2, S * 2 * kF);
+      if (rank == 0 && threadIdx.x == 0) a.sigma[krow] = sigma;
+      cb.template emit<EXT>(SM::rowptr(), p.uc, rank, a.kappa * sigma, (uint32_t)k, krow, out,
+                            sigma);
+      if constexpr (C > 1) {
+        __syncwarp();
+        cluster_arrive_relaxed();  // every remote value has fed a vote: the reads are done
+      } else {
+        __syncthreads();
+      }
+    }
+  }
+  if constexpr (C > 1) cluster_wait();  // the cluster's last reads of this CTA's rows
+}
+
+template <int S, int U, bool HALFZ, bool EXT>
+static cudaError_t launch_unit_t(const PlanDev& p, const CorrelateArgs& a, cudaStream_t s) {
+  constexpr int C = S / 2 / U;
+  return launch_clusters(unit_kernel<S, U, HALFZ, EXT>, C, kT * U, Lay<U>::total, U == 1 ? 2 : 1,
+                         p, a, s);
+}
+
+template <int S, int U>
+static cudaError_t launch_unit(const PlanDev& p, const CorrelateArgs& a, bool halfz,
+                               cudaStream_t s) {
+  const bool ext = a.proj || a.kappa_hi > 0.f || a.lag_end < (uint32_t)p.g.N;
+  if (halfz)
+    return ext ? launch_unit_t<S, U, true, true>(p, a, s) : launch_unit_t<S, U, true, false>(p, a, s);
+  return ext ? launch_unit_t<S, U, false, true>(p, a, s)
+             : launch_unit_t<S, U, false, false>(p, a, s);
+}
+
+}  // namespace unit
+}  // namespace bege

@@ -1,0 +1,81 @@
+"""The unit kernels (N >= 2^14) at the edges of their range: template lengths
+around the column length (one sample, odd, half a column, a column, folded
+over several), every launch shape, against the FP64 oracle; all shapes give
+the same bits, and a row gives the same bits wherever its range begins."""
+import numpy as np
+import pytest
+
+import synthetic as S
+from gpu_helpers import make_ctx, oracle_rho
+
+pytestmark = pytest.mark.gpu
+
+TOL = 1e-5        # sigma; FP32 rounding of the transforms reaches 2e-6
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    c = make_ctx()
+    yield c
+    c.close()
+
+
+@pytest.mark.parametrize("n,length", [(1 << 14, 1), (1 << 14, 4096), (1 << 14, 4097),
+                                      (1 << 14, 1 << 14), (1 << 15, 2047), (1 << 15, 8193),
+                                      (1 << 16, 7), (1 << 16, 4095), (1 << 16, 1 << 16),
+                                      (1 << 17, 4096), (1 << 17, 12289)])
+def test_edges_match_oracle_in_every_shape(ctx, n, length):
+    bank = S.random_samples_bank(5, length, 3 * n + length)
+    bank[3] = 0.0                                  # a row of zeros: no value, no tail
+    y = S.band_limited_noise(n, length)
+    rho, sig = oracle_rho(y, bank)
+    seg, bid = ctx.bege_load_segment(y), ctx.bege_define_bank_samples(bank)
+    default = ctx.bege_get_config(n)
+    seen = []
+    for shape in ctx.bege_list_configs(n):
+        ctx.bege_set_config(n, *shape)
+        dump = ctx.bege_dump_correlation(seg, bid, 0, 5)
+        job = ctx.bege_correlate(seg, bid, 0, 5, 3.0)
+        recs, total = ctx.bege_fetch_tails(job, sort=True)
+        gsig = ctx.bege_get_sigma(job, 5)
+        assert total == len(recs)
+        ctx.bege_release(job)
+        for k in range(5):
+            if k == 3:
+                assert gsig[k] == 0 and not dump[k].any() and not (recs["tmpl"] == k).any()
+                continue
+            assert abs(gsig[k] / sig[k] - 1) <= 1e-6
+            assert np.abs(dump[k] - rho[k]).max() <= TOL * sig[k]
+            hits = np.nonzero(np.abs(dump[k]) > np.float32(3.0) * gsig[k])[0]
+            mine = recs[recs["tmpl"] == k]
+            assert np.array_equal(mine["lag"], hits)
+            assert np.array_equal(mine["value"], dump[k][hits])
+        # the same row from a range that begins elsewhere
+        job = ctx.bege_correlate(seg, bid, 4, 5, 3.0)
+        assert ctx.bege_get_sigma(job, 1)[0] == gsig[4]
+        ctx.bege_release(job)
+        seen.append((dump, gsig, recs.copy()))
+    ctx.bege_set_config(n, *default)
+    for other in seen[1:]:
+        for a, b in zip(seen[0], other):
+            assert np.array_equal(a, b)
+    ctx.bege_release(seg)
+    ctx.bege_release(bid)
+
+
+def test_coefficients_and_tables_at_a_quarter_turn(ctx):
+    """One bin at a time: a cosine at bin j against a unit impulse gives the
+    cosine back at every lag (twiddles at 0, 1/4 and 1/2 turn, the self-mirrored
+    butterflies and both ends of the spectrum included)."""
+    n = 1 << 16
+    bank = np.zeros((1, 8), dtype=np.float32)
+    bank[0, 0] = 1.0
+    bid = ctx.bege_define_bank_samples(bank)
+    t = np.arange(n)
+    for j in (0, 1, 8, 128, 2048, 4096, 8192, 16383, 16384, 16385, 24576, 32767, 32768):
+        y = np.cos(2 * np.pi * ((j * t) % n) / n).astype(np.float32)
+        seg = ctx.bege_load_segment(y)
+        dump = ctx.bege_dump_correlation(seg, bid, 0, 1)[0]
+        ctx.bege_release(seg)
+        assert np.abs(dump - y).max() <= 2e-6, j
+    ctx.bege_release(bid)
