@@ -182,8 +182,9 @@ int get_plan(bege_ctx* ctx, int64_t n, std::shared_ptr<PlanHost>* out) {
   // tables: tw2 [16 R0], tw3 [F], wH [256 S], wR0S [R0 S], wS [S], wN [H]
   const size_t n_tw2 = 16 * g.R0, n_tw3 = g.F, n_wH = 256 * g.S, n_wR0S = g.R0 * g.S,
                n_wS = g.S, n_wN = g.H;
+  const bege::UnitGeo ug = bege::unit_geo(g);
   size_t n_unit = 0;
-  for (int t = 0; t < bege::kUnitTables; ++t) n_unit += bege::unit_table_size(g.S, t);
+  for (int t = 0; t < bege::kUnitTables; ++t) n_unit += bege::unit_table_size(ug, t);
   std::vector<float2> h(n_tw2 + n_tw3 + n_wH + n_wR0S + n_wS + n_wN + n_unit);
   size_t o = 0;
   const size_t o_tw2 = o;
@@ -210,8 +211,8 @@ int get_plan(bege_ctx* ctx, int64_t n, std::shared_ptr<PlanHost>* out) {
   size_t o_unit[bege::kUnitTables];
   for (int t = 0; t < bege::kUnitTables; ++t) {
     o_unit[t] = o;
-    for (int i = 0; i < bege::unit_table_size(g.S, t); ++i, ++o) {
-      const bege::Turn a = bege::unit_table_turn(g.S, t, i);
+    for (int i = 0; i < bege::unit_table_size(ug, t); ++i, ++o) {
+      const bege::Turn a = bege::unit_table_turn(ug, t, i);
       const double x = 2.0 * M_PI * (double)a.num / (double)a.den;
       h[o] = bege::rot_entry(std::cos(x), std::sin(x));
     }

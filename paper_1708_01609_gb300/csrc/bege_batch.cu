@@ -21,6 +21,7 @@ namespace {
 using namespace unit;
 
 constexpr int kNC = 2;          // columns of a CTA (one unit)
+constexpr int kT = Geo<kF>::T;
 constexpr int kCluster = 8;
 
 __device__ __forceinline__ int plan_index(int S) {
@@ -39,7 +40,7 @@ __device__ __forceinline__ void combine_group(const float2* uc, int grank, float
                                               int64_t krow, const TailOut& out) {
   Combine<S, 1> cb;
   cb.twiddles(uc, grank);
-  cb.template emit<false>(Sm<1>::rowptr(), uc, grank, thr, tmpl, krow, out, 0.f);
+  cb.template emit<false>(Sm<kF, 1>::rowptr(), uc, grank, thr, tmpl, krow, out, 0.f);
 }
 
 // One work item.  The stages do not depend on the column count S = N/8192, so
@@ -49,11 +50,11 @@ __device__ __forceinline__ void run_item(const BatchArgs& b, const ItemState* st
   const int S = st->sg.S;
   const int C = S / kNC;
   const int G = kCluster / C;
-  using SM = Sm<1>;
+  using SM = Sm<kF, 1>;
   cg::cluster_group cluster = cg::this_cluster();
   const int group = rank / C, grank = rank - group * C, gbase = group * C;
   const PlanDev& p = b.plans[plan_index(S)];
-  setup_unit<1>(p, S, grank, 0);
+  setup_unit<SM>(p, S, grank, 0);
   if (threadIdx.x < C)
     SM::rowptr()[threadIdx.x] = cluster.map_shared_rank(SM::rows(0), (unsigned)(gbase + threadIdx.x));
   __syncthreads();
@@ -64,23 +65,25 @@ __device__ __forceinline__ void run_item(const BatchArgs& b, const ItemState* st
     const int64_t krow = k - st->sg.k0;
     const TailOut out{st->sg.recs, st->sg.cap, st->sg.counter, nullptr};
     if (active) {
-      stage1<1, true, false>(0, S, grank, st->sg.bank + k * st->sg.Lp, (int)(st->sg.Lp / 2), 1);
-      unit_sync<1>(0);
-      stage2<1>(0);
-      mid_enter<1>(0, grank);
-      middle<1, 1>(0, grank, st->sg.AB);
-      mid_leave<1>(0, grank);
-      stage2i<1>(0);
-      unit_sync<1>(0);
+      stage1<SM, true, false, false>(0, S, grank, st->sg.bank + k * st->sg.Lp, (int)(st->sg.Lp / 2), 1);
+      SM::sync(0);
+      stage2<SM>(0);
+      mid_enter<SM, 1>(0, grank);
+      middle<SM, 1>(0, grank, st->sg.AB);
+      mid_leave<SM, 1>(0, grank);
+      stage2i<SM>(0);
+      SM::sync(0);
       if (C == 1) {  // one CTA holds the template: no other CTA is waited for
-        const float share = unit_power<1>(0);
+        const float share = unit_power<SM>(0);
         const float sigma = sigma_of(&share, 1, S * 2 * kF);
         if (threadIdx.x == 0) st->sg.sigma[krow] = sigma;
-        finish_s2<false>(p.uc, st->sg.kappa * sigma, (uint32_t)k, krow, out, sigma);
+        finish_s2<SM, false>(0, p.uc, st->sg.kappa * sigma, (uint32_t)k, krow, out, sigma);
       } else {
-        stage1i<1>(0);
+        float2 va[1][16], vb[1][16];
+        stage1i<SM>(0, va, vb);
+        store_blocks<SM>(0, va, vb);
         if (threadIdx.x == 0) {
-          const float share = unit_power<1>(0);
+          const float share = unit_power<SM>(0);
           for (int q = 0; q < C; ++q)
             *cluster.map_shared_rank(SM::sigall() + grank, (unsigned)(gbase + q)) = share;
         }
@@ -110,7 +113,7 @@ __global__ void __launch_bounds__(kT, 2) batch_kernel(BatchArgs b) {
   __shared__ ItemState st;
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = (int)cluster.block_rank();
-  unit::setup_common<1>(b.plans[0]);  // F-only tables: the same for every N
+  unit::setup_common<Sm<kF, 1>, kT>(b.plans[0]);  // F-only tables: the same for every N
   for (;;) {
     if (rank == 0 && threadIdx.x == 0) item_slot = (int)atomicAdd(b.queue, 1u);
     cluster.sync();
@@ -146,7 +149,7 @@ __global__ void __launch_bounds__(kT, 1) segment_batch_kernel(BatchArgs b,
 int batch_max_clusters() {
   static int cached = -1;
   if (cached >= 0) return cached;
-  constexpr size_t smem = unit::Lay<1>::total;
+  constexpr size_t smem = unit::Lay<kF, 1, false>::total;
   if (cudaFuncSetAttribute(batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
       cudaSuccess)
     return 0;
@@ -171,7 +174,7 @@ int batch_max_clusters() {
 }
 
 cudaError_t launch_batch(const BatchArgs& b, int clusters, cudaStream_t s) {
-  constexpr size_t smem = unit::Lay<1>::total;
+  constexpr size_t smem = unit::Lay<kF, 1, false>::total;
   cudaError_t e = cudaFuncSetAttribute(batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem);
   if (e != cudaSuccess) return e;

@@ -36,8 +36,9 @@
 // cluster hold all S columns and read each other's columns through
 // distributed shared memory only in the final S-point combine.
 //
-// This file: the segment kernel (every S), the one-column kernel (S = 1, N <=
-// 2^13) and the tail epilogue; bege_unit.cuh has the correlation for S >= 2.
+// This file: the segment kernel and the tail epilogue; bege_unit.cuh has the
+// correlation.  (The segment kernel takes N <= 2^13 as one column of F = H
+// points; the correlation always has at least two columns.)
 #pragma once
 
 #include <cooperative_groups.h>
@@ -201,16 +202,6 @@ __device__ __forceinline__ void forward_columns(int rank, const float* src, int 
   stockham_pass<F, NC, T, 16, 16 * R0, false>(SM::cols(), SM::tw3());
 }
 
-// One column (S = 1): the inverse transform has no column twiddle.
-template <int F, int T>
-__device__ __forceinline__ void inverse_column() {
-  using SM = Smem<F, 1>;
-  constexpr int R0 = F / 256;
-  stockham_pass<F, 1, T, R0, 1, true>(SM::cols(), nullptr);
-  stockham_pass<F, 1, T, 16, R0, true>(SM::cols(), SM::tw2());
-  stockham_pass<F, 1, T, 16, 16 * R0, true>(SM::cols(), SM::tw3());
-}
-
 // The bin pairs (j, H-j) held by a unit.  Unit 0 holds column 0 (pairs
 // a <-> (F-a) mod F, with a = 0 and a = F/2 paired with themselves) and
 // column S/2 (pairs a <-> F-1-a); unit i holds columns i and S-i (pairs
@@ -261,141 +252,42 @@ __device__ __forceinline__ float warp_sum(float v) {
 }
 
 // ---------------------------------------------------------------------------
-// Fused middle of the one-column pipeline for F = 4096 (S = 1, radix 16 x 16
-// x 16): the last forward pass, the spectral product with the Parseval sum,
-// and the first inverse pass, in registers.
-//
-// Forward pass 3 (Ns = 256) reads and writes the rows j + 256 r of its
-// butterfly j, and inverse pass 1 (Ns = 1) reads the same rows, so one thread
-// can carry a butterfly from the forward FFT into the inverse FFT.  Row
-// j + 256 r pairs with (256-j) + 256 (15-r), i.e. with row 15-r of the mirror
-// butterfly, so a thread that holds a butterfly and its mirror (128 threads;
-// thread 0 the two self-mirrored butterflies 0 and 128) forms every Y of
-// both.  Returns this thread's sum of |Y|^2; ends with the stores of inverse
-// pass 1 (callers synchronise before reading the column).
-// ---------------------------------------------------------------------------
-template <int T>
-__device__ __forceinline__ float fused_mid(const float4* __restrict__ AB, float* red_warp) {
-  constexpr int F = 4096;
-  using SM = Smem<F, 1>;
-  static_assert(T >= 128, "one item per thread");
-  constexpr int step = 256 + 16;             // padded distance of rows r -> r + 1
-  const int t = threadIdx.x;
-  const bool act = t < 128;
-  const bool self0 = t == 0;                 // butterflies 0 and 128 (each its own mirror)
-  const int ja = t, jb = self0 ? 128 : 256 - t;
-  float2 za[16], zb[16];
-  float acc = 0.f;
-  if (act) {
-    const float2* pa = SM::col(0) + pad(ja);
-    const float2* pb = SM::col(0) + pad(jb);
-#pragma unroll
-    for (int r = 0; r < 16; ++r) {
-      za[r] = pa[r * step];
-      zb[r] = pb[r * step];
-    }
-    const float2* ta = SM::tw3() + ja;
-    const float2* tb = SM::tw3() + jb;
-#pragma unroll
-    for (int r = 1; r < 16; ++r) {
-      za[r] = cmul(za[r], ta[r * 256]);
-      zb[r] = cmul(zb[r], tb[r * 256]);
-    }
-    dft<16, false>(za);
-    dft<16, false>(zb);
-    const float4* aba = AB + ja;
-    const float4* abb = AB + jb;
-    if (!self0) {
-      // za[r] (row ja + 256 r) pairs with zb[15 - r] (row jb + 256 (15 - r))
-#pragma unroll
-      for (int r = 0; r < 16; ++r) {
-        const float4 p = __ldcg(aba + 256 * r);
-        const float4 q = __ldcg(abb + 256 * (15 - r));
-        const float2 x = za[r], y = zb[15 - r];
-        const float2 ya = packed_product(x, y, p);
-        const float2 yb = packed_product(y, x, q);
-        acc = fmaf(ya.x, ya.x, fmaf(ya.y, ya.y, acc));
-        acc = fmaf(yb.x, yb.x, fmaf(yb.y, yb.y, acc));
-        za[r] = ya;
-        zb[15 - r] = yb;
-      }
-    } else {
-      // butterfly 0: rows 256 r pair with 256 ((16 - r) mod 16); r = 0, 8 self
-      float2 ya[16], yb[16];
-#pragma unroll
-      for (int r = 0; r < 16; ++r) {
-        const int rp = (16 - r) & 15;
-        const float4 p = __ldcg(aba + 256 * r);
-        ya[r] = packed_product(za[r], za[rp], p);
-        acc = fmaf(ya[r].x, ya[r].x, fmaf(ya[r].y, ya[r].y, acc));
-      }
-      // butterfly 128: rows 128 + 256 r pair with 128 + 256 (15 - r)
-#pragma unroll
-      for (int r = 0; r < 16; ++r) {
-        const float4 q = __ldcg(abb + 256 * r);
-        yb[r] = packed_product(zb[r], zb[15 - r], q);
-        acc = fmaf(yb[r].x, yb[r].x, fmaf(yb[r].y, yb[r].y, acc));
-      }
-#pragma unroll
-      for (int r = 0; r < 16; ++r) {
-        za[r] = ya[r];
-        zb[r] = yb[r];
-      }
-    }
-    dft<16, true>(za);
-    dft<16, true>(zb);
-  }
-  acc = warp_sum(acc);
-  if ((t & 31) == 0) red_warp[t >> 5] = acc;
-  __syncthreads();  // every load of the columns is done
-  if (act) {
-    // inverse pass 1 (Ns = 1): butterfly j writes rows 16 j + r
-    float2* qa = SM::col(0) + pad(16 * ja);
-    float2* qb = SM::col(0) + pad(16 * jb);
-#pragma unroll
-    for (int r = 0; r < 16; ++r) qa[r] = za[r];
-#pragma unroll
-    for (int r = 0; r < 16; ++r) qb[r] = zb[r];
-  }
-  return acc;
-}
-
-// ---------------------------------------------------------------------------
 // S1: segment spectrum D and product coefficients A, B (grid: C CTAs)
 // ---------------------------------------------------------------------------
 // Where the middle of bege_unit.cuh reads the coefficients of bin S a + b:
-// unit u, thread t of 256, row r, half h (the thread's butterfly or its
+// unit u, thread t of T = F / 16, row r, half h (the thread's butterfly or its
 // mirror, whose rows run backwards).  Since B_{H-j} = conj B_j, a mirror pair
 // keeps one B: rows 2 i, 2 i + 1 of a thread are the three float4 {A, A'} of
-// either row and {B, B}, 256 apart.  Thread 0 of unit 0 holds two butterflies
-// of column 0 that are their own mirrors: bins S 256 r have their B at row r
-// < 8 (row 0: the real B of r = 0 and of r = 8), bins S (128 + 256 r) at row
-// 8 + r.
+// either row and {B, B}, T apart.  Thread 0 of unit 0 holds two butterflies
+// of column 0 that are their own mirrors, rows 16 R r of it and 8 R + 16 R r: the
+// first have their B at row r < 8 (row 0: the real B of r = 0 and of r = 8),
+// the others at row 8 + r.
 struct CoefPlace {
   int a, b, bc;  // float2 index of A; of B or -1; component of a real B (else -1)
 };
 template <int F, int S>
 __host__ __device__ __forceinline__ CoefPlace coef_place(int b, int a) {
-  int k0 = a & 15, k1 = (a >> 4) & 15, r = a >> 8;
+  constexpr int R = F / 256, T = F / 16;
+  int k0 = a & (R - 1), k1 = (a / R) & 15, r = a / (16 * R);
   int u = 0, h = 0, t;
   if (b != 0 && b != S / 2) {
     h = b > S / 2;
     u = h ? S - b : b;
-    if (h) { k0 = 15 - k0; k1 = 15 - k1; }
-    t = (k0 < 8 ? 32 * k0 : 32 * (15 - k0) + 16) + k1;
+    if (h) { k0 = R - 1 - k0; k1 = 15 - k1; }
+    t = (k0 < R / 2 ? 32 * k0 : 32 * (R - 1 - k0) + 16) + k1;
   } else if (b != 0) {  // column S/2
-    h = k0 >= 8;
-    if (h) { k0 = 15 - k0; k1 = 15 - k1; }
-    t = 32 * k0 + 16 + k1;
-  } else if (k0 == 0) {  // column 0: butterfly j = k0 + 16 k1 and 256 - j
+    h = R == 1 ? k1 >= 8 : k0 >= R / 2;
+    if (h) { k0 = R - 1 - k0; k1 = 15 - k1; }
+    t = R == 1 ? 8 + k1 : 32 * k0 + 16 + k1;
+  } else if (k0 == 0) {  // column 0: butterfly j = k0 + R k1 and 16 R - j
     h = k1 >= 8;
     t = k1 <= 8 ? k1 & 7 : 16 - k1;
-  } else if (k0 == 8) {
+  } else if (k0 == R / 2) {
     h = k1 >= 8;
     t = 8 + (h ? 15 - k1 : k1);
   } else {
-    h = k0 > 8;
-    if (h) { k0 = 16 - k0; k1 = 15 - k1; }
+    h = k0 > R / 2;
+    if (h) { k0 = R - k0; k1 = 15 - k1; }
     t = 32 * k0 + k1;
   }
   int br = h ? -1 : r, bc = -1;
@@ -408,19 +300,20 @@ __host__ __device__ __forceinline__ CoefPlace coef_place(int b, int a) {
     }
   }
   if (h) r = 15 - r;
-  auto at = [&](int row, int third) { return 2 * (((u * 8 + (row >> 1)) * 3 + third) * 256 + t); };
+  auto at = [&](int row, int third) { return 2 * (((u * 8 + (row >> 1)) * 3 + third) * T + t); };
   return {at(r, r & 1) + h, br < 0 ? -1 : at(br, 2) + (br & 1), bc};
 }
-// Stores {A, B} of bin S a + b.  natural: at b F + a (one column, and the
-// tensor-core kernel).
+// Stores {A, B} of bin j; natural (the tensor-core kernel): at b F + a for j =
+// S a + b.
 template <int F, int S>
-__device__ __forceinline__ void store_coef(float4* AB, int b, int a, float4 ab, bool natural) {
-  if (S == 1 || natural) {
-    AB[b * F + a] = ab;
+__device__ __forceinline__ void store_coef(float4* AB, int j, float4 ab, bool natural) {
+  if (S > 1 && natural) {
+    AB[(j % S) * F + j / S] = ab;
     return;
   }
+  constexpr int Fu = S == 1 ? F / 2 : F, Su = S == 1 ? 2 : S;
   float2* c = reinterpret_cast<float2*>(AB);
-  const CoefPlace p = coef_place<F, S>(b, a);
+  const CoefPlace p = coef_place<Fu, Su>(j % Su, j / Su);
   c[p.a] = make_float2(ab.x, ab.y);
   if (p.bc >= 0)
     reinterpret_cast<float*>(c + p.b)[p.bc] = ab.z;
@@ -475,10 +368,10 @@ __device__ __forceinline__ void segment_body(const PlanDev& p, int rank,
         const float2 B = cmul(cmul(gg, de), cadd(Dx, cH));
         return make_float4(A.x, A.y, B.x, B.y);
       };
-      store_coef<F, S>(AB, q.b, q.a, coeffs(wj, Dj, cHj), natural);
+      store_coef<F, S>(AB, j, coeffs(wj, Dj, cHj), natural);
       D[j] = Dj;
       if (!self) {
-        store_coef<F, S>(AB, q.bp, q.ap, coeffs(p.wN[jp], Djp, cHjp), natural);
+        store_coef<F, S>(AB, jp, coeffs(p.wN[jp], Djp, cHjp), natural);
         D[jp] = Djp;
       }
       if (j == 0) D[H] = DH;
@@ -614,75 +507,6 @@ __device__ __forceinline__ void combine_and_emit(float2* const* colptr, int H, i
   }
 }
 
-// S2-S6 for N <= 2^13: one column, one CTA per template.
-template <int F, int T, int MINB, bool HALFZ, bool EXT>
-__global__ void __launch_bounds__(T, MINB) correlate_kernel(PlanDev p, CorrelateArgs a) {
-  using SM = Smem<F, 1>;
-  const int N = p.g.N, H = p.g.H;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  setup_common<F, 1, T>(p);
-  setup_columns<F, 1, 1, T>(p, 0);
-  __syncthreads();
-
-  const int nz = (int)(a.Lp / 2);
-  const int nfold = (nz + F - 1) / F;
-  const TailOut out{a.recs, a.cap, a.counter, a.dump, a.proj, a.kappa_hi, a.lag_end};
-  for (int64_t k = a.k0 + blockIdx.x; k < a.k1; k += gridDim.x) {
-    const float* src = a.bank + k * a.Lp;
-    if constexpr (F == 4096) {
-      // S2: forward passes 1-2; S2-S5 fused: forward pass 3, the product
-      // Y = conj(Z) A + Z' B with sum |Y|^2, inverse pass 1; S5: passes 2-3
-      fwd_first_pass<F, 1, 1, T, HALFZ>(0, src, nz, nfold);
-      stockham_pass<F, 1, T, 16, 16, false>(SM::cols(), SM::tw2());
-      fused_mid<T>(a.AB, SM::red());
-      __syncthreads();
-      stockham_pass<F, 1, T, 16, 16, true>(SM::cols(), SM::tw2());
-      stockham_pass<F, 1, T, 16, 256, true>(SM::cols(), SM::tw3());
-    } else {
-      // S2: template spectrum
-      forward_columns<F, 1, 1, T, HALFZ>(0, src, nz, nfold);
-      // S3 + S4: Y = conj(Z) A + Z' B over the bin pairs, sum |Y|^2
-      float acc = 0.f;
-      const int count = unit_items<F, 1>(0);
-#pragma unroll 2
-      for (int it = threadIdx.x; it < count; it += T) {
-        const PairItem q = pair_item<F, 1>(0, 0, it);
-        float2* cj = SM::col(q.sj) + pad(q.a);
-        float2* cp = SM::col(q.sp) + pad(q.ap);
-        const float4 abj = __ldcg(a.AB + q.a);
-        const float4 abp = __ldcg(a.AB + q.ap);
-        const float2 zj = *cj, zp = *cp;
-        const float2 yj = packed_product(zj, zp, abj);
-        acc = fmaf(yj.x, yj.x, fmaf(yj.y, yj.y, acc));
-        if (cj != cp) {
-          const float2 yp = packed_product(zp, zj, abp);
-          acc = fmaf(yp.x, yp.x, fmaf(yp.y, yp.y, acc));
-          *cp = yp;
-        }
-        *cj = yj;
-      }
-      acc = warp_sum(acc);
-      if (lane == 0) SM::red()[warp] = acc;
-      __syncthreads();
-      // S5: inverse column FFT
-      inverse_column<F, T>();
-    }
-    float tot = 0.f;  // Eq. PT on the packed spectrum
-#pragma unroll
-    for (int w = 0; w < T / 32; ++w) tot += SM::red()[w];
-    const float sigma = sqrtf(2.0f * tot) / (float)N;
-    const int64_t krow = k - a.k0;
-    if (threadIdx.x == 0) a.sigma[krow] = sigma;
-    // S6: threshold, warp-ballot compaction
-#pragma unroll 1
-    for (int n1 = threadIdx.x; n1 < F; n1 += T) {
-      const float2 t[1] = {SM::col(0)[pad(n1)]};
-      emit_row<1, F, EXT>(t, n1, H, a.kappa * sigma, (uint32_t)k, krow, out, sigma);
-    }
-    __syncthreads();  // the column is read before the next template overwrites it
-  }
-}
-
 // ---------------------------------------------------------------------------
 // Launch helpers
 // ---------------------------------------------------------------------------
@@ -692,9 +516,9 @@ static cudaError_t ensure_smem(K kernel, size_t bytes) {
 }
 
 // Launches `kern` with clusters of C CTAs (minb CTAs per SM), as many as fit
-// and are needed for the templates of a.
+// and are needed for the templates of a, `each` at a time per cluster.
 template <typename K>
-static cudaError_t launch_clusters(K kern, int C, int threads, size_t smem, int minb,
+static cudaError_t launch_clusters(K kern, int C, int threads, size_t smem, int minb, int each,
                                    const PlanDev& p, const CorrelateArgs& a, cudaStream_t s) {
   cudaError_t e = ensure_smem(kern, smem);
   if (e != cudaSuccess) return e;
@@ -719,21 +543,11 @@ static cudaError_t launch_clusters(K kern, int C, int threads, size_t smem, int 
   e = cudaOccupancyMaxActiveClusters(&max_clusters, kern, &cfg);
   if (e != cudaSuccess) return e;
   if (max_clusters < 1) return cudaErrorInvalidConfiguration;
-  int64_t want = a.k1 - a.k0;
+  int64_t want = (a.k1 - a.k0 + each - 1) / each;
   if (a.max_clusters > 0 && want > a.max_clusters) want = a.max_clusters;
   if (want > max_clusters) want = max_clusters;
   cfg.gridDim = dim3((unsigned)(want * C), 1, 1);
   return cudaLaunchKernelEx(&cfg, kern, p, a);
-}
-
-// The extended epilogue (bege_correlate_max, bege_correlate_band,
-// bege_correlate_ex) runs in its own instantiation.
-template <int F, int T, int MINB, bool HALFZ>
-static cudaError_t launch_corr_t(const PlanDev& p, const CorrelateArgs& a, cudaStream_t s) {
-  const bool ext = a.proj || a.kappa_hi > 0.f || a.lag_end < (uint32_t)p.g.N;
-  constexpr size_t smem = Lay<F, 1>::total;
-  return ext ? launch_clusters(correlate_kernel<F, T, MINB, HALFZ, true>, 1, T, smem, MINB, p, a, s)
-             : launch_clusters(correlate_kernel<F, T, MINB, HALFZ, false>, 1, T, smem, MINB, p, a, s);
 }
 
 template <int F, int S, int NC, int T>

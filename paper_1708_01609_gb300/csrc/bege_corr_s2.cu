@@ -1,12 +1,11 @@
-// Correlate kernels for S = 2 columns (N = 2^14).
+// Correlate kernels for N = 2^14 (two columns of 4096 points).
 #include "bege_unit.cuh"
 
 namespace bege {
 
-cudaError_t launch_correlate_s2(const PlanDev& p, const CorrelateArgs& a, CorrConfig c,
-                                 bool halfz, cudaStream_t s) {
-  if (c.nc == 2 && c.threads == 256) return unit::launch_unit<2, 1>(p, a, halfz, s);
-  return cudaErrorInvalidValue;
+cudaError_t launch_correlate_s2(const PlanDev& p, const CorrelateArgs& a, cudaStream_t s) {
+  return a.Lp <= unit::kF ? unit::launch_short<unit::kF, true>(p, a, s)
+                          : unit::launch_short<unit::kF, false>(p, a, s);
 }
 
 }  // namespace bege

@@ -48,27 +48,35 @@ struct PlanDev {
   const float2* wR0S;  // [R0*S]   w(R0 S)^q
   const float2* wS;    // [S]      wS^q
   const float2* wN;    // [H]      wN^j
-  // S >= 2, {cos, tan} sets of bege_unit.cuh (rot_entry, set_turns):
-  const float2* t1;    // [S][8]         stage 1: column b
-  const float2* t2;    // [S][8][16]     stage 2: column b, k0
-  const float2* t3;    // [S/2][8][256]  stage 3: unit, thread
-  const float2* u2;    // [8][16]        stage 2': n0
-  const float2* u1;    // [8][256]       stage 1': n0 + 16 n1
-  const float2* uc;    // [S/2][4096]    stage c: n
+  // tables of bege_unit.cuh for its columns (UnitGeo), {cos, tan} pairs
+  // (rot_entry, unit_table_turn)
+  const float2* t1;    // [S][R/2]     stage 1: column b
+  const float2* t2;    // [S][8][R]    stage 2: column b, k0
+  const float2* t3;    // [S/2][8][T]  stage 3: unit, thread
+  const float2* u2;    // [8][16]      stage 2': n0
+  const float2* u1;    // [R/2][256]   stage 1': n0 + 16 n1
+  const float2* uc;    // [S/2][F]     stage c: n
 };
 
-// Sizes (in float2) of the sets of an S-column plan, in the order t1, t2, t3,
-// u2, u1, uc; all 0 for S = 1.
+// The correlation's columns: S >= 2 of F points, R = F / 256 and T = F / 16
+// threads for two of them.
+struct UnitGeo {
+  int F, S, R, T;
+};
+constexpr __host__ __device__ UnitGeo unit_geo(const Geometry& g) {
+  return g.S == 1 ? UnitGeo{g.F / 2, 2, g.F / 512, g.F / 32} : UnitGeo{g.F, g.S, g.F / 256, g.F / 16};
+}
+
+// Sizes (in float2) of the pair tables, in the order t1, t2, t3, u2, u1, uc.
 constexpr int kUnitTables = 6;
-constexpr __host__ __device__ int unit_table_size(int S, int table) {
-  if (S < 2) return 0;
+constexpr __host__ __device__ int unit_table_size(const UnitGeo& g, int table) {
   switch (table) {
-    case 0: return 8 * S;
-    case 1: return 128 * S;
-    case 2: return 1024 * S;
+    case 0: return g.S * (g.R / 2);
+    case 1: return g.S * 8 * g.R;
+    case 2: return g.S / 2 * 8 * g.T;
     case 3: return 128;
-    case 4: return 2048;
-    default: return 2048 * S;
+    case 4: return g.R / 2 * 256;
+    default: return g.S / 2 * g.F;
   }
 }
 
@@ -76,53 +84,43 @@ constexpr __host__ __device__ int unit_table_size(int S, int table) {
 struct Turn {
   int64_t num, den;
 };
-inline __host__ __device__ Turn unit_table_turn(int S, int table, int i) {
-  int64_t x = 0, M = 1;  // base x / M turns
-  int q = 0;             // place in the 16-point set
+// Pair q of an R-point DFT with twiddle base x / M turns: the levels one
+// after the other, level l with (R / 2^(l+1)) x base + e / 2^(l+1), e < max(1, 2^(l-1)).
+inline __host__ __device__ Turn dft_pair_turn(int R, int q, int64_t x, int64_t M) {
+  int l = 0, n = 1;
+  while (q >= n) {
+    q -= n;
+    ++l;
+    n = l > 1 ? 1 << (l - 1) : 1;
+  }
+  const int64_t den = M << (l + 1);
+  return {((x * (R >> (l + 1)) << (l + 1)) + q * M) % den, den};
+}
+inline __host__ __device__ Turn unit_table_turn(const UnitGeo& g, int table, int i) {
+  const int R = g.R, S = g.S, T = g.T;
+  const int64_t H = (int64_t)S * g.F;
   switch (table) {
-    case 0: q = i & 7; x = i >> 3; M = 16 * S; break;
-    case 1: {
-      const int b = i >> 7, k0 = i & 15;
-      q = (i >> 4) & 7; x = S * k0 + b; M = 256 * S;
-      break;
-    }
+    case 0: return dft_pair_turn(R, i % (R / 2), i / (R / 2), R * S);
+    case 1: return dft_pair_turn(16, i / R % 8, (int64_t)S * (i % R) + i / (8 * R), 16 * R * S);
     case 2: {
       // thread t of the middle of unit u holds butterfly (k0, k1) of column b
-      const int u = i >> 11, t = i & 255, l = t & 15;
+      const int u = i / (8 * T), t = i % T, l = t & 15, w = t >> 5;
       int b = u, k0, k1 = l;
       if (u > 0) {
-        k0 = (t & 16) ? 15 - (t >> 5) : t >> 5;
-      } else if (t & 16) {
-        b = S / 2; k0 = t >> 5;
-      } else if (t >= 32) {
-        k0 = t >> 5;
+        k0 = (t & 16) ? R - 1 - w : w;
+      } else if (R == 1 ? l >= 8 : (t & 16) != 0) {
+        b = S / 2; k0 = w;
+        if (R == 1) k1 = l - 8;
+      } else if (w > 0) {
+        k0 = w;
       } else {
-        k0 = l < 8 ? 0 : 8; k1 = l & 7;
+        k0 = l < 8 ? 0 : R / 2; k1 = l & 7;
       }
-      q = (i >> 8) & 7; x = (int64_t)S * (k0 + 16 * k1) + b; M = 4096 * (int64_t)S;
-      break;
+      return dft_pair_turn(16, i / T % 8, (int64_t)S * (k0 + R * k1) + b, H);
     }
-    case 3: q = i >> 4; x = i & 15; M = 256; break;
-    case 4: q = i >> 8; x = i & 255; M = 4096; break;
-    default: {
-      // the S-point DFT uses the end of the set: S = 2 {base}, 4 {2 x base,
-      // base}, 8 {4 x, 2 x, base, base + 1/8}, 16 the whole set
-      const int e = i >> 12;
-      x = i & 4095; M = 4096 * (int64_t)S;
-      const int64_t den = 16 * M;
-      if (S == 16) { q = e; break; }
-      if (S == 8 && e == 3) return {(16 * x + 2 * M) % den, den};
-      const int levels = S == 8 ? 2 : S == 4 ? 1 : 0;
-      return {(16 * x << (levels - e)) % den, den};
-    }
-  }
-  const int64_t den = 16 * M;
-  switch (q) {
-    case 0: return {128 * x % den, den};
-    case 1: return {64 * x % den, den};
-    case 2: return {32 * x % den, den};
-    case 3: return {(32 * x + 2 * M) % den, den};
-    default: return {(16 * x + (q - 4) * M) % den, den};
+    case 3: return dft_pair_turn(16, i >> 4, i & 15, 256);
+    case 4: return dft_pair_turn(R, i >> 8, i & 255, g.F);
+    default: return dft_pair_turn(S, i / g.F, i % g.F, H);
   }
 }
 
@@ -205,16 +203,14 @@ struct MultiArgs {
 size_t multi_scratch_bytes(int sms);
 cudaError_t launch_correlate_multi(const PlanDev& p, const MultiArgs& a, cudaStream_t s);
 
-// Per-S launchers (one translation unit each); halfz: Lp <= F.
-cudaError_t launch_correlate_s1(const PlanDev& p, const CorrelateArgs& a, CorrConfig c, bool halfz,
+// Per-S launchers (one translation unit each).
+cudaError_t launch_correlate_s1(const PlanDev& p, const CorrelateArgs& a, cudaStream_t s);
+cudaError_t launch_correlate_s2(const PlanDev& p, const CorrelateArgs& a, cudaStream_t s);
+cudaError_t launch_correlate_s4(const PlanDev& p, const CorrelateArgs& a, CorrConfig c,
                                 cudaStream_t s);
-cudaError_t launch_correlate_s2(const PlanDev& p, const CorrelateArgs& a, CorrConfig c, bool halfz,
+cudaError_t launch_correlate_s8(const PlanDev& p, const CorrelateArgs& a, CorrConfig c,
                                 cudaStream_t s);
-cudaError_t launch_correlate_s4(const PlanDev& p, const CorrelateArgs& a, CorrConfig c, bool halfz,
-                                cudaStream_t s);
-cudaError_t launch_correlate_s8(const PlanDev& p, const CorrelateArgs& a, CorrConfig c, bool halfz,
-                                cudaStream_t s);
-cudaError_t launch_correlate_s16(const PlanDev& p, const CorrelateArgs& a, CorrConfig c, bool halfz,
+cudaError_t launch_correlate_s16(const PlanDev& p, const CorrelateArgs& a, CorrConfig c,
                                  cudaStream_t s);
 
 // Precision form: S2-S6 with the column FFTs on tcgen05 tensor cores.

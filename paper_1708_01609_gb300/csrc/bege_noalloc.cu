@@ -42,12 +42,12 @@ constexpr size_t kOffWR0S = kOffWH + al256(256 * 8 * sizeof(float2));
 constexpr size_t kOffWS = kOffWR0S + al256(256 * 8 * sizeof(float2));
 constexpr size_t kOffWN = kOffWS + al256(8 * sizeof(float2));
 constexpr size_t kOffUnit = kOffWN + al256(kMaxH * sizeof(float2));
-constexpr size_t unit_tables(int S, int upto) {
+constexpr size_t unit_tables(const UnitGeo& g, int upto) {
   size_t n = 0;
-  for (int t = 0; t < upto; ++t) n += unit_table_size(S, t);
+  for (int t = 0; t < upto; ++t) n += unit_table_size(g, t);
   return n;
 }
-constexpr size_t kScratchBytes = kOffUnit + al256(unit_tables(8, kUnitTables) * sizeof(float2));
+constexpr size_t kScratchBytes = kOffUnit + al256(unit_tables(UnitGeo{4096, 8, 16, 256}, kUnitTables) * sizeof(float2));
 
 static __device__ __align__(256) unsigned char g_search_scratch[kScratchBytes];
 
@@ -65,7 +65,8 @@ __global__ void search_tables_kernel(Geometry g, float2* tw2, float2* tw3, float
   const int64_t n_tw2 = 16 * g.R0, n_tw3 = g.F, n_wH = 256 * (int64_t)g.S,
                 n_wR0S = (int64_t)g.R0 * g.S, n_wS = g.S, n_wN = g.H;
   int64_t total = n_tw2 + n_tw3 + n_wH + n_wR0S + n_wS + n_wN;
-  for (int t = 0; t < kUnitTables; ++t) total += unit_table_size(g.S, t);
+  const UnitGeo ug = unit_geo(g);
+  for (int t = 0; t < kUnitTables; ++t) total += unit_table_size(ug, t);
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total;
        i += (int64_t)gridDim.x * blockDim.x) {
     int64_t j = i;
@@ -102,8 +103,8 @@ __global__ void search_tables_kernel(Geometry g, float2* tw2, float2* tw3, float
     j -= n_wN;
     const int64_t at = j;
     int t = 0;
-    while (j >= unit_table_size(g.S, t)) j -= unit_table_size(g.S, t++);
-    const Turn a = unit_table_turn(g.S, t, (int)j);
+    while (j >= unit_table_size(ug, t)) j -= unit_table_size(ug, t++);
+    const Turn a = unit_table_turn(ug, t, (int)j);
     double s, c;
     sincospi(2.0 * (double)a.num / (double)a.den, &s, &c);
     unit[at] = rot_entry(c, s);
@@ -173,7 +174,7 @@ extern "C" int bege_search_noalloc(const float* strain_dev, int64_t n, const flo
     p.wN = reinterpret_cast<const float2*>(base + kOffWN);
     float2* const unit = reinterpret_cast<float2*>(base + kOffUnit);
     const float2** const tables[kUnitTables] = {&p.t1, &p.t2, &p.t3, &p.u2, &p.u1, &p.uc};
-    for (int t = 0; t < kUnitTables; ++t) *tables[t] = unit + unit_tables(g.S, t);
+    for (int t = 0; t < kUnitTables; ++t) *tables[t] = unit + unit_tables(unit_geo(g), t);
     // The tables are rebuilt on every call, in stream order before this
     // call's kernels: the host keeps no record of which n the array holds,
     // which could disagree with the device's order of work.

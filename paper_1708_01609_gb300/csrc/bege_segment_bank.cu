@@ -73,13 +73,12 @@ cudaError_t launch_correlate(const PlanDev& p, const CorrelateArgs& a, CorrConfi
   if (a.k1 <= a.k0) return cudaSuccess;
   const Geometry& g = p.g;
   if (!config_valid(g, cfg)) return cudaErrorInvalidValue;
-  const bool halfz = (g.F == 4096) && (a.Lp <= g.F);
   switch (g.S) {
-    case 1: return launch_correlate_s1(p, a, cfg, halfz, s);
-    case 2: return launch_correlate_s2(p, a, cfg, halfz, s);
-    case 4: return launch_correlate_s4(p, a, cfg, halfz, s);
-    case 8: return launch_correlate_s8(p, a, cfg, halfz, s);
-    case 16: return launch_correlate_s16(p, a, cfg, halfz, s);
+    case 1: return launch_correlate_s1(p, a, s);
+    case 2: return launch_correlate_s2(p, a, s);
+    case 4: return launch_correlate_s4(p, a, cfg, s);
+    case 8: return launch_correlate_s8(p, a, cfg, s);
+    case 16: return launch_correlate_s16(p, a, cfg, s);
     default: return cudaErrorInvalidValue;
   }
 }

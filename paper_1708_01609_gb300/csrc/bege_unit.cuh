@@ -1,16 +1,18 @@
-// The correlation for N >= 2^14 (S >= 2 columns of F = 4096 points): per-stage
-// functions of one unit (two columns, 256 threads) shared by the single,
-// block and batch kernels, and the single-segment kernel itself.
+// The correlation: per-stage functions of one unit (two columns of F points,
+// F / 16 threads) shared by the single, block and batch kernels, and the
+// single-segment kernels themselves.  N >= 2^14 has S = N / 8192 columns of F =
+// 4096 points; shorter segments have S = 2 columns of F = N / 4 = 256 .. 2048.
 //
-// Stages.  With the column split of bege_corr.cuh, j = S a + b, write
-// a = k0 + 16 k1 + 256 k2 and m = n0 + 16 n1 + 256 n2.  Forward (z -> Z):
-//   1  over n2 -> k0   twiddle base (S k0' + b) 256 / H with k0' = 0: b / (16 S)
-//   2  over n1 -> k1   base (S k0 + b) / (256 S)
-//   3  over n0 -> k2   base (S (k0 + 16 k1) + b) / H
-// inverse (Y -> rho), n = n0 + 16 n1 + 256 n2 + 4096 n3:
+// Stages.  With the column split of bege_corr.cuh, j = S a + b, and R = F /
+// 256, write a = k0 + R k1 + 16 R k2 and m = n0 + 16 n1 + 256 n2 (k0, n2 < R,
+// the others < 16).  Forward (z -> Z):
+//   1  over n2 -> k0   twiddle base b / (R S)
+//   2  over n1 -> k1   base (S k0 + b) / (16 R S)
+//   3  over n0 -> k2   base (S (k0 + R k1) + b) / H
+// inverse (Y -> rho), n = n0 + 16 n1 + 256 n2 + F n3:
 //   3' over k2 -> n0   no twiddle
 //   2' over k1 -> n1   base n0 / 256
-//   1' over k0 -> n2   base (n0 + 16 n1) / 4096
+//   1' over k0 -> n2   base (n0 + 16 n1) / F
 //   c  over b  -> n3   base (n0 + 16 n1 + 256 n2) / H
 // (bases in turns; input r of a stage is turned by r times its base).  Each
 // stage is a decimation-in-time DFT whose input twiddles are w^r for one base
@@ -27,11 +29,11 @@
 // spectrum sits digit-reversed in shared memory, the product reads its
 // coefficients in the same order (coef_pos), and one ordering point between
 // stages is enough.  Stages 2, 3, 3', 2' exchange values only between
-// threads of the same k0; warp w of a unit holds k0 = w and 15 - w (a column
+// threads of the same k0; warp w of a unit holds k0 = w and R - 1 - w (a column
 // bin's mirror has every digit complemented), so between them a warp waits
 // for itself only and the warps drift: the loads of one overlap the
 // arithmetic of another.  Unit 0 (columns 0 and S/2, each its own mirror)
-// pairs k0 with 16 - k0 in column 0 and takes a barrier there.
+// pairs k0 with R - k0 in column 0 and hands over between warps there.
 //
 // Rows.  Block k0 (256 rows, 288 16-byte slots) of a unit holds its two
 // columns interleaved (float4 {slot 0, slot 1}, row i at slot i) between
@@ -60,58 +62,80 @@
 namespace bege {
 namespace unit {
 
-constexpr int kF = 4096;
-constexpr int kT = 256;         // threads of a unit
+constexpr int kF = 4096;        // column length of N >= 2^14
 constexpr int kBlk = 288;       // 16-byte slots of a block of 256 rows
 
-// Shared memory of a CTA with U units (bytes).
-template <int U>
+template <int F>
+struct Geo {
+  static constexpr int R = F / 256;   // radix of stages 1 and 1', blocks of a unit
+  static constexpr int T = F / 16;    // threads of a unit
+  static constexpr int W = T < 32 ? 1 : T / 32;
+  static constexpr int P = R / 2;     // pairs of an R-point DFT
+  static_assert(F == 256 || F == 512 || F == 1024 || F == 2048 || F == 4096, "column length");
+};
+
+// Shared memory of a CTA with U units (bytes).  ONE: every unit is the only
+// one of a template (S = 2), so they share all tables.
+template <int F, int U, bool ONE>
 struct Lay {
-  static constexpr size_t u1 = 0;                        // [8][256] float2: stage 1'
-  static constexpr size_t u2 = u1 + 8 * 256 * 8;         // [8][16] float2: stage 2'
+  using G = Geo<F>;
+  static constexpr size_t n3 = 8 * G::T * 8, n2 = 8 * G::R * 16, n1 = (G::P + 1) / 2 * 32;
+  static constexpr size_t u1 = 0;                        // [P][256] float2: stage 1'
+  static constexpr size_t u2 = u1 + G::P * 256 * 8;      // [8][16] float2: stage 2'
   static constexpr size_t ws = u2 + 8 * 16 * 8;          // [16] float2: w_S^q (folded templates)
   static constexpr size_t rowptr = ws + 16 * 8;          // [8] the units' rows in the cluster
   static constexpr size_t sigall = rowptr + 8 * 8;       // [8] units' shares of sum |Y|^2
-  static constexpr size_t units = sigall + 8 * 4;
+  static constexpr size_t red = sigall + 8 * 4;          // [U][W] warp sums
+  static constexpr size_t one = align16(red + U * G::W * 4);
+  static constexpr size_t units = one + (ONE ? n3 + n2 + n1 : 0);
   // within a unit
-  static constexpr size_t rows = 0;                      // 16 blocks
-  static constexpr size_t t3 = rows + 16 * kBlk * 16;    // [8][256] float2: stage 3
-  static constexpr size_t t2 = t3 + 8 * 256 * 8;         // [8][16] float4: stage 2, both columns
-  static constexpr size_t t1 = t2 + 8 * 16 * 16;         // [8] float4: stage 1, both columns
-  static constexpr size_t red = t1 + 8 * 16;             // [8] warp sums
-  static constexpr size_t unit_bytes = red + 8 * 4;
+  static constexpr size_t rows = 0;                      // R blocks
+  static constexpr size_t tab = rows + G::R * kBlk * 16; // its tables (ONE: at `one`)
+  static constexpr size_t unit_bytes = tab + (ONE ? 0 : n3 + n2 + n1);
   static constexpr size_t total = units + U * unit_bytes;
+  // tables: [8][T] float2: stage 3; [8][R] float4: stage 2, both columns;
+  // [P] float4: stage 1, both columns
   static_assert(units % 16 == 0 && unit_bytes % 16 == 0, "16-byte rows");
 };
 
-template <int U>
+template <int F, int U, bool ONE = false>
 struct Sm {
-  using L = Lay<U>;
+  using L = Lay<F, U, ONE>;
+  using G = Geo<F>;
   static __device__ __forceinline__ unsigned char* unit(int ui) {
     return smem_raw + L::units + (U == 1 ? 0 : ui * L::unit_bytes);
   }
+  static __device__ __forceinline__ unsigned char* tab(int ui) {
+    return ONE ? smem_raw + L::one : unit(ui) + L::tab;
+  }
   static __device__ __forceinline__ float4* rows(int ui) { return reinterpret_cast<float4*>(unit(ui) + L::rows); }
-  static __device__ __forceinline__ float2* t3(int ui) { return reinterpret_cast<float2*>(unit(ui) + L::t3); }
-  static __device__ __forceinline__ float4* t2(int ui) { return reinterpret_cast<float4*>(unit(ui) + L::t2); }
-  static __device__ __forceinline__ float4* t1(int ui) { return reinterpret_cast<float4*>(unit(ui) + L::t1); }
-  static __device__ __forceinline__ float* red(int ui) { return reinterpret_cast<float*>(unit(ui) + L::red); }
+  static __device__ __forceinline__ float2* t3(int ui) { return reinterpret_cast<float2*>(tab(ui)); }
+  static __device__ __forceinline__ float4* t2(int ui) { return reinterpret_cast<float4*>(tab(ui) + L::n3); }
+  static __device__ __forceinline__ float4* t1(int ui) { return reinterpret_cast<float4*>(tab(ui) + L::n3 + L::n2); }
+  static __device__ __forceinline__ float* red(int ui) { return reinterpret_cast<float*>(smem_raw + L::red) + ui * G::W; }
   static __device__ __forceinline__ float2* u1() { return reinterpret_cast<float2*>(smem_raw + L::u1); }
   static __device__ __forceinline__ float2* u2() { return reinterpret_cast<float2*>(smem_raw + L::u2); }
   static __device__ __forceinline__ float2* ws() { return reinterpret_cast<float2*>(smem_raw + L::ws); }
   static __device__ __forceinline__ float4** rowptr() { return reinterpret_cast<float4**>(smem_raw + L::rowptr); }
   static __device__ __forceinline__ float* sigall() { return reinterpret_cast<float*>(smem_raw + L::sigall); }
+  static __device__ __forceinline__ int tid() { return threadIdx.x & (G::T - 1); }
+  // the block k0 that this thread works on in stages 2 and 2', and its n0
+  static __device__ __forceinline__ int k0() {
+    if constexpr (G::R == 1) return 0;
+    const int w = tid() >> 5;
+    return (threadIdx.x & 16) ? G::R - 1 - w : w;
+  }
+  static __device__ __forceinline__ int n0() { return threadIdx.x & 15; }
+  // all threads of the unit
+  static __device__ __forceinline__ void sync(int ui) {
+    if constexpr (G::T <= 32)
+      __syncwarp();
+    else if constexpr (U == 1)
+      __syncthreads();
+    else
+      asm volatile("bar.sync %0, %1;" ::"r"(ui + 1), "n"(G::T) : "memory");
+  }
 };
-
-__device__ __forceinline__ int unit_tid() { return threadIdx.x & (kT - 1); }
-
-// All threads of the unit (barrier 0 where the CTA is one unit).
-template <int U>
-__device__ __forceinline__ void unit_sync(int ui) {
-  if constexpr (U == 1)
-    __syncthreads();
-  else
-    asm volatile("bar.sync %0, %1;" ::"r"(ui + 1), "n"(kT) : "memory");
-}
 
 __device__ __forceinline__ void cluster_arrive_relaxed() {
   asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
@@ -192,75 +216,57 @@ __device__ __forceinline__ void dft16x2(float2 (&a)[16], float2 (&b)[16], W w) {
   }
 }
 
-// S-point DFT (S = 2 .. 16) of one row, pairs w(q): the last entries of the
-// 16-point set, i.e. S = 8: {4 x base, 2 x, base, base + 1/8}, S = 4: {2 x,
-// base}, S = 2: {base}.
+// S-point DFT (S = 2 .. 16) of one row.  Level l (of log2 S) of the pairs w(q)
+// holds (S / 2^(l+1)) x base + i / 2^(l+1) turns for i < max(1, 2^(l-1)), the
+// levels one after the other: S/2 pairs.
 template <int S, bool INV, class W>
 __device__ __forceinline__ void dft_row(float2 (&x)[S], W w) {
   int q = 0;
-  if constexpr (S == 16) {
-    const float2 s = w(0);
 #pragma unroll
-    for (int r = 0; r < 8; ++r) bfly<INV, 0>(x[r], x[r + 8], s.x, s.y);
-    q = 1;
-  }
-  if constexpr (S >= 8) {
-    const float2 s = w(q);
+  for (int half = S / 2; half >= 1; half >>= 1) {
+    const int groups = S / 2 / half;           // 2^l groups of 2 half inputs
+    const int n = groups > 1 ? groups / 2 : 1; // distinct pairs; the others are turned by 1/4
 #pragma unroll
-    for (int o = 0; o < S; o += 16)
+    for (int i = 0; i < n; ++i) {
+      const float2 s = w(q + i);
+      // group index: the bits of i reversed in front, the 1/4-turn bit last
+      int g = 0;
 #pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        bfly<INV, 0>(x[o + r], x[o + r + 4], s.x, s.y);
-        if constexpr (S == 16) bfly<INV, 1>(x[8 + r], x[12 + r], s.x, s.y);
-      }
-    ++q;
-  }
-  if constexpr (S >= 4) {
-    constexpr int P = S == 16 ? 2 : 1;  // distinct twiddles of this level
+      for (int b = 1; b < n; b <<= 1) g = 2 * g + ((i & b) ? 1 : 0);
+      const int o = groups > 1 ? 4 * half * g : 0;
 #pragma unroll
-    for (int p = 0; p < P; ++p) {
-      const float2 s = w(q + p);
-#pragma unroll
-      for (int r = 0; r < 2; ++r) {
-        bfly<INV, 0>(x[8 * p + r], x[8 * p + r + 2], s.x, s.y);
-        if constexpr (S >= 8) bfly<INV, 1>(x[8 * p + 4 + r], x[8 * p + 4 + r + 2], s.x, s.y);
+      for (int r = 0; r < half; ++r) {
+        bfly<INV, 0>(x[o + r], x[o + r + half], s.x, s.y);
+        if (groups > 1) bfly<INV, 1>(x[o + 2 * half + r], x[o + 3 * half + r], s.x, s.y);
       }
     }
-    q += P;
-  }
-  constexpr int P = S >= 8 ? S / 4 : 1;
-#pragma unroll
-  for (int i = 0; i < P; ++i) {
-    const float2 s = w(q + i);
-    const int o = S == 16 ? 8 * (i & 1) + 4 * (i >> 1) : 4 * i;
-    bfly<INV, 0>(x[o], x[o + 1], s.x, s.y);
-    if constexpr (S >= 4) bfly<INV, 1>(x[o + 2], x[o + 3], s.x, s.y);
+    q += n;
   }
 }
 
 // ---------------------------------------------------------------------------
 // Set-up
 // ---------------------------------------------------------------------------
-template <int U>
+template <class SM, int THREADS>
 __device__ __forceinline__ void setup_common(const PlanDev& p) {
-  using SM = Sm<U>;
-  for (int i = threadIdx.x; i < 8 * 256; i += kT * U) SM::u1()[i] = p.u1[i];
-  for (int i = threadIdx.x; i < 8 * 16; i += kT * U) SM::u2()[i] = p.u2[i];
+  for (int i = threadIdx.x; i < SM::G::P * 256; i += THREADS) SM::u1()[i] = p.u1[i];
+  for (int i = threadIdx.x; i < 8 * 16; i += THREADS) SM::u2()[i] = p.u2[i];
 }
 
-// Tables of unit ug (columns ug and S - ug; unit 0: 0 and S/2) in slot ui.
-template <int U>
+// Tables of unit ug (columns ug and S - ug; unit 0: 0 and S/2) in slot ui, by
+// its threads.
+template <class SM>
 __device__ __forceinline__ void setup_unit(const PlanDev& p, int S, int ug, int ui) {
-  using SM = Sm<U>;
-  const int t = unit_tid();
+  using G = typename SM::G;
+  const int t = SM::tid();
   const int ba = ug, bb = ug == 0 ? S / 2 : S - ug;
-  for (int i = t; i < 8 * 256; i += kT) SM::t3(ui)[i] = p.t3[ug * 2048 + i];
-  if (t < 128) {
-    const float2 a = p.t2[ba * 128 + t], b = p.t2[bb * 128 + t];
-    SM::t2(ui)[t] = make_float4(a.x, a.y, b.x, b.y);
+  for (int i = t; i < 8 * G::T; i += G::T) SM::t3(ui)[i] = p.t3[ug * 8 * G::T + i];
+  for (int i = t; i < 8 * G::R; i += G::T) {
+    const float2 a = p.t2[ba * 8 * G::R + i], b = p.t2[bb * 8 * G::R + i];
+    SM::t2(ui)[i] = make_float4(a.x, a.y, b.x, b.y);
   }
-  if (t < 8) {
-    const float2 a = p.t1[ba * 8 + t], b = p.t1[bb * 8 + t];
+  if (t < G::P) {
+    const float2 a = p.t1[ba * G::P + t], b = p.t1[bb * G::P + t];
     SM::t1(ui)[t] = make_float4(a.x, a.y, b.x, b.y);
   }
   if (ui == 0 && t < 16) SM::ws()[t] = t < S ? p.wS[t] : make_float2(1.f, 0.f);
@@ -269,57 +275,82 @@ __device__ __forceinline__ void setup_unit(const PlanDev& p, int S, int ug, int 
 // ---------------------------------------------------------------------------
 // Stages
 // ---------------------------------------------------------------------------
-// Stage 1 from the template's nz complex samples z (upper half of the columns
-// zero with HALFZ; otherwise folded over nfold multiples of F).  WAIT: the
-// cluster's reads of the previous contents of the rows are awaited after the
-// loads and the arithmetic, before the stores.
-template <int U, bool HALFZ, bool WAIT>
+// Writes the outputs of an R-point stage over n2 / k0: butterfly i of a thread
+// holds rows tid + T i + 256 r, output k at v[i][rev<R>(k)].
+template <class SM>
+__device__ __forceinline__ void store_blocks(int ui, const float2 (&va)[16 / SM::G::R][SM::G::R],
+                                             const float2 (&vb)[16 / SM::G::R][SM::G::R]) {
+  constexpr int R = SM::G::R, T = SM::G::T;
+  float4* row = SM::rows(ui) + SM::tid();
+#pragma unroll
+  for (int i = 0; i < 16 / R; ++i)
+#pragma unroll
+    for (int k = 0; k < R; ++k)
+      row[k * kBlk + T * i] = make_float4(va[i][rev<R>(k)].x, va[i][rev<R>(k)].y,
+                                          vb[i][rev<R>(k)].x, vb[i][rev<R>(k)].y);
+}
+
+// Stage 1 from the template's nz complex samples z.  HALFZ: the upper half of
+// the columns is zero (nz <= F / 2).  ONE: two columns (S = 2) and nz <= 2 F.
+// Otherwise folded over nfold multiples of F.  WAIT: the cluster's reads of the
+// previous contents of the rows are awaited after the loads and the
+// arithmetic, before the stores.
+template <class SM, bool HALFZ, bool ONE, bool WAIT>
 __device__ __forceinline__ void stage1(int ui, int S, int ug, const float* __restrict__ src,
                                        int nz, int nfold) {
-  using SM = Sm<U>;
+  constexpr int R = SM::G::R, T = SM::G::T, F = 256 * R;
   const float2* z = reinterpret_cast<const float2*>(src);
-  const int j = unit_tid();
-  float2 va[16], vb[16];
-  if constexpr (HALFZ) {
+  const int t = SM::tid();
+  auto load = [&](int m) { return m < nz ? __ldg(z + m) : make_float2(0.f, 0.f); };
+  float2 va[16 / R][R], vb[16 / R][R];
 #pragma unroll
-    for (int r = 0; r < 8; ++r) {
-      const int m = j + 256 * r;
-      va[r] = vb[r] = m < nz ? __ldg(z + m) : make_float2(0.f, 0.f);
-    }
-  } else {
+  for (int i = 0; i < 16 / R; ++i)
 #pragma unroll
-    for (int r = 0; r < 16; ++r) {
-      const int m = j + 256 * r;
-      va[r] = vb[r] = m < nz ? __ldg(z + m) : make_float2(0.f, 0.f);
+    for (int r = 0; r < (HALFZ ? R / 2 : R); ++r) {
+      const int m = t + T * i + 256 * r;
+      const float2 x = load(m);
+      if constexpr (ONE && !HALFZ) {
+        const float2 y = load(m + F);
+        va[i][r] = cadd(x, y);
+        vb[i][r] = csub(x, y);
+      } else {
+        va[i][r] = vb[i][r] = x;
+      }
     }
+  if constexpr (!HALFZ && !ONE) {
     const int bb = ug == 0 ? S / 2 : S - ug;
 #pragma unroll 1
     for (int f = 1; f < nfold; ++f) {
       const float2 wa = SM::ws()[(ug * f) & (S - 1)], wb = SM::ws()[(bb * f) & (S - 1)];
 #pragma unroll
-      for (int r = 0; r < 16; ++r) {
-        const int m = j + 256 * r + kF * f;
-        const float2 x = m < nz ? __ldg(z + m) : make_float2(0.f, 0.f);
-        va[r] = cadd(va[r], cmul(x, wa));
-        vb[r] = cadd(vb[r], cmul(x, wb));
-      }
+      for (int i = 0; i < 16 / R; ++i)
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          const float2 x = load(t + T * i + 256 * r + F * f);
+          va[i][r] = cadd(va[i][r], cmul(x, wa));
+          vb[i][r] = cadd(vb[i][r], cmul(x, wb));
+        }
     }
   }
   const float4* w = SM::t1(ui);
-  dft16x2<false, HALFZ>(va, vb, [&](int q) { return w[q]; });
-  if constexpr (WAIT) cluster_wait();
-  float4* row = SM::rows(ui) + j;
+  if constexpr (R == 16) {
+    dft16x2<false, HALFZ>(va[0], vb[0], [&](int q) { return w[q]; });
+  } else {
+    static_assert(!HALFZ || R == 16, "half-zero columns of 4096 points only");
 #pragma unroll
-  for (int k = 0; k < 16; ++k) row[k * kBlk] = make_float4(va[rev<16>(k)].x, va[rev<16>(k)].y,
-                                                          vb[rev<16>(k)].x, vb[rev<16>(k)].y);
+    for (int i = 0; i < 16 / R; ++i) {
+      dft_row<R, false>(va[i], [&](int q) { return make_float2(w[q].x, w[q].y); });
+      dft_row<R, false>(vb[i], [&](int q) { return make_float2(w[q].z, w[q].w); });
+    }
+  }
+  if constexpr (WAIT) cluster_wait();
+  store_blocks<SM>(ui, va, vb);
 }
 
 // Stage 2: rows n0 + 16 n1 of block k0, interleaved in, separate out.
-template <int U>
+template <class SM>
 __device__ __forceinline__ void stage2(int ui) {
-  using SM = Sm<U>;
-  const int lane = threadIdx.x & 31, w8 = unit_tid() >> 5;
-  const int k0 = lane < 16 ? w8 : 15 - w8, n0 = lane & 15;
+  const int k0 = SM::k0(), n0 = SM::n0();
   float4* blk = SM::rows(ui) + k0 * kBlk;
   float2 va[16], vb[16];
 #pragma unroll
@@ -329,7 +360,7 @@ __device__ __forceinline__ void stage2(int ui) {
     vb[r] = make_float2(v.z, v.w);
   }
   const float4* w = SM::t2(ui) + k0;
-  dft16x2<false, false>(va, vb, [&](int q) { return w[16 * q]; });
+  dft16x2<false, false>(va, vb, [&](int q) { return w[SM::G::R * q]; });
   __syncwarp();
   float2* c = reinterpret_cast<float2*>(blk) + n0;
 #pragma unroll
@@ -344,27 +375,28 @@ __device__ __forceinline__ void stage2(int ui) {
 struct MidItem {
   int sa, sb, k0, k1, k0b, k1b;
 };
+template <int R>
 __device__ __forceinline__ MidItem mid_item(bool unit0, int t) {
   MidItem m;
-  const int l = t & 15, w8 = t >> 5;
+  const int l = t & 15, w = t >> 5;
   if (!unit0) {
     m.sa = 0; m.sb = 1;
-    m.k0 = (t & 16) ? 15 - w8 : w8; m.k1 = l;
-    m.k0b = 15 - m.k0; m.k1b = 15 - l;
-  } else if (t & 16) {
+    m.k0 = (t & 16) ? R - 1 - w : w; m.k1 = l;
+    m.k0b = R - 1 - m.k0; m.k1b = 15 - l;
+  } else if (R == 1 ? l >= 8 : (t & 16) != 0) {  // column S/2
     m.sa = m.sb = 1;
-    m.k0 = w8; m.k1 = l;
-    m.k0b = 15 - w8; m.k1b = 15 - l;
+    m.k0 = w; m.k1 = R == 1 ? l - 8 : l;
+    m.k0b = R - 1 - w; m.k1b = 15 - m.k1;
   } else {
     m.sa = m.sb = 0;
-    if (w8 > 0) {
-      m.k0 = w8; m.k1 = l;
-      m.k0b = 16 - w8; m.k1b = 15 - l;
+    if (w > 0) {
+      m.k0 = w; m.k1 = l;
+      m.k0b = R - w; m.k1b = 15 - l;
     } else if (l < 8) {
       m.k0 = m.k0b = 0;
       m.k1 = l; m.k1b = l == 0 ? 8 : 16 - l;
     } else {
-      m.k0 = m.k0b = 8;
+      m.k0 = m.k0b = R / 2;
       m.k1 = l - 8; m.k1b = 15 - m.k1;
     }
   }
@@ -387,14 +419,14 @@ __device__ __forceinline__ float4 ld_coef(const float4* p) {
 // set of twiddles).  MULTI: the spectrum is kept in `scratch` (32 values a
 // thread, stride kT) for the block's other segments, or with `reload` read
 // from there.  AHEAD: pairs of rows whose coefficients are loaded ahead.
-template <int U, int AHEAD, bool MULTI = false, bool WAIT = false>
+template <class SM, int AHEAD, bool MULTI = false, bool WAIT = false>
 __device__ __forceinline__ void middle(int ui, int ug, const float4* __restrict__ coef,
                                        float2* __restrict__ scratch = nullptr,
                                        bool reload = false) {
-  using SM = Sm<U>;
-  const int t = unit_tid();
+  constexpr int kT = SM::G::T;
+  const int t = SM::tid();
   const bool unit0 = ug == 0, self = unit0 && t == 0;
-  const MidItem m = mid_item(unit0, t);
+  const MidItem m = mid_item<SM::G::R>(unit0, t);
   float4* pa = SM::rows(ui) + m.k0 * kBlk + (m.sa * 144 + m.k1 * 9);
   float4* pb = SM::rows(ui) + m.k0b * kBlk + (m.sb * 144 + m.k1b * 9);
   const float4* ab = coef + (size_t)ug * (24 * kT) + t;
@@ -442,7 +474,7 @@ __device__ __forceinline__ void middle(int ui, int ug, const float4* __restrict_
       }
       const float2* w = SM::t3(ui) + t;
       dft16x2<false, false>(xa, xb, [&](int q) {
-        const float2 s = w[256 * q];
+        const float2 s = w[kT * q];
         return make_float4(s.x, s.y, s.x, s.y);
       });
 #pragma unroll
@@ -508,7 +540,8 @@ __device__ __forceinline__ void middle(int ui, int ug, const float4* __restrict_
   }
   dft<16, true>(za);
   dft<16, true>(yb);
-  acc = warp_sum(acc);
+#pragma unroll
+  for (int o = kT < 32 ? 8 : 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
   if ((t & 31) == 0) SM::red(ui)[t >> 5] = acc;
   if constexpr (WAIT) cluster_wait();
 #pragma unroll
@@ -531,12 +564,12 @@ __device__ __forceinline__ void pair_sync(int id) {
 __device__ __forceinline__ void pair_arrive(int id) {
   asm volatile("bar.arrive %0, 64;" ::"r"(id) : "memory");
 }
-template <int U>
+template <class SM, int U>
 __device__ __forceinline__ void mid_enter(int ui, int ug) {
   __syncwarp();
-  if (ug != 0) return;
+  if (ug != 0 || SM::G::T <= 32) return;
   if constexpr (U > 1) {
-    unit_sync<U>(ui);
+    SM::sync(ui);
   } else {
     const int w8 = threadIdx.x >> 5;
     if (w8 < 7) pair_arrive(w8 + 1);
@@ -544,12 +577,12 @@ __device__ __forceinline__ void mid_enter(int ui, int ug) {
     if (w8 > 0) pair_sync(w8);
   }
 }
-template <int U>
+template <class SM, int U>
 __device__ __forceinline__ void mid_leave(int ui, int ug) {
   __syncwarp();
-  if (ug != 0) return;
+  if (ug != 0 || SM::G::T <= 32) return;
   if constexpr (U > 1) {
-    unit_sync<U>(ui);
+    SM::sync(ui);
   } else {
     const int w8 = threadIdx.x >> 5;
     pair_arrive(w8 == 0 ? 15 : 7 + w8);
@@ -558,11 +591,9 @@ __device__ __forceinline__ void mid_leave(int ui, int ug) {
 }
 
 // Stage 2': separate in, interleaved out.
-template <int U>
+template <class SM>
 __device__ __forceinline__ void stage2i(int ui) {
-  using SM = Sm<U>;
-  const int lane = threadIdx.x & 31, w8 = unit_tid() >> 5;
-  const int k0 = lane < 16 ? w8 : 15 - w8, n0 = lane & 15;
+  const int k0 = SM::k0(), n0 = SM::n0();
   float4* blk = SM::rows(ui) + k0 * kBlk;
   const float2* c = reinterpret_cast<const float2*>(blk) + n0;
   float2 va[16], vb[16];
@@ -583,46 +614,43 @@ __device__ __forceinline__ void stage2i(int ui) {
                                    vb[rev<16>(k)].y);
 }
 
-// Stage 1': rows j of every block, in place; outputs by n2 in natural order.
-template <int U>
-__device__ __forceinline__ void stage1i_compute(int ui, float2 (&va)[16], float2 (&vb)[16]) {
-  using SM = Sm<U>;
-  const int j = unit_tid();
-  const float4* row = SM::rows(ui) + j;
+// Stage 1': rows of every block, in place; output n2 at v[i][rev<R>(n2)] (see
+// store_blocks).
+template <class SM>
+__device__ __forceinline__ void stage1i(int ui, float2 (&va)[16 / SM::G::R][SM::G::R],
+                                        float2 (&vb)[16 / SM::G::R][SM::G::R]) {
+  constexpr int R = SM::G::R, T = SM::G::T;
+  const int t = SM::tid();
+  const float4* row = SM::rows(ui) + t;
 #pragma unroll
-  for (int r = 0; r < 16; ++r) {
-    const float4 v = row[r * kBlk];
-    va[r] = make_float2(v.x, v.y);
-    vb[r] = make_float2(v.z, v.w);
+  for (int i = 0; i < 16 / R; ++i)
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const float4 v = row[r * kBlk + T * i];
+      va[i][r] = make_float2(v.x, v.y);
+      vb[i][r] = make_float2(v.z, v.w);
+    }
+#pragma unroll
+  for (int i = 0; i < 16 / R; ++i) {
+    const float2* w = SM::u1() + t + T * i;
+    if constexpr (R == 16) {
+      dft16x2<true, false>(va[i], vb[i], [&](int q) {
+        const float2 s = w[256 * q];
+        return make_float4(s.x, s.y, s.x, s.y);
+      });
+    } else {
+      dft_row<R, true>(va[i], [&](int q) { return w[256 * q]; });
+      dft_row<R, true>(vb[i], [&](int q) { return w[256 * q]; });
+    }
   }
-  const float2* w = SM::u1() + j;
-  dft16x2<true, false>(va, vb, [&](int q) {
-    const float2 s = w[256 * q];
-    return make_float4(s.x, s.y, s.x, s.y);
-  });
-}
-template <int U>
-__device__ __forceinline__ void stage1i_store(int ui, const float2 (&va)[16],
-                                              const float2 (&vb)[16]) {
-  float4* row = Sm<U>::rows(ui) + unit_tid();
-#pragma unroll
-  for (int k = 0; k < 16; ++k)
-    row[k * kBlk] = make_float4(va[rev<16>(k)].x, va[rev<16>(k)].y, vb[rev<16>(k)].x,
-                                vb[rev<16>(k)].y);
-}
-template <int U>
-__device__ __forceinline__ void stage1i(int ui) {
-  float2 va[16], vb[16];
-  stage1i_compute<U>(ui, va, vb);
-  stage1i_store<U>(ui, va, vb);
 }
 
 // Sum |Y|^2 of a unit, in warp order (after a barrier that follows the middle).
-template <int U>
+template <class SM>
 __device__ __forceinline__ float unit_power(int ui) {
   float s = 0.f;
 #pragma unroll
-  for (int w = 0; w < 8; ++w) s += Sm<U>::red(ui)[w];
+  for (int w = 0; w < SM::G::W; ++w) s += SM::red(ui)[w];
   return s;
 }
 
@@ -641,6 +669,7 @@ template <int S, int U>
 struct Combine {
   static constexpr int C = S / 2 / U;
   static constexpr int per = kF / C;
+  static constexpr int kT = Geo<kF>::T;
   static constexpr int R = per / (kT * U);
   float2 w[R][S / 2];
 
@@ -691,31 +720,36 @@ struct Combine {
   }
 };
 
-// S = 2 (one unit, no cluster): stage 1', stage c and the tails in one go.
-// The rows reach shared memory only where some value of the warp passes.
-template <bool EXT>
-__device__ __forceinline__ void finish_s2(const float2* __restrict__ uc, float thr, uint32_t tmpl,
-                                          int64_t krow, const TailOut& a, float sigma) {
-  constexpr int S = 2;
-  const int j = unit_tid();
-  float2 va[16], vb[16];
-  stage1i_compute<1>(0, va, vb);
+// S = 2 (the unit holds the whole template): stage 1', stage c and the tails
+// in one go.  The rows reach shared memory only where some value of the warp
+// passes.
+template <class SM, bool EXT>
+__device__ __forceinline__ void finish_s2(int ui, const float2* __restrict__ uc, float thr,
+                                          uint32_t tmpl, int64_t krow, const TailOut& a,
+                                          float sigma) {
+  constexpr int S = 2, R = SM::G::R, T = SM::G::T, F = 256 * R;
+  const int t = SM::tid();
+  float2 va[16 / R][R], vb[16 / R][R];
+  stage1i<SM>(ui, va, vb);
   float big = 0.f;
 #pragma unroll
-  for (int k = 0; k < 16; ++k) {
-    const float2 s = __ldg(uc + j + 256 * k);
-    float2 &x = va[rev<16>(k)], &y = vb[rev<16>(k)];
-    bfly<true, 0>(x, y, s.x, s.y);
-    big = fmaxf(big, fmaxf(fmaxf(fabsf(x.x), fabsf(x.y)), fmaxf(fabsf(y.x), fabsf(y.y))));
-  }
-  if (a.dump || __any_sync(0xffffffffu, big > thr * (float)(S * kF))) {
-    stage1i_store<1>(0, va, vb);  // this thread's own rows
-    const float4* row = Sm<1>::rows(0) + j;
+  for (int i = 0; i < 16 / R; ++i)
+#pragma unroll
+    for (int k = 0; k < R; ++k) {
+      const float2 s = __ldg(uc + t + T * i + 256 * k);
+      float2 &x = va[i][rev<R>(k)], &y = vb[i][rev<R>(k)];
+      bfly<true, 0>(x, y, s.x, s.y);
+      big = fmaxf(big, fmaxf(fmaxf(fabsf(x.x), fabsf(x.y)), fmaxf(fabsf(y.x), fabsf(y.y))));
+    }
+  if (__any_sync(0xffffffffu, a.dump || big > thr * (float)(S * F))) {
+    store_blocks<SM>(ui, va, vb);  // this thread's own rows
+    const float4* row = SM::rows(ui) + t;
 #pragma unroll 1
-    for (int k = 0; k < 16; ++k) {
-      const float4 v = row[k * kBlk];
+    for (int q = 0; q < 16; ++q) {
+      const int i = q / R, k = q & (R - 1);
+      const float4 v = row[k * kBlk + T * i];
       float2 o[2] = {make_float2(v.x, v.y), make_float2(v.z, v.w)};
-      emit_row<S, kF, EXT>(o, j + 256 * k, S * kF, thr, tmpl, krow, a, sigma);
+      emit_row<S, F, EXT>(o, t + T * i + 256 * k, S * F, thr, tmpl, krow, a, sigma);
     }
   }
 }
@@ -724,92 +758,138 @@ __device__ __forceinline__ void finish_s2(const float2* __restrict__ uc, float t
 // S2-S6 of one segment: C = S / 2 / U CTAs of a cluster share a template
 // ---------------------------------------------------------------------------
 template <int S, int U, bool HALFZ, bool EXT>
-__global__ void __launch_bounds__(kT * U, U == 1 ? 2 : 1) unit_kernel(PlanDev p, CorrelateArgs a) {
+__global__ void __launch_bounds__(256 * U, U == 1 ? 2 : 1) unit_kernel(PlanDev p, CorrelateArgs a) {
   constexpr int C = S / 2 / U;
-  using SM = Sm<U>;
+  using SM = Sm<kF, U>;
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = C == 1 ? 0 : (int)cluster.block_rank();
-  const int ui = U == 1 ? 0 : (int)threadIdx.x / kT;
+  const int ui = U == 1 ? 0 : (int)threadIdx.x / SM::G::T;
   const int ug = rank * U + ui;
-  setup_common<U>(p);
-  setup_unit<U>(p, S, ug, ui);
-  if constexpr (C > 1) {
-    if (threadIdx.x < S / 2)
-      SM::rowptr()[threadIdx.x] = cluster.map_shared_rank(
-          SM::rows(0), (unsigned)threadIdx.x / U) + (threadIdx.x % U) * (SM::L::unit_bytes / 16);
-    cluster_arrive();  // paired with the wait of the first stage 1
-  } else if constexpr (S > 2) {
-    if (threadIdx.x < S / 2) SM::rowptr()[threadIdx.x] = SM::rows((int)threadIdx.x);
+  setup_common<SM, 256 * U>(p);
+  setup_unit<SM>(p, S, ug, ui);
+  if (threadIdx.x < S / 2) {
+    const int c = (int)threadIdx.x / U, u = (int)threadIdx.x % U;
+    float4* const rows = C == 1 ? SM::rows(0) : cluster.map_shared_rank(SM::rows(0), (unsigned)c);
+    SM::rowptr()[threadIdx.x] = rows + u * (SM::L::unit_bytes / 16);
   }
+  if constexpr (C > 1) cluster_arrive();  // paired with the wait of the first stage 1
   __syncthreads();
 
   const int cid = blockIdx.x / C, ncl = gridDim.x / C;
   const int nz = (int)(a.Lp / 2), nfold = (nz + kF - 1) / kF;
   const TailOut out{a.recs, a.cap, a.counter, a.dump, a.proj, a.kappa_hi, a.lag_end};
   for (int64_t k = a.k0 + cid; k < a.k1; k += ncl) {
-    stage1<U, HALFZ, (C > 1)>(ui, S, ug, a.bank + k * a.Lp, nz, nfold);
-    unit_sync<U>(ui);
-    stage2<U>(ui);
-    mid_enter<U>(ui, ug);
-    middle<U, (S <= 4 ? 2 : 1)>(ui, ug, a.AB);
-    mid_leave<U>(ui, ug);
-    stage2i<U>(ui);
-    unit_sync<U>(ui);
+    stage1<SM, HALFZ, false, (C > 1)>(ui, S, ug, a.bank + k * a.Lp, nz, nfold);
+    SM::sync(ui);
+    stage2<SM>(ui);
+    mid_enter<SM, U>(ui, ug);
+    middle<SM, (S <= 4 ? 2 : 1)>(ui, ug, a.AB);
+    mid_leave<SM, U>(ui, ug);
+    stage2i<SM>(ui);
+    SM::sync(ui);
     const int64_t krow = k - a.k0;
-    if constexpr (S == 2) {
-      const float share = unit_power<U>(0);
-      const float sigma = sigma_of(&share, 1, S * 2 * kF);
-      if (threadIdx.x == 0) a.sigma[krow] = sigma;
-      finish_s2<EXT>(p.uc, a.kappa * sigma, (uint32_t)k, krow, out, sigma);
-    } else {
-      stage1i<U>(ui);
-      if (unit_tid() == 0) {
-        const float share = unit_power<U>(ui);
+    {
+      float2 va[1][16], vb[1][16];
+      stage1i<SM>(ui, va, vb);
+      store_blocks<SM>(ui, va, vb);
+    }
+    if (SM::tid() == 0) {
+      const float share = unit_power<SM>(ui);
 #pragma unroll
-        for (int q = 0; q < C; ++q) {
-          if constexpr (C > 1)
-            *cluster.map_shared_rank(SM::sigall() + ug, (unsigned)q) = share;
-          else
-            SM::sigall()[ug] = share;
-        }
+      for (int q = 0; q < C; ++q) {
+        if constexpr (C > 1)
+          *cluster.map_shared_rank(SM::sigall() + ug, (unsigned)q) = share;
+        else
+          SM::sigall()[ug] = share;
       }
-      if constexpr (C > 1) cluster_arrive();
-      Combine<S, U> cb;
-      cb.twiddles(p.uc, rank);
-      if constexpr (C > 1)
-        cluster_wait();  // every row and share of the cluster is ready
-      else
-        __syncthreads();
-      const float sigma = sigma_of(SM::sigall(), S / 2, S * 2 * kF);
-      if (rank == 0 && threadIdx.x == 0) a.sigma[krow] = sigma;
-      cb.template emit<EXT>(SM::rowptr(), p.uc, rank, a.kappa * sigma, (uint32_t)k, krow, out,
-                            sigma);
-      if constexpr (C > 1) {
-        __syncwarp();
-        cluster_arrive_relaxed();  // every remote value has fed a vote: the reads are done
-      } else {
-        __syncthreads();
-      }
+    }
+    if constexpr (C > 1) cluster_arrive();
+    Combine<S, U> cb;
+    cb.twiddles(p.uc, rank);
+    if constexpr (C > 1)
+      cluster_wait();  // every row and share of the cluster is ready
+    else
+      __syncthreads();
+    const float sigma = sigma_of(SM::sigall(), S / 2, S * 2 * kF);
+    if (rank == 0 && threadIdx.x == 0) a.sigma[krow] = sigma;
+    cb.template emit<EXT>(SM::rowptr(), p.uc, rank, a.kappa * sigma, (uint32_t)k, krow, out, sigma);
+    if constexpr (C > 1) {
+      __syncwarp();
+      cluster_arrive_relaxed();  // every remote value has fed a vote: the reads are done
+    } else {
+      __syncthreads();
     }
   }
   if constexpr (C > 1) cluster_wait();  // the cluster's last reads of this CTA's rows
 }
 
+// S = 2: the units of a CTA (256 threads) take templates of their own and wait
+// for nobody else; those beyond the last template repeat the CTA's first and
+// write nothing.  Bound as above.  A unit of F / 16 threads keeps every thread
+// at work, where one column of N / 2 points per CTA of 256 threads left seven
+// eighths of them idle in the passes at N = 2^10; two units of 16 threads share
+// a warp there.  Per template (2^18 chirps of N samples at most, GB300),
+// against that kernel: N = 2^10 13.5 -> 2.3 ns, 2^11 16.5 -> 4.5, 2^12 23.6 ->
+// 9.2, 2^13 29.4 -> 19.0.
+template <int F, bool HALFZ, bool EXT>
+__global__ void __launch_bounds__(256, 2) short_kernel(PlanDev p, CorrelateArgs a) {
+  constexpr int U = 4096 / F;
+  using SM = Sm<F, U, true>;
+  const int ui = U == 1 ? 0 : (int)threadIdx.x / SM::G::T;
+  setup_common<SM, 256>(p);
+  if (ui == 0) setup_unit<SM>(p, 2, 0, 0);
+  __syncthreads();
+
+  const int nz = (int)(a.Lp / 2);
+  for (int64_t base = a.k0 + (int64_t)blockIdx.x * U; base < a.k1; base += (int64_t)gridDim.x * U) {
+    const bool active = base + ui < a.k1;
+    const int64_t k = active ? base + ui : base;
+    stage1<SM, HALFZ, true, false>(ui, 2, 0, a.bank + k * a.Lp, nz, 0);
+    SM::sync(ui);
+    stage2<SM>(ui);
+    mid_enter<SM, U>(ui, 0);
+    middle<SM, 2>(ui, 0, a.AB);
+    mid_leave<SM, U>(ui, 0);
+    stage2i<SM>(ui);
+    SM::sync(ui);
+    const int64_t krow = k - a.k0;
+    const float share = unit_power<SM>(ui);
+    const float sigma = sigma_of(&share, 1, 4 * F);
+    if (active && SM::tid() == 0) a.sigma[krow] = sigma;
+    const TailOut out{a.recs, a.cap, a.counter, active ? a.dump : nullptr, a.proj, a.kappa_hi,
+                      a.lag_end};
+    finish_s2<SM, EXT>(ui, p.uc, active ? a.kappa * sigma : INFINITY, (uint32_t)k, krow, out, sigma);
+  }
+}
+
 template <int S, int U, bool HALFZ, bool EXT>
 static cudaError_t launch_unit_t(const PlanDev& p, const CorrelateArgs& a, cudaStream_t s) {
   constexpr int C = S / 2 / U;
-  return launch_clusters(unit_kernel<S, U, HALFZ, EXT>, C, kT * U, Lay<U>::total, U == 1 ? 2 : 1,
-                         p, a, s);
+  return launch_clusters(unit_kernel<S, U, HALFZ, EXT>, C, 256 * U, Lay<kF, U, false>::total,
+                         U == 1 ? 2 : 1, 1, p, a, s);
+}
+
+// The extended epilogue (bege_correlate_max, bege_correlate_band,
+// bege_correlate_ex) runs in its own instantiation.
+static bool extended(const PlanDev& p, const CorrelateArgs& a) {
+  return a.proj || a.kappa_hi > 0.f || a.lag_end < (uint32_t)p.g.N;
 }
 
 template <int S, int U>
-static cudaError_t launch_unit(const PlanDev& p, const CorrelateArgs& a, bool halfz,
-                               cudaStream_t s) {
-  const bool ext = a.proj || a.kappa_hi > 0.f || a.lag_end < (uint32_t)p.g.N;
-  if (halfz)
-    return ext ? launch_unit_t<S, U, true, true>(p, a, s) : launch_unit_t<S, U, true, false>(p, a, s);
-  return ext ? launch_unit_t<S, U, false, true>(p, a, s)
-             : launch_unit_t<S, U, false, false>(p, a, s);
+static cudaError_t launch_unit(const PlanDev& p, const CorrelateArgs& a, cudaStream_t s) {
+  if (a.Lp <= kF)
+    return extended(p, a) ? launch_unit_t<S, U, true, true>(p, a, s)
+                          : launch_unit_t<S, U, true, false>(p, a, s);
+  return extended(p, a) ? launch_unit_t<S, U, false, true>(p, a, s)
+                        : launch_unit_t<S, U, false, false>(p, a, s);
+}
+
+template <int F, bool HALFZ>
+static cudaError_t launch_short(const PlanDev& p, const CorrelateArgs& a, cudaStream_t s) {
+  constexpr int U = 4096 / F;
+  constexpr size_t smem = Lay<F, U, true>::total;
+  return extended(p, a) ? launch_clusters(short_kernel<F, HALFZ, true>, 1, 256, smem, 2, U, p, a, s)
+                        : launch_clusters(short_kernel<F, HALFZ, false>, 1, 256, smem, 2, U, p, a, s);
 }
 
 }  // namespace unit

@@ -1,5 +1,5 @@
-"""The unit kernels (N >= 2^14) at the edges of their range: template lengths
-around the column length (one sample, odd, half a column, a column, folded
+"""The correlate kernels at the edges of their range: every segment length,
+fewer templates than a CTA has units (N <= 2^13), template lengths around the column length (one sample, odd, half a column, a column, folded
 over several), every launch shape, against the FP64 oracle; all shapes give
 the same bits, and a row gives the same bits wherever its range begins."""
 import numpy as np
@@ -20,7 +20,9 @@ def ctx():
     c.close()
 
 
-@pytest.mark.parametrize("n,length", [(1 << 14, 1), (1 << 14, 4096), (1 << 14, 4097),
+@pytest.mark.parametrize("n,length", [(1 << 10, 1), (1 << 10, 1 << 10), (1 << 11, 513),
+                                      (1 << 12, 2049), (1 << 12, 1 << 12), (1 << 13, 4095),
+                                      (1 << 13, 4097), (1 << 14, 1), (1 << 14, 4096), (1 << 14, 4097),
                                       (1 << 14, 1 << 14), (1 << 15, 2047), (1 << 15, 8193),
                                       (1 << 16, 7), (1 << 16, 4095), (1 << 16, 1 << 16),
                                       (1 << 17, 4096), (1 << 17, 12289)])
