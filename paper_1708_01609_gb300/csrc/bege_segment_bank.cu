@@ -88,58 +88,108 @@ cudaError_t launch_correlate(const PlanDev& p, const CorrelateArgs& a, CorrConfi
 // symmetric banks (Fig. 2 caption): w[m] = T(m) (sin(2 pi phase(m)) +
 // sin(2 pi phase(L - 1 - m))), the chirp forward and backward in time.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ double chirp_sin(unsigned long long alpha, unsigned long long beta,
-                                            int64_t m) {
-  const unsigned long long um = (unsigned long long)m;
-  // phase in cycles * 2^64, exact modulo one cycle
-  const unsigned long long ph = alpha * um + beta * (um * um);
-  const double c = (double)(long long)ph * 0x1p-64;  // in [-1/2, 1/2)
-  return sinpi(2.0 * c);
+// sin(2 pi phase / 2^64) at kKeep samples m0, m0 + d, m0 + 2 d, ...: the phase
+// alpha m + beta m^2 (cycles * 2^64, exact modulo one cycle) is quadratic in m,
+// so the unit phasor advances by a factor that itself advances by the constant
+// factor `turn` = exp(2 pi i 2 beta d^2); the two start values are exact
+// phases, and kKeep steps of FP64 products leave errors below 1e-14.
+constexpr int kChirpThreads = 256;
+constexpr int kKeep = 16;
+
+struct Phasor {
+  double c, s;
+};
+__device__ __forceinline__ Phasor phasor(unsigned long long cycles) {
+  Phasor p;
+  sincospi((double)(long long)cycles * 0x1p-63, &p.s, &p.c);  // half turns in [-1, 1)
+  return p;
+}
+__device__ __forceinline__ Phasor turned(Phasor a, Phasor b) {
+  return {fma(a.c, b.c, -a.s * b.s), fma(a.c, b.s, a.s * b.c)};
+}
+__device__ __forceinline__ void add_chirp(unsigned long long alpha, unsigned long long beta,
+                                          int64_t m0, int64_t d, Phasor turn, double (&v)[kKeep]) {
+  const unsigned long long m = (unsigned long long)m0, e = (unsigned long long)d;
+  Phasor p = phasor(alpha * m + beta * (m * m));
+  Phasor step = phasor(alpha * e + beta * (2 * m * e + e * e));
+#pragma unroll
+  for (int i = 0; i < kKeep; ++i) {
+    v[i] += p.s;
+    p = turned(p, step);
+    step = turned(step, turn);
+  }
 }
 
-__device__ __forceinline__ double chirp_sample(unsigned long long alpha, unsigned long long beta,
-                                               int64_t m, int64_t L, int width, double denom,
-                                               bool symmetric) {
-  double s = chirp_sin(alpha, beta, m);
-  if (symmetric) s += chirp_sin(alpha, beta, L - 1 - m);
-  const int64_t mm = m < L - 1 - m ? m : L - 1 - m;
-  double t = 1.0;
-  if (mm <= width) t = 0.5 * (1.0 - cospi(2.0 * (double)mm / denom));
-  return t * s;
+// Samples base + 256 i of thread threadIdx.x, unscaled (0 from L on).
+__device__ __forceinline__ void chirp_samples(unsigned long long alpha, unsigned long long beta,
+                                              int64_t base, int64_t L, int width, double denom,
+                                              bool symmetric, Phasor turn, double (&v)[kKeep]) {
+  const int64_t m0 = base + threadIdx.x;
+#pragma unroll
+  for (int i = 0; i < kKeep; ++i) v[i] = 0.0;
+  if (m0 >= L) return;
+  add_chirp(alpha, beta, m0, kChirpThreads, turn, v);
+  if (symmetric) add_chirp(alpha, beta, L - 1 - m0, -kChirpThreads, turn, v);
+#pragma unroll
+  for (int i = 0; i < kKeep; ++i) {
+    const int64_t m = m0 + (int64_t)kChirpThreads * i;
+    const int64_t mm = m < L - 1 - m ? m : L - 1 - m;
+    if (m >= L)
+      v[i] = 0.0;
+    else if (mm <= width)
+      v[i] *= 0.5 * (1.0 - cospi(2.0 * (double)mm / denom));
+  }
 }
 
-__global__ void __launch_bounds__(256) bank_chirp_kernel(const unsigned long long* __restrict__ ab,
-                                                         int64_t L, int64_t Lp, double frac,
-                                                         bool symmetric,
-                                                         float* __restrict__ bank) {
+// One CTA per row.  Bound: FP64 (two lanes' worth per SM and cycle).  Rows of
+// up to 4096 samples are evaluated once and kept in registers between the
+// norm and the store; a sample costs two complex products and its share of
+// the start values, about 14 FP64 instructions, where two evaluations of sinpi
+// took about 60.
+__global__ void __launch_bounds__(kChirpThreads)
+bank_chirp_kernel(const unsigned long long* __restrict__ ab, int64_t L, int64_t Lp, double frac,
+                  bool symmetric, float* __restrict__ bank) {
   __shared__ double red[8];
+  __shared__ Phasor shared_turn;
   const int64_t k = blockIdx.x;
   const unsigned long long alpha = ab[2 * k], beta = ab[2 * k + 1];
   const int width = (frac > 0.0 && L >= 2) ? (int)floor(frac * (double)(L - 1) / 2.0) : -1;
   const double denom = frac * (double)(L - 1);
+  if (threadIdx.x == 0)
+    shared_turn = phasor(beta * (2ull * kChirpThreads * kChirpThreads));
+  __syncthreads();
+  const Phasor turn = shared_turn;
+  constexpr int64_t kChunk = kChirpThreads * kKeep;
+  double v[kKeep];
   double acc = 0.0;
-  for (int64_t m = threadIdx.x; m < L; m += blockDim.x) {
-    const double v = chirp_sample(alpha, beta, m, L, width, denom, symmetric);
-    acc = fma(v, v, acc);
+  for (int64_t base = 0; base < L; base += kChunk) {
+    chirp_samples(alpha, beta, base, L, width, denom, symmetric, turn, v);
+#pragma unroll
+    for (int i = 0; i < kKeep; ++i) acc = fma(v[i], v[i], acc);
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
   __syncthreads();
   double norm = 0.0;
-  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) norm += red[w];
+  for (int w = 0; w < kChirpThreads / 32; ++w) norm += red[w];
   const double scale = norm > 0.0 ? 1.0 / sqrt(norm) : 0.0;
   float* row = bank + k * Lp;
-  for (int64_t m = threadIdx.x; m < Lp; m += blockDim.x)
-    row[m] = m < L ? (float)(chirp_sample(alpha, beta, m, L, width, denom, symmetric) * scale)
-                   : 0.f;
+  for (int64_t base = 0; base < Lp; base += kChunk) {
+    if (L > kChunk) chirp_samples(alpha, beta, base, L, width, denom, symmetric, turn, v);
+#pragma unroll
+    for (int i = 0; i < kKeep; ++i) {
+      const int64_t m = base + threadIdx.x + (int64_t)kChirpThreads * i;
+      if (m < Lp) row[m] = (float)(v[i] * scale);
+    }
+  }
 }
 
 cudaError_t launch_bank_chirp(const unsigned long long* alpha_beta, int64_t count, int64_t L,
                               int64_t Lp, double taper_frac, bool symmetric, float* bank,
                               cudaStream_t s) {
   if (count <= 0) return cudaSuccess;
-  bank_chirp_kernel<<<(unsigned)count, 256, 0, s>>>(alpha_beta, L, Lp, taper_frac, symmetric,
+  bank_chirp_kernel<<<(unsigned)count, kChirpThreads, 0, s>>>(alpha_beta, L, Lp, taper_frac, symmetric,
                                                     bank);
   return cudaGetLastError();
 }
