@@ -164,12 +164,6 @@ struct bege_ctx {
 
 namespace {
 
-// exp(-2 pi i k / M) in FP64, rounded once to FP32.
-float2 wexp(int64_t k, int64_t M) {
-  const double a = -2.0 * M_PI * (double)(k % M) / (double)M;
-  return make_float2((float)std::cos(a), (float)std::sin(a));
-}
-
 int get_plan(bege_ctx* ctx, int64_t n, std::shared_ptr<PlanHost>* out) {
   auto it = ctx->plans.find(n);
   if (it != ctx->plans.end()) {
@@ -179,66 +173,16 @@ int get_plan(bege_ctx* ctx, int64_t n, std::shared_ptr<PlanHost>* out) {
   auto p = std::make_shared<PlanHost>();
   p->g = bege::make_geometry(n);
   const bege::Geometry& g = p->g;
-  // tables: tw2 [16 R0], tw3 [F], wH [256 S], wR0S [R0 S], wS [S], wN [H]
-  const size_t n_tw2 = 16 * g.R0, n_tw3 = g.F, n_wH = 256 * g.S, n_wR0S = g.R0 * g.S,
-               n_wS = g.S, n_wN = g.H;
-  const bege::UnitGeo ug = bege::unit_geo(g);
-  size_t n_unit = 0;
-  for (int t = 0; t < bege::kUnitTables; ++t) n_unit += bege::unit_table_size(ug, t);
-  std::vector<float2> h(n_tw2 + n_tw3 + n_wH + n_wR0S + n_wS + n_wN + n_unit);
-  size_t o = 0;
-  const size_t o_tw2 = o;
-  for (int r = 0; r < 16; ++r)
-    for (int k = 0; k < g.R0; ++k) h[o + r * g.R0 + k] = wexp((int64_t)k * r, 16 * g.R0);
-  o += n_tw2;
-  const size_t o_tw3 = o;
-  const int ns3 = g.F / 16;
-  for (int r = 0; r < 16; ++r)
-    for (int k = 0; k < ns3; ++k) h[o + r * ns3 + k] = wexp((int64_t)k * r, g.F);
-  o += n_tw3;
-  const size_t o_wH = o;
-  for (size_t k = 0; k < n_wH; ++k) h[o + k] = wexp((int64_t)k, g.H);
-  o += n_wH;
-  const size_t o_wR0S = o;
-  for (size_t k = 0; k < n_wR0S; ++k) h[o + k] = wexp((int64_t)k, (int64_t)g.R0 * g.S);
-  o += n_wR0S;
-  const size_t o_wS = o;
-  for (size_t k = 0; k < n_wS; ++k) h[o + k] = wexp((int64_t)k, g.S);
-  o += n_wS;
-  const size_t o_wN = o;
-  for (size_t k = 0; k < n_wN; ++k) h[o + k] = wexp((int64_t)k, g.N);
-  o += n_wN;
-  size_t o_unit[bege::kUnitTables];
-  for (int t = 0; t < bege::kUnitTables; ++t) {
-    o_unit[t] = o;
-    for (int i = 0; i < bege::unit_table_size(ug, t); ++i, ++o) {
-      const bege::Turn a = bege::unit_table_turn(ug, t, i);
-      const double x = 2.0 * M_PI * (double)a.num / (double)a.den;
-      h[o] = bege::rot_entry(std::cos(x), std::sin(x));
-    }
-  }
-  int rc = ctx->alloc(&p->tables, h.size() * sizeof(float2));
+  int rc = ctx->alloc(&p->tables, (size_t)bege::plan_floats2(g) * sizeof(float2));
   if (rc) return rc;
-  cudaError_t e = cudaMemcpy(p->tables.ptr, h.data(), h.size() * sizeof(float2),
-                             cudaMemcpyHostToDevice);
+  float2* const base = static_cast<float2*>(p->tables.ptr);
+  cudaError_t e = bege::launch_plan_tables(g, base, nullptr);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);  // read by kernels of any stream
   if (e != cudaSuccess) {
     ctx->release(&p->tables);
     return cuda_fail(e, "plan tables");
   }
-  const float2* base = static_cast<const float2*>(p->tables.ptr);
-  p->dev.g = g;
-  p->dev.tw2 = base + o_tw2;
-  p->dev.tw3 = base + o_tw3;
-  p->dev.wH = base + o_wH;
-  p->dev.wR0S = base + o_wR0S;
-  p->dev.wS = base + o_wS;
-  p->dev.wN = base + o_wN;
-  p->dev.t1 = base + o_unit[0];
-  p->dev.t2 = base + o_unit[1];
-  p->dev.t3 = base + o_unit[2];
-  p->dev.u2 = base + o_unit[3];
-  p->dev.u1 = base + o_unit[4];
-  p->dev.uc = base + o_unit[5];
+  p->dev = bege::plan_at(g, base);
   ctx->plans[n] = p;
   *out = p;
   return BEGE_OK;

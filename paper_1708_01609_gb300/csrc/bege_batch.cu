@@ -136,12 +136,7 @@ __global__ void __launch_bounds__(kT, 2) batch_kernel(BatchArgs b) {
 __global__ void __launch_bounds__(kT, 1) segment_batch_kernel(BatchArgs b,
                                                              const SegJob* __restrict__ jobs) {
   const SegJob j = jobs[blockIdx.x];
-  switch (j.S) {
-    case 2: segment_body<kF, 2, kNC, kT>(b.plans[0], j.rank, j.y, j.D, j.AB, false); break;
-    case 4: segment_body<kF, 4, kNC, kT>(b.plans[1], j.rank, j.y, j.D, j.AB, false); break;
-    case 8: segment_body<kF, 8, kNC, kT>(b.plans[2], j.rank, j.y, j.D, j.AB, false); break;
-    default: segment_body<kF, 16, kNC, kT>(b.plans[3], j.rank, j.y, j.D, j.AB, false); break;
-  }
+  segment_unit<Sm<kF, 1>, false>(b.plans[plan_index(j.S)], j.S, j.rank, j.y, j.D, j.AB, false);
 }
 
 }  // namespace
@@ -195,7 +190,7 @@ cudaError_t launch_batch(const BatchArgs& b, int clusters, cudaStream_t s) {
 
 cudaError_t launch_segment_batch(const BatchArgs& b, const SegJob* jobs, int njobs,
                                  cudaStream_t s) {
-  constexpr size_t smem = bege::Lay<kF, kNC>::total;
+  constexpr size_t smem = unit::Lay<kF, 1, false>::total;
   cudaError_t e = cudaFuncSetAttribute(segment_batch_kernel,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;

@@ -19,7 +19,7 @@
 //     A_j = g_j^2 D_j + d_j^2 conj D_{H-j},  B_j = g_j d_j (D_j + conj D_{H-j}),
 //     g_j = (1 + i wN^-j)/2,  d_j = (1 - i wN^-j)/2,
 // where A, B depend on the segment only and are computed once per segment
-// (segment_kernel).  By Parseval on the packed spectrum
+// (segment_kernel in bege_unit.cuh).  By Parseval on the packed spectrum
 //     sigma^2 = (1/N) sum_n rho_n^2 = 2 sum_{j<H} |Y_j|^2 / N^2,
 // the same quantity as Eq. PT's sum over the spectrum of rho.
 //
@@ -36,15 +36,15 @@
 // cluster hold all S columns and read each other's columns through
 // distributed shared memory only in the final S-point combine.
 //
-// This file: the segment kernel and the tail epilogue; bege_unit.cuh has the
-// correlation.  (The segment kernel takes N <= 2^13 as one column of F = H
-// points; the correlation always has at least two columns.)
+// This file: column maps, the tail epilogue and the launch; bege_unit.cuh has
+// the segment and correlate kernels, bege_corr_tc.cu the tensor-core form.
 #pragma once
 
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
+
 
 #include "bege_fft.cuh"
 #include "bege_internal.h"
@@ -53,39 +53,9 @@ namespace bege {
 
 namespace cg = cooperative_groups;
 
-// ---------------------------------------------------------------------------
-// Shared-memory layout: compile-time offsets for (F, NC) so every access is
-// a shared-memory instruction with an immediate offset.
-// ---------------------------------------------------------------------------
 __host__ __device__ constexpr size_t align16(size_t x) { return (x + 15) & ~size_t(15); }
 
-template <int F, int NC>
-struct Lay {
-  static constexpr int CS = col_stride<F>();
-  static constexpr size_t cols = 0;
-  static constexpr size_t tw3 = cols + align16(size_t(NC) * CS * 8);
-  static constexpr size_t tw2 = tw3 + align16(size_t(F) * 8);
-  static constexpr size_t twin = tw2 + align16(256 * 8);
-  static constexpr size_t rin = twin + align16(size_t(NC) * 256 * 8);
-  static constexpr size_t ws = rin + align16(size_t(NC) * 16 * 8);
-  static constexpr size_t red = ws + align16(16 * 8);
-  static constexpr size_t total = red + align16(32 * 4);
-};
-
 extern __shared__ __align__(16) unsigned char smem_raw[];
-
-template <int F, int NC>
-struct Smem {
-  using L = Lay<F, NC>;
-  static __device__ __forceinline__ float2* cols() { return reinterpret_cast<float2*>(smem_raw + L::cols); }
-  static __device__ __forceinline__ float2* col(int c) { return cols() + c * L::CS; }
-  static __device__ __forceinline__ float2* tw3() { return reinterpret_cast<float2*>(smem_raw + L::tw3); }
-  static __device__ __forceinline__ float2* tw2() { return reinterpret_cast<float2*>(smem_raw + L::tw2); }
-  static __device__ __forceinline__ float2* twin() { return reinterpret_cast<float2*>(smem_raw + L::twin); }
-  static __device__ __forceinline__ float2* rin() { return reinterpret_cast<float2*>(smem_raw + L::rin); }
-  static __device__ __forceinline__ float2* ws() { return reinterpret_cast<float2*>(smem_raw + L::ws); }
-  static __device__ __forceinline__ float* red() { return reinterpret_cast<float*>(smem_raw + L::red); }
-};
 
 // Column ownership for S columns split over C = S/NC CTAs.
 template <int S, int NC>
@@ -117,90 +87,6 @@ struct ColMap {
     *slot = S == 1 ? 0 : 2 * (unit % UPC) + second;
   }
 };
-
-// Twiddle tables that depend on F only (the Stockham passes).
-template <int F, int NC, int T>
-__device__ void setup_common(const PlanDev& p) {
-  using SM = Smem<F, NC>;
-  for (int i = threadIdx.x; i < F; i += T) SM::tw3()[i] = p.tw3[i];
-  for (int i = threadIdx.x; i < 16 * (F / 256); i += T) SM::tw2()[i] = p.tw2[i];
-}
-
-// Column twiddles of this CTA's slots (CTA `rank` of the S/NC that share the
-// columns).
-template <int F, int S, int NC, int T>
-__device__ void setup_columns(const PlanDev& p, int rank) {
-  using SM = Smem<F, NC>;
-  const int t = threadIdx.x;
-  for (int i = t; i < NC * 256; i += T) {
-    const int c = i >> 8, j = i & 255;
-    SM::twin()[i] = p.wH[ColMap<S, NC>::slot_column(rank, c) * j];
-  }
-  for (int i = t; i < NC * 16; i += T) {
-    const int c = i >> 4, r = i & 15;
-    const int b = ColMap<S, NC>::slot_column(rank, c);
-    SM::rin()[i] = r < F / 256 ? p.wR0S[b * r] : make_float2(1.f, 0.f);
-  }
-  if (t < 16) SM::ws()[t] = t < S ? p.wS[t] : make_float2(1.f, 0.f);
-}
-
-// First forward pass (radix R0 = F/256, Ns = 1) fused with the load of
-// u_b[m1] = wH^(b m1) sum_{m2} z[m1 + F m2] wS^(b m2) from global memory.
-// src holds nz complex samples z[m] (interleaved floats).  HALFZ: nz <= F/2
-// and the upper half of every radix-16 input vector is zero.
-template <int F, int S, int NC, int T, bool HALFZ>
-__device__ __forceinline__ void fwd_first_pass(int rank, const float* __restrict__ src, int nz,
-                                               int nfold) {
-  using SM = Smem<F, NC>;
-  constexpr int R0 = F / 256;
-  constexpr int RL = HALFZ ? R0 / 2 : R0;  // inputs that can be non-zero
-  constexpr int total = NC * 256;
-  const float2* z = reinterpret_cast<const float2*>(src);
-#pragma unroll
-  for (int i = 0; i < (total + T - 1) / T; ++i) {
-    const int idx = threadIdx.x + i * T;
-    if ((total % T == 0) || idx < total) {
-      const int c = idx >> 8, j = idx & 255;
-      float2 v[R0];
-#pragma unroll
-      for (int r = 0; r < R0; ++r) {
-        const int m1 = j + r * 256;
-        float2 acc = make_float2(0.f, 0.f);
-        if (r < RL) {
-          if (m1 < nz) acc = __ldg(z + m1);
-          if (!HALFZ && nfold > 1) {
-            const int b = ColMap<S, NC>::slot_column(rank, c);
-            for (int m2 = 1; m2 < nfold; ++m2) {
-              const int m = m1 + F * m2;
-              if (m < nz) acc = cadd(acc, cmul(__ldg(z + m), SM::ws()[(b * m2) & (S - 1)]));
-            }
-          }
-        }
-        v[r] = acc;
-      }
-      if constexpr (S != 1) {
-        const float2 tj = SM::twin()[c * 256 + j];
-        const float2* rin = SM::rin() + c * 16;
-#pragma unroll
-        for (int r = 0; r < RL; ++r) v[r] = cmul(cmul(v[r], tj), rin[r]);
-      }
-      dft<R0, false, HALFZ>(v);
-      float2* col = SM::col(c) + pad(j * R0);
-#pragma unroll
-      for (int r = 0; r < R0; ++r) col[r] = v[r];  // R0 <= 16 consecutive: one pad group
-    }
-  }
-  __syncthreads();
-}
-
-template <int F, int S, int NC, int T, bool HALFZ>
-__device__ __forceinline__ void forward_columns(int rank, const float* src, int nz, int nfold) {
-  using SM = Smem<F, NC>;
-  constexpr int R0 = F / 256;
-  fwd_first_pass<F, S, NC, T, HALFZ>(rank, src, nz, nfold);
-  stockham_pass<F, NC, T, 16, R0, false>(SM::cols(), SM::tw2());
-  stockham_pass<F, NC, T, 16, 16 * R0, false>(SM::cols(), SM::tw3());
-}
 
 // The bin pairs (j, H-j) held by a unit.  Unit 0 holds column 0 (pairs
 // a <-> (F-a) mod F, with a = 0 and a = F/2 paired with themselves) and
@@ -249,141 +135,6 @@ __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
-}
-
-// ---------------------------------------------------------------------------
-// S1: segment spectrum D and product coefficients A, B (grid: C CTAs)
-// ---------------------------------------------------------------------------
-// Where the middle of bege_unit.cuh reads the coefficients of bin S a + b:
-// unit u, thread t of T = F / 16, row r, half h (the thread's butterfly or its
-// mirror, whose rows run backwards).  Since B_{H-j} = conj B_j, a mirror pair
-// keeps one B: rows 2 i, 2 i + 1 of a thread are the three float4 {A, A'} of
-// either row and {B, B}, T apart.  Thread 0 of unit 0 holds two butterflies
-// of column 0 that are their own mirrors, rows 16 R r of it and 8 R + 16 R r: the
-// first have their B at row r < 8 (row 0: the real B of r = 0 and of r = 8),
-// the others at row 8 + r.
-struct CoefPlace {
-  int a, b, bc;  // float2 index of A; of B or -1; component of a real B (else -1)
-};
-template <int F, int S>
-__host__ __device__ __forceinline__ CoefPlace coef_place(int b, int a) {
-  constexpr int R = F / 256, T = F / 16;
-  int k0 = a & (R - 1), k1 = (a / R) & 15, r = a / (16 * R);
-  int u = 0, h = 0, t;
-  if (b != 0 && b != S / 2) {
-    h = b > S / 2;
-    u = h ? S - b : b;
-    if (h) { k0 = R - 1 - k0; k1 = 15 - k1; }
-    t = (k0 < R / 2 ? 32 * k0 : 32 * (R - 1 - k0) + 16) + k1;
-  } else if (b != 0) {  // column S/2
-    h = R == 1 ? k1 >= 8 : k0 >= R / 2;
-    if (h) { k0 = R - 1 - k0; k1 = 15 - k1; }
-    t = R == 1 ? 8 + k1 : 32 * k0 + 16 + k1;
-  } else if (k0 == 0) {  // column 0: butterfly j = k0 + R k1 and 16 R - j
-    h = k1 >= 8;
-    t = k1 <= 8 ? k1 & 7 : 16 - k1;
-  } else if (k0 == R / 2) {
-    h = k1 >= 8;
-    t = 8 + (h ? 15 - k1 : k1);
-  } else {
-    h = k0 > R / 2;
-    if (h) { k0 = R - k0; k1 = 15 - k1; }
-    t = 32 * k0 + k1;
-  }
-  int br = h ? -1 : r, bc = -1;
-  if (u == 0 && t == 0) {
-    if (h) {
-      br = r < 8 ? 8 + r : -1;
-    } else {
-      br = r < 8 ? r : r == 8 ? 0 : -1;
-      bc = r == 0 ? 0 : r == 8 ? 1 : -1;
-    }
-  }
-  if (h) r = 15 - r;
-  auto at = [&](int row, int third) { return 2 * (((u * 8 + (row >> 1)) * 3 + third) * T + t); };
-  return {at(r, r & 1) + h, br < 0 ? -1 : at(br, 2) + (br & 1), bc};
-}
-// Stores {A, B} of bin j; natural (the tensor-core kernel): at b F + a for j =
-// S a + b.
-template <int F, int S>
-__device__ __forceinline__ void store_coef(float4* AB, int j, float4 ab, bool natural) {
-  if (S > 1 && natural) {
-    AB[(j % S) * F + j / S] = ab;
-    return;
-  }
-  constexpr int Fu = S == 1 ? F / 2 : F, Su = S == 1 ? 2 : S;
-  float2* c = reinterpret_cast<float2*>(AB);
-  const CoefPlace p = coef_place<Fu, Su>(j % Su, j / Su);
-  c[p.a] = make_float2(ab.x, ab.y);
-  if (p.bc >= 0)
-    reinterpret_cast<float*>(c + p.b)[p.bc] = ab.z;
-  else if (p.b >= 0)
-    c[p.b] = make_float2(ab.z, ab.w);
-}
-
-template <int F, int S, int NC, int T>
-__device__ __forceinline__ void segment_body(const PlanDev& p, int rank,
-                                             const float* __restrict__ y,
-                                             float2* __restrict__ D, float4* __restrict__ AB,
-                                             bool natural) {
-  using SM = Smem<F, NC>;
-  constexpr int UPC = ColMap<S, NC>::UPC;
-  const int H = p.g.H;
-  setup_common<F, NC, T>(p);
-  setup_columns<F, S, NC, T>(p, rank);
-  __syncthreads();
-  forward_columns<F, S, NC, T, false>(rank, y, H, S);
-
-  for (int ui = 0; ui < UPC; ++ui) {
-    const int ug = rank * UPC + ui;
-    const int count = unit_items<F, S>(ug);
-    for (int it = threadIdx.x; it < count; it += T) {
-      const PairItem q = pair_item<F, S>(ug, ui, it);
-      const float2 zj = SM::col(q.sj)[pad(q.a)];
-      const float2 zp = SM::col(q.sp)[pad(q.ap)];
-      const int j = S * q.a + q.b;
-      const int jp = S * q.ap + q.bp;
-      const bool self = (j == jp);
-      // D_j = (Zj + conj Zp)/2 - (i/2) wN^j (Zj - conj Zp)
-      const float2 wj = p.wN[j];
-      const float2 sj = cadd(zj, cconj(zp)), dj = csub(zj, cconj(zp));
-      const float2 dd = cmul(wj, dj);
-      const float2 Dj = make_float2(0.5f * (sj.x + dd.y), 0.5f * (sj.y - dd.x));
-      float2 Djp = Dj;
-      if (!self) {
-        const float2 wp = p.wN[jp];
-        const float2 sp = cadd(zp, cconj(zj)), dp = csub(zp, cconj(zj));
-        const float2 de = cmul(wp, dp);
-        Djp = make_float2(0.5f * (sp.x + de.y), 0.5f * (sp.y - de.x));
-      }
-      const float2 DH = make_float2(zj.x - zj.y, 0.f);  // D_{N/2}, used when j == 0
-      // conj D_{H-j}: for j = 0 it is the Nyquist bin, otherwise conj D_jp
-      const float2 cHj = (j == 0) ? DH : cconj(Djp);
-      const float2 cHjp = cconj(Dj);
-      auto coeffs = [](float2 w, float2 Dx, float2 cH) {
-        // g = (1 + i conj w)/2, d = (1 - i conj w)/2 with i conj(w) = (w.y, w.x)
-        const float2 gg = make_float2(0.5f * (1.f + w.y), 0.5f * w.x);
-        const float2 de = make_float2(0.5f * (1.f - w.y), -0.5f * w.x);
-        const float2 A = cadd(cmul(cmul(gg, gg), Dx), cmul(cmul(de, de), cH));
-        const float2 B = cmul(cmul(gg, de), cadd(Dx, cH));
-        return make_float4(A.x, A.y, B.x, B.y);
-      };
-      store_coef<F, S>(AB, j, coeffs(wj, Dj, cHj), natural);
-      D[j] = Dj;
-      if (!self) {
-        store_coef<F, S>(AB, jp, coeffs(p.wN[jp], Djp, cHjp), natural);
-        D[jp] = Djp;
-      }
-      if (j == 0) D[H] = DH;
-    }
-  }
-}
-
-template <int F, int S, int NC, int T>
-__global__ void __launch_bounds__(T, 1)
-segment_kernel(PlanDev p, const float* __restrict__ y, float2* __restrict__ D,
-               float4* __restrict__ AB, bool natural) {
-  segment_body<F, S, NC, T>(p, blockIdx.x, y, D, AB, natural);
 }
 
 // ---------------------------------------------------------------------------
@@ -548,17 +299,6 @@ static cudaError_t launch_clusters(K kern, int C, int threads, size_t smem, int 
   if (want > max_clusters) want = max_clusters;
   cfg.gridDim = dim3((unsigned)(want * C), 1, 1);
   return cudaLaunchKernelEx(&cfg, kern, p, a);
-}
-
-template <int F, int S, int NC, int T>
-static cudaError_t launch_segment_t(const PlanDev& p, const float* y, float2* D, float4* AB,
-                                    bool natural, cudaStream_t s) {
-  constexpr size_t smem = Lay<F, NC>::total;
-  auto kern = segment_kernel<F, S, NC, T>;
-  cudaError_t e = ensure_smem(kern, smem);
-  if (e != cudaSuccess) return e;
-  kern<<<ColMap<S, NC>::C, T, smem, s>>>(p, y, D, AB, natural);
-  return cudaGetLastError();
 }
 
 }  // namespace bege

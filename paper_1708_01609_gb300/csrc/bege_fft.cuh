@@ -1,5 +1,4 @@
-// Register-level DFT kernels and shared-memory Stockham passes for the
-// column FFTs of the correlation (Eq. 3S).  Forward kernel exp(-i ...) as in
+// Register-level DFT kernels for the column FFTs of the correlation (Eq. 3S).  Forward kernel exp(-i ...) as in
 // Eq. A2; the inverse uses exp(+i ...) without the 1/N factor.
 #pragma once
 
@@ -138,22 +137,12 @@ __device__ __forceinline__ void dft8(float2 (&x)[8]) {
 }
 
 // 16 = 4 x 4: DFT4 over the stride-4 index, twiddle w16^(n2 k1), DFT4 over
-// the offset index, then transpose to natural order.  HALFZ: inputs 8..15
-// are known to be zero (a zero-padded half), which shortens the first DFT4s.
-template <bool INV, bool HALFZ = false>
+// the offset index, then transpose to natural order.
+template <bool INV>
 __device__ __forceinline__ void dft16(float2 (&x)[16]) {
 #pragma unroll
   for (int n2 = 0; n2 < 4; ++n2) {
-    if constexpr (HALFZ) {
-      const float2 a = x[n2], b = x[n2 + 4];
-      const float2 mb = mul_mi<INV>(b);
-      x[n2] = cadd(a, b);
-      x[n2 + 8] = csub(a, b);
-      x[n2 + 4] = cadd(a, mb);
-      x[n2 + 12] = csub(a, mb);
-    } else {
-      dft4<INV>(x[n2], x[n2 + 4], x[n2 + 8], x[n2 + 12]);
-    }
+    dft4<INV>(x[n2], x[n2 + 4], x[n2 + 8], x[n2 + 12]);
   }
   // DFT4 over n2 of x[n2 + 4 k1] w16^(n2 k1), the twiddles merged into it
   dft4_tw16<INV, 0>(x[0], x[1], x[2], x[3]);
@@ -169,9 +158,8 @@ __device__ __forceinline__ void dft16(float2 (&x)[16]) {
   for (int i = 0; i < 16; ++i) x[i] = t[i];
 }
 
-template <int R, bool INV, bool HALFZ = false>
+template <int R, bool INV>
 __device__ __forceinline__ void dft(float2 (&x)[R]) {
-  static_assert(!HALFZ || R == 16, "half-zero DFT only for radix 16");
   if constexpr (R == 1) {
   } else if constexpr (R == 2) {
     dft2<INV>(x[0], x[1]);
@@ -181,75 +169,8 @@ __device__ __forceinline__ void dft(float2 (&x)[R]) {
     dft8<INV>(x);
   } else {
     static_assert(R == 16, "radix");
-    dft16<INV, HALFZ>(x);
+    dft16<INV>(x);
   }
-}
-
-// One in-place Stockham pass of radix R over NC columns of length F in
-// shared memory (column c at cols + c * col_stride<F>(), padded indexing).
-// Butterfly j reads col[j + r F/R], twiddles by w(NS R)^(k r) with
-// k = j mod NS (table tw[r*NS + k]), and writes col[(j-k) R + k + r NS].
-// Butterflies are taken in rounds of T threads; since F/R divides T every
-// round covers whole columns, so a round can load, synchronise and store
-// without touching the columns of the next round.  Each thread holds one
-// butterfly (R complex values) across a barrier: holding two (one round)
-// costs fewer barriers but spills at 128 registers and measured slower.
-// With F/R and NS multiples of 16 the padded addresses of a butterfly are
-// one base plus constants.
-template <int F, int NC, int T, int R, int NS, bool INV, bool TRAIL = true>
-__device__ __forceinline__ void stockham_pass(float2* cols, const float2* tw) {
-  constexpr int NB = F / R;
-  static_assert(T % NB == 0, "rounds must cover whole columns");
-  constexpr int total = NC * NB;
-  constexpr int rounds = (total + T - 1) / T;
-  constexpr int CS = col_stride<F>();
-#pragma unroll
-  for (int i = 0; i < rounds; ++i) {
-    const int idx = threadIdx.x + i * T;
-    const bool act = (total % T == 0) || idx < total;
-    const int c = idx / NB, j = idx - c * NB;
-    const int k = j & (NS - 1);
-    float2 v[R];
-    if (act) {
-      const float2* col = cols + c * CS;
-      if constexpr (NB % 16 == 0) {
-        const float2* p = col + pad(j);
-#pragma unroll
-        for (int r = 0; r < R; ++r) v[r] = p[r * (NB + NB / 16)];
-      } else {
-#pragma unroll
-        for (int r = 0; r < R; ++r) v[r] = col[pad(j + r * NB)];
-      }
-      if constexpr (NS > 1) {
-        const float2* t = tw + k;
-#pragma unroll
-        for (int r = 1; r < R; ++r) v[r] = INV ? cmulc(v[r], t[r * NS]) : cmul(v[r], t[r * NS]);
-      }
-      dft<R, INV>(v);
-    }
-    __syncthreads();
-    if (act) {
-      float2* col = cols + c * CS;
-      const int base = (j - k) * R + k;
-      if constexpr (NS % 16 == 0) {
-        float2* p = col + pad(base);
-#pragma unroll
-        for (int r = 0; r < R; ++r) p[r * (NS + NS / 16)] = v[r];
-      } else if constexpr (NS == 1 && R == 16) {
-        float2* p = col + pad(base);
-#pragma unroll
-        for (int r = 0; r < R; ++r) p[r] = v[r];
-      } else {
-#pragma unroll
-        for (int r = 0; r < R; ++r) col[pad(base + r * NS)] = v[r];
-      }
-    }
-  }
-  // TRAIL = false: the caller's next pass runs the same rounds over the same
-  // columns, so with two or more rounds each column's stores here and its
-  // loads there are separated by a later round's barrier (of this pass or
-  // of the next); with one round they are not, and the barrier stays
-  if constexpr (TRAIL || rounds < 2) __syncthreads();
 }
 
 }  // namespace bege

@@ -27,7 +27,6 @@ struct Geometry {
   int H;    // N / 2 complex samples
   int F;    // column FFT length (512..4096)
   int S;    // columns = H / F (1..16)
-  int R0;   // radix of the first Stockham pass = F / 256
 };
 
 // Launch shape of the correlate kernel: columns per CTA (the cluster has
@@ -38,16 +37,11 @@ struct CorrConfig {
   int threads;
 };
 
-// Device twiddle tables for one N (computed in FP64 on the host, rounded to
-// FP32 once).  wX^k means exp(-2 pi i k / X).
+// Device tables for one N (plan_tables_kernel: FP64, rounded to FP32 once).  wX^k means exp(-2 pi i k / X).
 struct PlanDev {
   Geometry g;
-  const float2* tw2;   // [16*R0]  Stockham pass 2: [r*R0 + k] = w(16 R0)^(k r)
-  const float2* tw3;   // [F]      Stockham pass 3: [r*(F/16) + k] = wF^(k r)
-  const float2* wH;    // [256*S]  wH^k
-  const float2* wR0S;  // [R0*S]   w(R0 S)^q
-  const float2* wS;    // [S]      wS^q
-  const float2* wN;    // [H]      wN^j
+  const float2* wS;    // [S of UnitGeo] wS^q
+  const float2* wN;    // [H]            wN^j
   // tables of bege_unit.cuh for its columns (UnitGeo), {cos, tan} pairs
   // (rot_entry, unit_table_turn)
   const float2* t1;    // [S][R/2]     stage 1: column b
@@ -134,6 +128,17 @@ inline __host__ __device__ float2 rot_entry(double c, double s) {
 }
 
 Geometry make_geometry(int64_t n);
+
+// The tables of geometry g in an array of plan_floats2(g) float2 at `base`,
+// and the kernel that writes them there.
+constexpr __host__ __device__ int plan_floats2(const Geometry& g) {
+  const UnitGeo u = unit_geo(g);
+  int n = u.S + g.H;
+  for (int t = 0; t < kUnitTables; ++t) n += unit_table_size(u, t);
+  return n;
+}
+PlanDev plan_at(const Geometry& g, float2* base);
+cudaError_t launch_plan_tables(const Geometry& g, float2* base, cudaStream_t s);
 
 // Record `msg` as the calling thread's last error (bege_last_error) and
 // return `code`.

@@ -20,7 +20,6 @@
 #include <mutex>
 #include <string>
 
-#include "bege_corr.cuh"
 #include "bege_internal.h"
 
 namespace bege {
@@ -35,81 +34,11 @@ constexpr size_t al256(size_t x) { return (x + 255) & ~size_t(255); }
 // Byte offsets of the regions of the scratch array (sized for N = 2^16).
 constexpr size_t kOffAB = 0;
 constexpr size_t kOffD = kOffAB + al256(kMaxH * sizeof(float4));
-constexpr size_t kOffTw2 = kOffD + al256((kMaxH + 1) * sizeof(float2));
-constexpr size_t kOffTw3 = kOffTw2 + al256(256 * sizeof(float2));
-constexpr size_t kOffWH = kOffTw3 + al256(4096 * sizeof(float2));
-constexpr size_t kOffWR0S = kOffWH + al256(256 * 8 * sizeof(float2));
-constexpr size_t kOffWS = kOffWR0S + al256(256 * 8 * sizeof(float2));
-constexpr size_t kOffWN = kOffWS + al256(8 * sizeof(float2));
-constexpr size_t kOffUnit = kOffWN + al256(kMaxH * sizeof(float2));
-constexpr size_t unit_tables(const UnitGeo& g, int upto) {
-  size_t n = 0;
-  for (int t = 0; t < upto; ++t) n += unit_table_size(g, t);
-  return n;
-}
-constexpr size_t kScratchBytes = kOffUnit + al256(unit_tables(UnitGeo{4096, 8, 16, 256}, kUnitTables) * sizeof(float2));
+constexpr size_t kOffTables = kOffD + al256((kMaxH + 1) * sizeof(float2));
+constexpr Geometry kMaxGeometry{(int)kMaxN, (int)kMaxH, 4096, (int)(kMaxH / 4096)};
+constexpr size_t kScratchBytes = kOffTables + al256(plan_floats2(kMaxGeometry) * sizeof(float2));
 
 static __device__ __align__(256) unsigned char g_search_scratch[kScratchBytes];
-
-// exp(-2 pi i k / M) from the FP64 sincospi, rounded once to FP32.
-__device__ __forceinline__ float2 unit_root(int64_t k, int64_t M) {
-  double s, c;
-  sincospi(-2.0 * (double)(k % M) / (double)M, &s, &c);
-  return make_float2((float)c, (float)s);
-}
-
-// The twiddle tables of PlanDev for geometry g, written into the scratch
-// regions (same definitions as the tables the context uploads).
-__global__ void search_tables_kernel(Geometry g, float2* tw2, float2* tw3, float2* wH,
-                                     float2* wR0S, float2* wS, float2* wN, float2* unit) {
-  const int64_t n_tw2 = 16 * g.R0, n_tw3 = g.F, n_wH = 256 * (int64_t)g.S,
-                n_wR0S = (int64_t)g.R0 * g.S, n_wS = g.S, n_wN = g.H;
-  int64_t total = n_tw2 + n_tw3 + n_wH + n_wR0S + n_wS + n_wN;
-  const UnitGeo ug = unit_geo(g);
-  for (int t = 0; t < kUnitTables; ++t) total += unit_table_size(ug, t);
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    int64_t j = i;
-    if (j < n_tw2) {
-      tw2[j] = unit_root((j % g.R0) * (j / g.R0), 16 * (int64_t)g.R0);
-      continue;
-    }
-    j -= n_tw2;
-    if (j < n_tw3) {
-      const int64_t ns = g.F / 16;
-      tw3[j] = unit_root((j % ns) * (j / ns), g.F);
-      continue;
-    }
-    j -= n_tw3;
-    if (j < n_wH) {
-      wH[j] = unit_root(j, g.H);
-      continue;
-    }
-    j -= n_wH;
-    if (j < n_wR0S) {
-      wR0S[j] = unit_root(j, (int64_t)g.R0 * g.S);
-      continue;
-    }
-    j -= n_wR0S;
-    if (j < n_wS) {
-      wS[j] = unit_root(j, g.S);
-      continue;
-    }
-    j -= n_wS;
-    if (j < n_wN) {
-      wN[j] = unit_root(j, g.N);
-      continue;
-    }
-    j -= n_wN;
-    const int64_t at = j;
-    int t = 0;
-    while (j >= unit_table_size(ug, t)) j -= unit_table_size(ug, t++);
-    const Turn a = unit_table_turn(ug, t, (int)j);
-    double s, c;
-    sincospi(2.0 * (double)a.num / (double)a.den, &s, &c);
-    unit[at] = rot_entry(c, s);
-  }
-}
 
 // Per-device set-up: the device address of the scratch array, looked up once
 // per device with that device current.
@@ -164,25 +93,13 @@ extern "C" int bege_search_noalloc(const float* strain_dev, int64_t n, const flo
       g_addr[dev] = static_cast<unsigned char*>(p);
     }
     base = g_addr[dev];
-    PlanDev p{};
-    p.g = g;
-    p.tw2 = reinterpret_cast<const float2*>(base + kOffTw2);
-    p.tw3 = reinterpret_cast<const float2*>(base + kOffTw3);
-    p.wH = reinterpret_cast<const float2*>(base + kOffWH);
-    p.wR0S = reinterpret_cast<const float2*>(base + kOffWR0S);
-    p.wS = reinterpret_cast<const float2*>(base + kOffWS);
-    p.wN = reinterpret_cast<const float2*>(base + kOffWN);
-    float2* const unit = reinterpret_cast<float2*>(base + kOffUnit);
-    const float2** const tables[kUnitTables] = {&p.t1, &p.t2, &p.t3, &p.u2, &p.u1, &p.uc};
-    for (int t = 0; t < kUnitTables; ++t) *tables[t] = unit + unit_tables(unit_geo(g), t);
     // The tables are rebuilt on every call, in stream order before this
     // call's kernels: the host keeps no record of which n the array holds,
     // which could disagree with the device's order of work.
-    search_tables_kernel<<<64, 256, 0, s>>>(
-        g, const_cast<float2*>(p.tw2), const_cast<float2*>(p.tw3), const_cast<float2*>(p.wH),
-        const_cast<float2*>(p.wR0S), const_cast<float2*>(p.wS), const_cast<float2*>(p.wN), unit);
-    e = cudaGetLastError();
+    float2* const tables = reinterpret_cast<float2*>(base + kOffTables);
+    e = launch_plan_tables(g, tables, s);
     if (e != cudaSuccess) return set_last_error(BEGE_ECUDA, cudaGetErrorString(e));
+    const PlanDev p = plan_at(g, tables);
     float4* AB = reinterpret_cast<float4*>(base + kOffAB);
     float2* D = reinterpret_cast<float2*>(base + kOffD);
     e = launch_segment(p, strain_dev, D, AB, false, s);

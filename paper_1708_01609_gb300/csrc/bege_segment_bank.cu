@@ -1,6 +1,6 @@
-// Geometry, launch-shape tables, the segment-spectrum kernel launcher and
+// Geometry, plan tables, launch shapes, the segment-spectrum launcher and
 // chirp-bank synthesis.
-#include "bege_corr.cuh"
+#include "bege_unit.cuh"
 
 namespace bege {
 
@@ -10,8 +10,47 @@ Geometry make_geometry(int64_t n) {
   g.H = g.N / 2;
   g.F = g.H < 4096 ? g.H : 4096;
   g.S = g.H / g.F;
-  g.R0 = g.F / 256;
   return g;
+}
+
+PlanDev plan_at(const Geometry& g, float2* base) {
+  PlanDev p{};
+  p.g = g;
+  const UnitGeo u = unit_geo(g);
+  const float2** const table[kUnitTables] = {&p.t1, &p.t2, &p.t3, &p.u2, &p.u1, &p.uc};
+  for (int t = 0; t < kUnitTables; ++t) {
+    *table[t] = base;
+    base += unit_table_size(u, t);
+  }
+  p.wS = base;
+  p.wN = base + u.S;
+  return p;
+}
+
+// One table entry per thread (plan_at's order).
+__global__ void __launch_bounds__(256) plan_tables_kernel(Geometry g, float2* __restrict__ base) {
+  int i = blockIdx.x * 256 + threadIdx.x;
+  if (i >= plan_floats2(g)) return;
+  float2* const out = base + i;
+  const UnitGeo u = unit_geo(g);
+  double s, c;
+  for (int t = 0; t < kUnitTables; ++t) {
+    if (i < unit_table_size(u, t)) {
+      const Turn a = unit_table_turn(u, t, i);
+      sincospi(2.0 * (double)a.num / (double)a.den, &s, &c);
+      *out = rot_entry(c, s);
+      return;
+    }
+    i -= unit_table_size(u, t);
+  }
+  const bool ws = i < u.S;  // exp(-2 pi i k / S), then exp(-2 pi i j / N)
+  sincospi(-2.0 * (double)(ws ? i : i - u.S) / (double)(ws ? u.S : g.N), &s, &c);
+  *out = make_float2((float)c, (float)s);
+}
+
+cudaError_t launch_plan_tables(const Geometry& g, float2* base, cudaStream_t s) {
+  plan_tables_kernel<<<(plan_floats2(g) + 255) / 256, 256, 0, s>>>(g, base);
+  return cudaGetLastError();
 }
 
 int correlate_configs(const Geometry& g, CorrConfig* out, int max) {
@@ -50,20 +89,12 @@ CorrConfig default_config(const Geometry& g) {
 
 cudaError_t launch_segment(const PlanDev& p, const float* y, float2* D, float4* AB, bool natural,
                            cudaStream_t s) {
-  const Geometry& g = p.g;
-  switch (g.S) {
-    case 1:
-      switch (g.F) {
-        case 512: return launch_segment_t<512, 1, 1, 256>(p, y, D, AB, natural, s);
-        case 1024: return launch_segment_t<1024, 1, 1, 256>(p, y, D, AB, natural, s);
-        case 2048: return launch_segment_t<2048, 1, 1, 256>(p, y, D, AB, natural, s);
-        case 4096: return launch_segment_t<4096, 1, 1, 256>(p, y, D, AB, natural, s);
-        default: return cudaErrorInvalidValue;
-      }
-    case 2: return launch_segment_t<4096, 2, 2, 256>(p, y, D, AB, natural, s);
-    case 4: return launch_segment_t<4096, 4, 4, 512>(p, y, D, AB, natural, s);
-    case 8: return launch_segment_t<4096, 8, 4, 512>(p, y, D, AB, natural, s);
-    case 16: return launch_segment_t<4096, 16, 4, 512>(p, y, D, AB, natural, s);
+  switch (unit_geo(p.g).F) {
+    case 256: return unit::launch_segment_t<256, true>(p, y, D, AB, natural, s);
+    case 512: return unit::launch_segment_t<512, true>(p, y, D, AB, natural, s);
+    case 1024: return unit::launch_segment_t<1024, true>(p, y, D, AB, natural, s);
+    case 2048: return unit::launch_segment_t<2048, true>(p, y, D, AB, natural, s);
+    case 4096: return unit::launch_segment_t<4096, false>(p, y, D, AB, natural, s);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -412,11 +412,59 @@ __device__ __forceinline__ float4 ld_coef(const float4* p) {
   return v;
 }
 
+// Stage 3 of the two butterflies m of thread tid: za[k2] = Z, zb[r] = conj Z of
+// the mirror at its row 15 - r, which are the outputs of the same twiddled
+// DFT on the conjugated inputs (so both butterflies use one set of twiddles);
+// self: zb[r] = Z of its own row r.
+template <class SM>
+__device__ __forceinline__ const float4* mid_row(int ui, int slot, int k0, int k1) {
+  return SM::rows(ui) + k0 * kBlk + (slot * 144 + k1 * 9);
+}
+template <class SM>
+__device__ __forceinline__ void stage3(int ui, const MidItem& m, bool self, float2 (&za)[16],
+                                       float2 (&zb)[16]) {
+  constexpr int kT = SM::G::T;
+  const int t = SM::tid();
+  const float4* pa = mid_row<SM>(ui, m.sa, m.k0, m.k1);
+  const float4* pb = mid_row<SM>(ui, m.sb, m.k0b, m.k1b);
+  float2 xa[16], xb[16];
+#pragma unroll
+  for (int r = 0; r < 8; ++r) {
+    const float4 v = pa[r], u = pb[r];
+    xa[2 * r] = make_float2(v.x, v.y);
+    xa[2 * r + 1] = make_float2(v.z, v.w);
+    xb[2 * r] = make_float2(u.x, -u.y);
+    xb[2 * r + 1] = make_float2(u.z, -u.w);
+  }
+  if (self) {  // butterfly (0, 8) has its own base, 1/32 turn, and no mirror
+    constexpr float c[16] = {1.f, 0.98078528040323044913f, 0.92387953251128675613f,
+                             0.83146961230254523708f, 0.70710678118654752440f,
+                             0.55557023301960222474f, 0.38268343236508977173f,
+                             0.19509032201612826785f, 0.f, -0.19509032201612826785f,
+                             -0.38268343236508977173f, -0.55557023301960222474f,
+                             -0.70710678118654752440f, -0.83146961230254523708f,
+                             -0.92387953251128675613f, -0.98078528040323044913f};
+#pragma unroll
+    for (int r = 1; r < 16; ++r) {
+      const float s = r < 8 ? c[8 - r] : c[r - 8];  // sin(2 pi r / 32)
+      xb[r] = cmul(cconj(xb[r]), make_float2(c[r], -s));
+    }
+    xb[0] = cconj(xb[0]);
+  }
+  const float2* w = SM::t3(ui) + t;
+  dft16x2<false, false>(xa, xb, [&](int q) {
+    const float2 s = w[kT * q];
+    return make_float4(s.x, s.y, s.x, s.y);
+  });
+#pragma unroll
+  for (int r = 0; r < 16; ++r) {
+    za[r] = xa[rev<16>(r)];
+    zb[r] = xb[rev<16>(r)];
+  }
+}
+
 // Stage 3, the product with sum |Y|^2, stage 3' of thread t's two
-// butterflies, in place.  zb holds the mirror's outputs conjugated and
-// reversed, g[r] = conj Z[mirror row 15 - r], which are the outputs of the
-// same twiddled DFT on the conjugated inputs (so both butterflies use one
-// set of twiddles).  MULTI: the spectrum is kept in `scratch` (32 values a
+// butterflies, in place.  MULTI: the spectrum is kept in `scratch` (32 values a
 // thread, stride kT) for the block's other segments, or with `reload` read
 // from there.  AHEAD: pairs of rows whose coefficients are loaded ahead.
 template <class SM, int AHEAD, bool MULTI = false, bool WAIT = false>
@@ -427,8 +475,8 @@ __device__ __forceinline__ void middle(int ui, int ug, const float4* __restrict_
   const int t = SM::tid();
   const bool unit0 = ug == 0, self = unit0 && t == 0;
   const MidItem m = mid_item<SM::G::R>(unit0, t);
-  float4* pa = SM::rows(ui) + m.k0 * kBlk + (m.sa * 144 + m.k1 * 9);
-  float4* pb = SM::rows(ui) + m.k0b * kBlk + (m.sb * 144 + m.k1b * 9);
+  float4* pa = const_cast<float4*>(mid_row<SM>(ui, m.sa, m.k0, m.k1));
+  float4* pb = const_cast<float4*>(mid_row<SM>(ui, m.sb, m.k0b, m.k1b));
   const float4* ab = coef + (size_t)ug * (24 * kT) + t;
   float2 za[16], zb[16];
   // the coefficients of the first AHEAD pairs of rows are under way during
@@ -447,42 +495,7 @@ __device__ __forceinline__ void middle(int ui, int ug, const float4* __restrict_
       zb[r] = __ldcg(scratch + (16 + r) * kT + t);
     }
   } else {
-    {
-      float2 xa[16], xb[16];
-#pragma unroll
-      for (int r = 0; r < 8; ++r) {
-        const float4 v = pa[r], u = pb[r];
-        xa[2 * r] = make_float2(v.x, v.y);
-        xa[2 * r + 1] = make_float2(v.z, v.w);
-        xb[2 * r] = make_float2(u.x, -u.y);
-        xb[2 * r + 1] = make_float2(u.z, -u.w);
-      }
-      if (self) {  // butterfly (0, 8) has its own base, 1/32 turn, and no mirror
-        constexpr float c[16] = {1.f, 0.98078528040323044913f, 0.92387953251128675613f,
-                                 0.83146961230254523708f, 0.70710678118654752440f,
-                                 0.55557023301960222474f, 0.38268343236508977173f,
-                                 0.19509032201612826785f, 0.f, -0.19509032201612826785f,
-                                 -0.38268343236508977173f, -0.55557023301960222474f,
-                                 -0.70710678118654752440f, -0.83146961230254523708f,
-                                 -0.92387953251128675613f, -0.98078528040323044913f};
-#pragma unroll
-        for (int r = 1; r < 16; ++r) {
-          const float s = r < 8 ? c[8 - r] : c[r - 8];  // sin(2 pi r / 32)
-          xb[r] = cmul(cconj(xb[r]), make_float2(c[r], -s));
-        }
-        xb[0] = cconj(xb[0]);
-      }
-      const float2* w = SM::t3(ui) + t;
-      dft16x2<false, false>(xa, xb, [&](int q) {
-        const float2 s = w[kT * q];
-        return make_float4(s.x, s.y, s.x, s.y);
-      });
-#pragma unroll
-      for (int r = 0; r < 16; ++r) {
-        za[r] = xa[rev<16>(r)];
-        zb[r] = xb[rev<16>(r)];
-      }
-    }
+    stage3<SM>(ui, m, self, za, zb);
     if (MULTI && scratch) {
 #pragma unroll
       for (int r = 0; r < 16; ++r) {
@@ -568,7 +581,7 @@ template <class SM, int U>
 __device__ __forceinline__ void mid_enter(int ui, int ug) {
   __syncwarp();
   if (ug != 0 || SM::G::T <= 32) return;
-  if constexpr (U > 1) {
+  if constexpr (U > 1 || SM::G::W != 8) {
     SM::sync(ui);
   } else {
     const int w8 = threadIdx.x >> 5;
@@ -581,7 +594,7 @@ template <class SM, int U>
 __device__ __forceinline__ void mid_leave(int ui, int ug) {
   __syncwarp();
   if (ug != 0 || SM::G::T <= 32) return;
-  if constexpr (U > 1) {
+  if constexpr (U > 1 || SM::G::W != 8) {
     SM::sync(ui);
   } else {
     const int w8 = threadIdx.x >> 5;
@@ -643,6 +656,161 @@ __device__ __forceinline__ void stage1i(int ui, float2 (&va)[16 / SM::G::R][SM::
       dft_row<R, true>(vb[i], [&](int q) { return w[256 * q]; });
     }
   }
+}
+
+// ---------------------------------------------------------------------------
+// S1: segment spectrum D and product coefficients A, B of a unit
+// ---------------------------------------------------------------------------
+// The strain takes the template's stages 1 to 3 (folded over the S multiples
+// of F), so a thread ends with the bins of a butterfly and its mirror: D, A
+// and B of both follow in registers.
+struct BinPair {
+  float2 A, B, Am, Bm;  // of bin j and of bin H - j
+};
+// Bins j and jm = H - j (j = 0: jm = 0 stands for the Nyquist bin's partner).
+__device__ __forceinline__ BinPair bin_pair(const PlanDev& p, int j, int jm, float2 zj, float2 zm,
+                                            float2* __restrict__ D) {
+  const int H = p.g.H;
+  // D_j = (Zj + conj Zm)/2 - (i/2) wN^j (Zj - conj Zm)
+  auto spectrum = [](float2 w, float2 x, float2 y) {
+    const float2 s = cadd(x, cconj(y)), d = csub(x, cconj(y));
+    const float2 e = cmul(w, d);
+    return make_float2(0.5f * (s.x + e.y), 0.5f * (s.y - e.x));
+  };
+  auto coeffs = [](float2 w, float2 Dx, float2 cH, float2& A, float2& B) {
+    // g = (1 + i conj w)/2, d = (1 - i conj w)/2 with i conj(w) = (w.y, w.x)
+    const float2 g = make_float2(0.5f * (1.f + w.y), 0.5f * w.x);
+    const float2 d = make_float2(0.5f * (1.f - w.y), -0.5f * w.x);
+    A = cadd(cmul(cmul(g, g), Dx), cmul(cmul(d, d), cH));
+    B = cmul(cmul(g, d), cadd(Dx, cH));
+  };
+  const float2 wj = p.wN[j], wm = p.wN[jm];
+  const float2 Dj = spectrum(wj, zj, zm);
+  const float2 Dm = j == jm ? Dj : spectrum(wm, zm, zj);
+  const float2 DH = make_float2(zj.x - zj.y, 0.f);  // D_{N/2}, used when j == 0
+  BinPair o;
+  coeffs(wj, Dj, j == 0 ? DH : cconj(Dm), o.A, o.B);
+  coeffs(wm, Dm, j == 0 ? DH : cconj(Dj), o.Am, o.Bm);
+  D[j] = Dj;
+  if (j != jm) D[jm] = Dm;
+  if (j == 0) D[H] = DH;
+  return o;
+}
+
+// natural: {A, B} of bin j at (j mod S) F + j / S (the tensor-core kernel);
+// otherwise where middle reads them.  The first T threads of the CTA run the
+// stages and leave the spectrum in shared memory by thread and row (Z of row r
+// at 2 r T + t, of its mirror at (2 r + 1) T + t; thread 0 of unit 0: rows r
+// of its two butterflies), and all of them form the pairs: a loop over 16 T
+// items keeps the code short (unrolled over the 16 rows of a butterfly it took
+// 25 us for N = 2^12, mostly instruction fetches) and every thread at work.
+template <class SM, bool ONE>
+__device__ __forceinline__ void segment_unit(const PlanDev& p, int S, int ug,
+                                             const float* __restrict__ y, float2* __restrict__ D,
+                                             float4* __restrict__ AB, bool natural) {
+  constexpr int R = SM::G::R, T = SM::G::T, F = 256 * R;
+  const bool fft = threadIdx.x < (T < 32 ? 32 : T);  // F = 256: a second unit repeats the first
+  const int ui = T < 32 ? ((int)threadIdx.x / T) & 1 : 0;
+  if ((int)threadIdx.x < T) setup_unit<SM>(p, S, ug, 0);
+  __syncthreads();
+  if (fft) stage1<SM, false, ONE, false>(ui, S, ug, y, p.g.H, S);
+  __syncthreads();
+  if (fft) stage2<SM>(ui);
+  __syncthreads();
+  float2* const z = reinterpret_cast<float2*>(SM::rows(ui));
+  {
+    const int t = SM::tid();
+    float2 za[16], zb[16];
+    const bool self = ug == 0 && t == 0;
+    if (fft) stage3<SM>(ui, mid_item<R>(ug == 0, t), self, za, zb);
+    __syncthreads();  // the rows have been read
+    if (fft) {
+#pragma unroll
+      for (int r = 0; r < 16; ++r) {
+        z[2 * r * T + t] = za[r];
+        z[(2 * r + 1) * T + t] = self ? zb[r] : cconj(zb[r]);
+      }
+    }
+  }
+  __syncthreads();
+  const float2* const zs = reinterpret_cast<const float2*>(SM::rows(0));
+  auto place = [&](int j, float2 A, float2 B) {
+    AB[(j % S) * F + j / S] = make_float4(A.x, A.y, B.x, B.y);
+  };
+  auto bin = [&](int b, int k0, int k1, int k2) { return S * (k0 + R * k1 + 16 * R * k2) + b; };
+  float2* const af = reinterpret_cast<float2*>(AB + (size_t)ug * (24 * T));
+  // third q of the pair of rows that holds `row`: {A, A'} of either row, {B, B}
+  auto third = [&](int row, int q, int t) { return 2 * ((3 * (row >> 1) + q) * T + t); };
+#pragma unroll 2
+  for (int it = threadIdx.x; it < 16 * T; it += blockDim.x) {
+    const int t = it & (T - 1), r = it / T;
+    if (ug != 0 || t != 0) {
+      const MidItem m = mid_item<R>(ug == 0, t);
+      const int ba = ug == 0 ? m.sa * (S / 2) : ug, bb = ug == 0 ? ba : S - ug;
+      const int j = bin(ba, m.k0, m.k1, r), jm = bin(bb, m.k0b, m.k1b, 15 - r);
+      const BinPair o = bin_pair(p, j, jm, zs[2 * r * T + t], zs[(2 * r + 1) * T + t], D);
+      if (natural) {
+        place(j, o.A, o.B);
+        place(jm, o.Am, o.Bm);
+      } else {
+        *reinterpret_cast<float4*>(af + third(r, r & 1, t)) =
+            make_float4(o.A.x, o.A.y, o.Am.x, o.Am.y);
+        af[third(r, 2, t) + (r & 1)] = o.B;
+      }
+      continue;
+    }
+    // rows r and (16 - r) mod 16 of butterfly (0, 0), r and 15 - r of (0, 8);
+    // where the product's thread 0 looks for them, see middle
+    if (r <= 8) {
+      const int rm = (16 - r) & 15, j = bin(0, 0, 0, r), jm = bin(0, 0, 0, rm);
+      const BinPair o = bin_pair(p, j, jm, zs[2 * r * T], zs[2 * rm * T], D);
+      if (natural) {
+        place(j, o.A, o.B);
+        if (jm != j) place(jm, o.Am, o.Bm);
+      } else {
+        af[third(r, r & 1, 0)] = o.A;
+        if (jm != j) af[third(rm, rm & 1, 0)] = o.Am;
+        float2* const b = af + third(r & 7, 2, 0) + (r & 1);
+        if (r == 0)
+          b->x = o.B.x;
+        else if (r == 8)
+          b->y = o.B.x;
+        else
+          *b = o.B;
+      }
+    }
+    if (r < 8) {
+      const int j = bin(0, 0, 8, r), jm = bin(0, 0, 8, 15 - r);
+      const BinPair o = bin_pair(p, j, jm, zs[(2 * r + 1) * T], zs[(2 * (15 - r) + 1) * T], D);
+      if (natural) {
+        place(j, o.A, o.B);
+        place(jm, o.Am, o.Bm);
+      } else {
+        af[third(15 - r, (15 - r) & 1, 0) + 1] = o.A;
+        af[third(r, r & 1, 0) + 1] = o.Am;
+        af[third(8 + r, 2, 0) + (r & 1)] = o.B;
+      }
+    }
+  }
+}
+
+// One CTA of 256 threads per unit.
+template <int F, bool ONE>
+__global__ void __launch_bounds__(256, 1)
+segment_kernel(PlanDev p, const float* __restrict__ y, float2* __restrict__ D,
+               float4* __restrict__ AB, bool natural) {
+  segment_unit<Sm<F, F == 256 ? 2 : 1, ONE>, ONE>(p, unit_geo(p.g).S, blockIdx.x, y, D, AB, natural);
+}
+
+template <int F, bool ONE>
+static cudaError_t launch_segment_t(const PlanDev& p, const float* y, float2* D, float4* AB,
+                                    bool natural, cudaStream_t s) {
+  constexpr size_t smem = Lay<F, F == 256 ? 2 : 1, ONE>::total;
+  auto kern = segment_kernel<F, ONE>;
+  cudaError_t e = ensure_smem(kern, smem);
+  if (e != cudaSuccess) return e;
+  kern<<<unit_geo(p.g).S / 2, 256, smem, s>>>(p, y, D, AB, natural);
+  return cudaGetLastError();
 }
 
 // Sum |Y|^2 of a unit, in warp order (after a barrier that follows the middle).
