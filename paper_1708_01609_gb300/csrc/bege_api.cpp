@@ -67,6 +67,7 @@ struct Segment {
   int32_t channel = 0;
   DevBuf D, AB;
   std::shared_ptr<PlanHost> plan;
+  bool loaded = false;  // its kernel is known to have finished
 };
 
 struct Bank {
@@ -74,10 +75,14 @@ struct Bank {
   DevBuf w;
 };
 
+// What a job needs beside its segment and bank; kept by the context between
+// jobs (events included: creating three costs more than a small launch).
 struct JobBuffers {
   DevBuf sigma, recs, counter;
   int64_t sigma_cap = 0;
   uint64_t rec_cap = 0;
+  cudaEvent_t done = nullptr;
+  cudaEvent_t k_start = nullptr, k_stop = nullptr;  // around the correlate kernel
 };
 
 struct Job {
@@ -88,16 +93,9 @@ struct Job {
   DevBuf proj;        // per-lag maximum over the bank (bege_correlate_max), n_proj words
   int64_t n_proj = 0;
   DevBuf scratch;     // bege_correlate_multi: the group's template-spectrum scratch
-  cudaEvent_t done = nullptr;
-  cudaEvent_t k_start = nullptr, k_stop = nullptr;  // around the correlate kernel
+  bool counted = false;             // the finished job's counter has been read into
+  unsigned long long count[2] = {};  // {tail count, status}
 };
-
-static void destroy_job_events(Job* j) {
-  if (j->done) cudaEventDestroy(j->done);
-  if (j->k_start) cudaEventDestroy(j->k_start);
-  if (j->k_stop) cudaEventDestroy(j->k_stop);
-  j->done = j->k_start = j->k_stop = nullptr;
-}
 
 struct BatchEntryHost {
   int64_t n = 0;
@@ -137,12 +135,27 @@ struct bege_ctx {
   std::vector<std::unique_ptr<JobBuffers>> pool;
   std::map<int64_t, bege::CorrConfig> configs;  // chosen launch shape per N
 
+  // Segment buffers (spectrum, coefficients, staged strain) of released
+  // segments, all idle, for the next segment of that length: cudaMalloc and
+  // cudaFree of these few buffers took 10 us of a small search, and 100 us
+  // where the driver gave back and fetched a whole block each time.  At most
+  // kSpareBytes, and given back whenever an allocation would not fit.
+  static constexpr uint64_t kSpareBytes = 4u << 20;
+  std::vector<DevBuf> spare;
+  uint64_t spare_bytes = 0;
+
   int alloc(DevBuf* b, size_t bytes) {
+    if (cfg.hbm_budget_bytes && this->bytes + bytes > cfg.hbm_budget_bytes) drop_spare();
     if (cfg.hbm_budget_bytes && this->bytes + bytes > cfg.hbm_budget_bytes)
       return fail(BEGE_EBUDGET, "device allocation of " + std::to_string(bytes) +
                                     " bytes exceeds the HBM budget");
     void* p = nullptr;
     cudaError_t e = cudaMalloc(&p, bytes ? bytes : 16);
+    if (e != cudaSuccess && !spare.empty()) {
+      cudaGetLastError();
+      drop_spare();
+      e = cudaMalloc(&p, bytes ? bytes : 16);
+    }
     if (e != cudaSuccess) {
       cudaGetLastError();
       return fail(BEGE_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
@@ -159,6 +172,42 @@ struct bege_ctx {
     }
     b->ptr = nullptr;
     b->bytes = 0;
+  }
+  // As alloc and release, by way of the spare buffers.  keep: no work that
+  // uses the buffer is unfinished.
+  int take(DevBuf* b, size_t bytes) {
+    for (size_t i = 0; i < spare.size(); ++i) {
+      if (spare[i].bytes == bytes) {
+        *b = spare[i];
+        spare[i] = spare.back();
+        spare.pop_back();
+        spare_bytes -= bytes;
+        return BEGE_OK;
+      }
+    }
+    return alloc(b, bytes);
+  }
+  void keep(DevBuf* b) {
+    if (!b->ptr || spare_bytes + b->bytes > kSpareBytes) {
+      release(b);
+      return;
+    }
+    spare_bytes += b->bytes;
+    spare.push_back(*b);
+    *b = DevBuf{};
+  }
+  void drop_spare() {
+    for (DevBuf& b : spare) release(&b);
+    spare.clear();
+    spare_bytes = 0;
+  }
+  void free_buffers(JobBuffers* b) {
+    release(&b->sigma);
+    release(&b->recs);
+    release(&b->counter);
+    for (cudaEvent_t e : {b->done, b->k_start, b->k_stop})
+      if (e) cudaEventDestroy(e);
+    b->done = b->k_start = b->k_stop = nullptr;
   }
 };
 
@@ -213,11 +262,11 @@ int segment_common(bege_ctx* ctx, const float* y_dev, int64_t n, int32_t channel
   seg->channel = channel;
   seg->plan = plan;
   const bege::Geometry& g = plan->g;
-  rc = ctx->alloc(&seg->D, (size_t)(g.H + 1) * sizeof(float2));
+  rc = ctx->take(&seg->D, (size_t)(g.H + 1) * sizeof(float2));
   if (rc) return rc;
-  rc = ctx->alloc(&seg->AB, (size_t)g.H * sizeof(float4));
+  rc = ctx->take(&seg->AB, (size_t)g.H * sizeof(float4));
   if (rc) {
-    ctx->release(&seg->D);
+    ctx->keep(&seg->D);
     return rc;
   }
   cudaError_t e = bege::launch_segment(plan->dev, y_dev, static_cast<float2*>(seg->D.ptr),
@@ -255,9 +304,30 @@ int take_job_buffers(bege_ctx* ctx, int64_t nsig, uint64_t cap, std::unique_ptr<
     ctx->release(&b->recs);
     return rc;
   }
+  cudaError_t e = cudaEventCreateWithFlags(&b->done, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaEventCreate(&b->k_start);
+  if (e == cudaSuccess) e = cudaEventCreate(&b->k_stop);
+  if (e != cudaSuccess) {
+    ctx->free_buffers(b.get());
+    return cuda_fail(e, "job events");
+  }
   b->sigma_cap = nsig;
   b->rec_cap = cap;
   *out = std::move(b);
+  return BEGE_OK;
+}
+
+// Waits for a job; its {tail count, status} (read from the device once).
+int wait_counted(Job* j) {
+  cudaError_t e = cudaEventSynchronize(j->buf->done);
+  if (e != cudaSuccess) return cuda_fail(e, "job");
+  if (!j->counted) {
+    e = cudaMemcpy(j->count, j->buf->counter.ptr, 16, cudaMemcpyDeviceToHost);
+    if (e != cudaSuccess) return cuda_fail(e, "tail count");
+    j->counted = true;
+  }
+  if (j->count[1] & 0xffffffffull)
+    return fail(BEGE_ETIMEDOUT, "a bounded device wait gave up; results of this job are invalid");
   return BEGE_OK;
 }
 
@@ -472,19 +542,13 @@ int bege_destroy(bege_ctx* ctx) {
     DeviceGuard dg(ctx->device);
     std::lock_guard<std::mutex> lk(ctx->mu);
     for (auto& kv : ctx->jobs) {
-      if (kv.second->done) cudaEventSynchronize(kv.second->done);
-      destroy_job_events(kv.second.get());
+      cudaEventSynchronize(kv.second->buf->done);
       ctx->release(&kv.second->proj);
       ctx->release(&kv.second->scratch);
-      ctx->release(&kv.second->buf->sigma);
-      ctx->release(&kv.second->buf->recs);
-      ctx->release(&kv.second->buf->counter);
+      ctx->free_buffers(kv.second->buf.get());
     }
-    for (auto& b : ctx->pool) {
-      ctx->release(&b->sigma);
-      ctx->release(&b->recs);
-      ctx->release(&b->counter);
-    }
+    for (auto& b : ctx->pool) ctx->free_buffers(b.get());
+    ctx->drop_spare();
     for (auto& kv : ctx->batches) destroy_batch(ctx, kv.second.get());
     for (auto& kv : ctx->segs) {
       ctx->release(&kv.second->D);
@@ -506,7 +570,7 @@ int bege_load_segment(bege_ctx* ctx, const float* strain, int64_t n, int32_t cha
   std::lock_guard<std::mutex> lk(ctx->mu);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   DevBuf tmp;
-  int rc = ctx->alloc(&tmp, (size_t)n * sizeof(float));
+  int rc = ctx->take(&tmp, (size_t)n * sizeof(float));
   if (rc) return rc;
   cudaError_t e = cudaMemcpyAsync(tmp.ptr, strain, (size_t)n * sizeof(float),
                                   cudaMemcpyHostToDevice, s);
@@ -515,11 +579,15 @@ int bege_load_segment(bege_ctx* ctx, const float* strain, int64_t n, int32_t cha
     return cuda_fail(e, "strain upload");
   }
   rc = segment_common(ctx, static_cast<const float*>(tmp.ptr), n, channel, s, seg_id);
-  // the segment kernel reads tmp on stream s; wait before freeing it
+  // the segment kernel reads tmp on stream s; wait before it is reused
   cudaError_t e2 = cudaStreamSynchronize(s);
-  ctx->release(&tmp);
+  if (e2 == cudaSuccess)
+    ctx->keep(&tmp);
+  else
+    ctx->release(&tmp);
   if (rc) return rc;
   if (e2 != cudaSuccess) return cuda_fail(e2, "segment kernel");
+  ctx->segs[*seg_id]->loaded = true;
   return BEGE_OK;
 }
 
@@ -659,12 +727,10 @@ static int correlate_impl(bege_ctx* ctx, int32_t seg_id, int32_t bank_id, int64_
     }
     job->n_proj = seg->n;
   }
-  cudaError_t e = cudaEventCreateWithFlags(&job->done, cudaEventDisableTiming);
-  if (e == cudaSuccess && project) e = cudaMemsetAsync(job->proj.ptr, 0, job->proj.bytes, s);
-  if (e == cudaSuccess) e = cudaEventCreate(&job->k_start);
-  if (e == cudaSuccess) e = cudaEventCreate(&job->k_stop);
+  cudaError_t e = cudaSuccess;
+  if (project) e = cudaMemsetAsync(job->proj.ptr, 0, job->proj.bytes, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(job->buf->counter.ptr, 0, 16, s);
-  if (e == cudaSuccess) e = cudaEventRecord(job->k_start, s);
+  if (e == cudaSuccess) e = cudaEventRecord(job->buf->k_start, s);
   if (e == cudaSuccess) {
     bege::CorrelateArgs a{};
     a.AB = static_cast<const float4*>(seg->AB.ptr);
@@ -694,10 +760,9 @@ static int correlate_impl(bege_ctx* ctx, int32_t seg_id, int32_t bank_id, int64_
       e = bege::launch_correlate(seg->plan->dev, a, cc, s);
     }
   }
-  if (e == cudaSuccess) e = cudaEventRecord(job->k_stop, s);
-  if (e == cudaSuccess) e = cudaEventRecord(job->done, s);
+  if (e == cudaSuccess) e = cudaEventRecord(job->buf->k_stop, s);
+  if (e == cudaSuccess) e = cudaEventRecord(job->buf->done, s);
   if (e != cudaSuccess) {
-    destroy_job_events(job.get());
     ctx->release(&job->proj);
     ctx->pool.push_back(std::move(job->buf));
     return cuda_fail(e, "correlate");
@@ -752,7 +817,6 @@ int bege_correlate_multi(bege_ctx* ctx, const int32_t* seg_ids, int32_t n_seg, i
   std::vector<std::unique_ptr<Job>> jobs;
   auto unwind = [&](int rc) {
     for (auto& j : jobs) {
-      destroy_job_events(j.get());
       ctx->release(&j->scratch);
       if (j->buf) ctx->pool.push_back(std::move(j->buf));
     }
@@ -769,10 +833,7 @@ int bege_correlate_multi(bege_ctx* ctx, const int32_t* seg_ids, int32_t n_seg, i
     Job* j = jobs.back().get();
     int rc = take_job_buffers(ctx, k_end - k_begin, ctx->cfg.tail_capacity, &j->buf);
     if (rc) return unwind(rc);
-    e = cudaEventCreateWithFlags(&j->done, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventCreate(&j->k_start);
-    if (e == cudaSuccess) e = cudaEventCreate(&j->k_stop);
-    if (e == cudaSuccess) e = cudaMemsetAsync(j->buf->counter.ptr, 0, 16, s);
+    e = cudaMemsetAsync(j->buf->counter.ptr, 0, 16, s);
     if (e != cudaSuccess) return unwind(cuda_fail(e, "multi-segment job"));
   }
   int rc = ctx->alloc(&jobs[0]->scratch, bege::multi_scratch_bytes(sms));
@@ -793,11 +854,11 @@ int bege_correlate_multi(bege_ctx* ctx, const int32_t* seg_ids, int32_t n_seg, i
   }
   a.scratch = static_cast<float2*>(jobs[0]->scratch.ptr);
   for (auto& j : jobs)
-    if (e == cudaSuccess) e = cudaEventRecord(j->k_start, s);
+    if (e == cudaSuccess) e = cudaEventRecord(j->buf->k_start, s);
   if (e == cudaSuccess) e = bege::launch_correlate_multi(segs[0]->plan->dev, a, s);
   for (auto& j : jobs) {
-    if (e == cudaSuccess) e = cudaEventRecord(j->k_stop, s);
-    if (e == cudaSuccess) e = cudaEventRecord(j->done, s);
+    if (e == cudaSuccess) e = cudaEventRecord(j->buf->k_stop, s);
+    if (e == cudaSuccess) e = cudaEventRecord(j->buf->done, s);
   }
   if (e != cudaSuccess) return unwind(cuda_fail(e, "multi-segment correlate"));
   for (int32_t i = 0; i < n_seg; ++i) {
@@ -855,15 +916,10 @@ int bege_fetch_max(bege_ctx* ctx, int32_t job_id, float* snr, int32_t* tmpl, int
   if (!j) return fail(BEGE_EINVAL, "unknown job handle");
   if (!j->proj.ptr) return fail(BEGE_EINVAL, "the job was not started by bege_correlate_max");
   if (n != j->n_proj) return fail(BEGE_EINVAL, "n must equal the segment length");
-  cudaError_t e = cudaEventSynchronize(j->done);
-  if (e != cudaSuccess) return cuda_fail(e, "job");
-  unsigned long long cs[2] = {0, 0};
-  e = cudaMemcpy(cs, j->buf->counter.ptr, 16, cudaMemcpyDeviceToHost);
-  if (e != cudaSuccess) return cuda_fail(e, "tail count");
-  if (cs[1] & 0xffffffffull)
-    return fail(BEGE_ETIMEDOUT, "a bounded device wait gave up; results of this job are invalid");
+  int rc = wait_counted(j);
+  if (rc) return rc;
   std::vector<unsigned long long> w((size_t)n);
-  e = cudaMemcpy(w.data(), j->proj.ptr, (size_t)n * sizeof(unsigned long long),
+  cudaError_t e = cudaMemcpy(w.data(), j->proj.ptr, (size_t)n * sizeof(unsigned long long),
                  cudaMemcpyDeviceToHost);
   if (e != cudaSuccess) return cuda_fail(e, "projection");
   for (int64_t i = 0; i < n; ++i) {
@@ -887,8 +943,8 @@ int bege_job_kernel_ms(bege_ctx* ctx, int32_t job_id, float* ms) {
   std::lock_guard<std::mutex> lk(ctx->mu);
   Job* j = find_job(ctx, job_id);
   if (!j) return fail(BEGE_EINVAL, "unknown job handle");
-  cudaError_t e = cudaEventSynchronize(j->done);
-  if (e == cudaSuccess) e = cudaEventElapsedTime(ms, j->k_start, j->k_stop);
+  cudaError_t e = cudaEventSynchronize(j->buf->done);
+  if (e == cudaSuccess) e = cudaEventElapsedTime(ms, j->buf->k_start, j->buf->k_stop);
   if (e != cudaSuccess) return cuda_fail(e, "kernel time");
   return BEGE_OK;
 }
@@ -899,7 +955,7 @@ int bege_query(bege_ctx* ctx, int32_t job_id) {
   std::lock_guard<std::mutex> lk(ctx->mu);
   Job* j = find_job(ctx, job_id);
   if (!j) return fail(BEGE_EINVAL, "unknown job handle");
-  cudaError_t e = cudaEventQuery(j->done);
+  cudaError_t e = cudaEventQuery(j->buf->done);
   if (e == cudaErrorNotReady) return BEGE_ENOTREADY;
   if (e != cudaSuccess) return cuda_fail(e, "job");
   return BEGE_OK;
@@ -921,19 +977,15 @@ int bege_fetch_tails(bege_ctx* ctx, int32_t job_id, bege_tail* out, int64_t capa
   std::lock_guard<std::mutex> lk(ctx->mu);
   Job* j = find_job(ctx, job_id);
   if (!j) return fail(BEGE_EINVAL, "unknown job handle");
-  cudaError_t e = cudaEventSynchronize(j->done);
-  if (e != cudaSuccess) return cuda_fail(e, "job");
-  unsigned long long cs[2] = {0, 0};
-  e = cudaMemcpy(cs, j->buf->counter.ptr, 16, cudaMemcpyDeviceToHost);
-  if (e != cudaSuccess) return cuda_fail(e, "tail count");
-  const unsigned long long total = cs[0];
-  if (cs[1] & 0xffffffffull)
-    return fail(BEGE_ETIMEDOUT, "a bounded device wait gave up; results of this job are invalid");
+  int rc = wait_counted(j);
+  if (rc) return rc;
+  const unsigned long long total = j->count[0];
   uint64_t ncopy = total;
   if (ncopy > j->buf->rec_cap) ncopy = j->buf->rec_cap;
   if (ncopy > (uint64_t)capacity) ncopy = (uint64_t)capacity;
   if (ncopy) {
-    e = cudaMemcpy(out, j->buf->recs.ptr, ncopy * sizeof(bege_tail), cudaMemcpyDeviceToHost);
+    cudaError_t e = cudaMemcpy(out, j->buf->recs.ptr, ncopy * sizeof(bege_tail),
+                               cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return cuda_fail(e, "tail records");
   }
   *n_written = (int64_t)ncopy;
@@ -951,7 +1003,7 @@ int bege_get_sigma(bege_ctx* ctx, int32_t job_id, float* out, int64_t count) {
   Job* j = find_job(ctx, job_id);
   if (!j) return fail(BEGE_EINVAL, "unknown job handle");
   if (count != j->k1 - j->k0) return fail(BEGE_EINVAL, "count must equal k_end - k_begin");
-  cudaError_t e = cudaEventSynchronize(j->done);
+  cudaError_t e = cudaEventSynchronize(j->buf->done);
   if (e == cudaSuccess)
     e = cudaMemcpy(out, j->buf->sigma.ptr, (size_t)count * sizeof(float), cudaMemcpyDeviceToHost);
   if (e != cudaSuccess) return cuda_fail(e, "sigma");
@@ -985,7 +1037,6 @@ int bege_dump_correlation(bege_ctx* ctx, int32_t seg_id, int32_t bank_id, int64_
   ctx->release(&d);
   Job* j = find_job(ctx, job);
   if (j) {
-    destroy_job_events(j);
     ctx->pool.push_back(std::move(j->buf));
     ctx->jobs.erase(job);
   }
@@ -1051,10 +1102,9 @@ int bege_autotune(bege_ctx* ctx, int32_t seg_id, int32_t bank_id, int64_t k_begi
       if (rc) return rc;
       Job* j = find_job(ctx, job);
       float ms = 0.f;
-      cudaError_t e = cudaEventSynchronize(j->done);
-      if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, j->k_start, j->k_stop);
-      destroy_job_events(j);
-      ctx->pool.push_back(std::move(j->buf));
+      cudaError_t e = cudaEventSynchronize(j->buf->done);
+      if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, j->buf->k_start, j->buf->k_stop);
+        ctx->pool.push_back(std::move(j->buf));
       ctx->jobs.erase(job);
       if (e != cudaSuccess) return cuda_fail(e, "autotune");
       if (r > 0) t.push_back(ms);
@@ -1396,8 +1446,7 @@ int bege_release(bege_ctx* ctx, int32_t handle) {
   std::lock_guard<std::mutex> lk(ctx->mu);
   auto ji = ctx->jobs.find(handle);
   if (ji != ctx->jobs.end()) {
-    cudaEventSynchronize(ji->second->done);
-    destroy_job_events(ji->second.get());
+    cudaEventSynchronize(ji->second->buf->done);
     ctx->release(&ji->second->proj);
     ctx->release(&ji->second->scratch);
     ctx->pool.push_back(std::move(ji->second->buf));
@@ -1412,9 +1461,12 @@ int bege_release(bege_ctx* ctx, int32_t handle) {
   }
   auto si = ctx->segs.find(handle);
   if (si != ctx->segs.end()) {
-    cudaDeviceSynchronize();
-    ctx->release(&si->second->D);
-    ctx->release(&si->second->AB);
+    // what may still use the segment: its own kernel, jobs not released yet
+    if (!si->second->loaded) cudaDeviceSynchronize();
+    for (auto& kv : ctx->jobs)
+      if (kv.second->seg == handle) cudaEventSynchronize(kv.second->buf->done);
+    ctx->keep(&si->second->D);
+    ctx->keep(&si->second->AB);
     ctx->segs.erase(si);
     return BEGE_OK;
   }

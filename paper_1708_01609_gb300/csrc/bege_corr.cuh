@@ -45,6 +45,7 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <atomic>
 
 #include "bege_fft.cuh"
 #include "bege_internal.h"
@@ -266,12 +267,46 @@ static cudaError_t ensure_smem(K kernel, size_t bytes) {
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
+// Clusters of C CTAs of `kern` that fit on the current device at once.  The
+// answer does not change, so each kernel keeps it per device (the query and
+// the attribute take longer than a launch).
+template <auto kern>
+static cudaError_t resident_clusters(int C, int threads, size_t smem, int minb, int* out) {
+  constexpr int kDevices = 64;
+  static std::atomic<int> known[kDevices];
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < kDevices && (*out = known[dev].load(std::memory_order_acquire)) > 0) return cudaSuccess;
+  e = ensure_smem(kern, smem);
+  if (e != cudaSuccess) return e;
+  e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)C;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  cfg.blockDim = dim3((unsigned)threads, 1, 1);
+  cfg.gridDim = dim3((unsigned)(sms / C * C * minb), 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  e = cudaOccupancyMaxActiveClusters(out, kern, &cfg);
+  if (e != cudaSuccess) return e;
+  if (*out < 1) return cudaErrorInvalidConfiguration;
+  if (dev < kDevices) known[dev].store(*out, std::memory_order_release);
+  return cudaSuccess;
+}
+
 // Launches `kern` with clusters of C CTAs (minb CTAs per SM), as many as fit
 // and are needed for the templates of a, `each` at a time per cluster.
-template <typename K>
-static cudaError_t launch_clusters(K kern, int C, int threads, size_t smem, int minb, int each,
+template <auto kern>
+static cudaError_t launch_clusters(int C, int threads, size_t smem, int minb, int each,
                                    const PlanDev& p, const CorrelateArgs& a, cudaStream_t s) {
-  cudaError_t e = ensure_smem(kern, smem);
+  int clusters = 0;
+  cudaError_t e = resident_clusters<kern>(C, threads, smem, minb, &clusters);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
@@ -284,19 +319,9 @@ static cudaError_t launch_clusters(K kern, int C, int threads, size_t smem, int 
   cfg.blockDim = dim3((unsigned)threads, 1, 1);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
-  int dev = 0, sms = 0;
-  e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e != cudaSuccess) return e;
-  cfg.gridDim = dim3((unsigned)(sms / C * C * minb), 1, 1);
-  int max_clusters = 0;
-  e = cudaOccupancyMaxActiveClusters(&max_clusters, kern, &cfg);
-  if (e != cudaSuccess) return e;
-  if (max_clusters < 1) return cudaErrorInvalidConfiguration;
   int64_t want = (a.k1 - a.k0 + each - 1) / each;
   if (a.max_clusters > 0 && want > a.max_clusters) want = a.max_clusters;
-  if (want > max_clusters) want = max_clusters;
+  if (want > clusters) want = clusters;
   cfg.gridDim = dim3((unsigned)(want * C), 1, 1);
   return cudaLaunchKernelEx(&cfg, kern, p, a);
 }

@@ -1033,8 +1033,8 @@ __global__ void __launch_bounds__(256, 2) short_kernel(PlanDev p, CorrelateArgs 
 template <int S, int U, bool HALFZ, bool EXT>
 static cudaError_t launch_unit_t(const PlanDev& p, const CorrelateArgs& a, cudaStream_t s) {
   constexpr int C = S / 2 / U;
-  return launch_clusters(unit_kernel<S, U, HALFZ, EXT>, C, 256 * U, Lay<kF, U, false>::total,
-                         U == 1 ? 2 : 1, 1, p, a, s);
+  return launch_clusters<unit_kernel<S, U, HALFZ, EXT>>(C, 256 * U, Lay<kF, U, false>::total,
+                                                        U == 1 ? 2 : 1, 1, p, a, s);
 }
 
 // The extended epilogue (bege_correlate_max, bege_correlate_band,
@@ -1056,8 +1056,9 @@ template <int F, bool HALFZ>
 static cudaError_t launch_short(const PlanDev& p, const CorrelateArgs& a, cudaStream_t s) {
   constexpr int U = 4096 / F;
   constexpr size_t smem = Lay<F, U, true>::total;
-  return extended(p, a) ? launch_clusters(short_kernel<F, HALFZ, true>, 1, 256, smem, 2, U, p, a, s)
-                        : launch_clusters(short_kernel<F, HALFZ, false>, 1, 256, smem, 2, U, p, a, s);
+  return extended(p, a)
+             ? launch_clusters<short_kernel<F, HALFZ, true>>(1, 256, smem, 2, U, p, a, s)
+             : launch_clusters<short_kernel<F, HALFZ, false>>(1, 256, smem, 2, U, p, a, s);
 }
 
 }  // namespace unit
