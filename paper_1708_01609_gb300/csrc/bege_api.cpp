@@ -852,7 +852,7 @@ int bege_correlate_multi(bege_ctx* ctx, const int32_t* seg_ids, int32_t n_seg, i
     a.cap[i] = jobs[i]->buf->rec_cap;
     a.counter[i] = static_cast<unsigned long long*>(jobs[i]->buf->counter.ptr);
   }
-  a.scratch = static_cast<float2*>(jobs[0]->scratch.ptr);
+  a.scratch = static_cast<float4*>(jobs[0]->scratch.ptr);
   for (auto& j : jobs)
     if (e == cudaSuccess) e = cudaEventRecord(j->buf->k_start, s);
   if (e == cudaSuccess) e = bege::launch_correlate_multi(segs[0]->plan->dev, a, s);

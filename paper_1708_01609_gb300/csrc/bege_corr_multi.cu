@@ -4,7 +4,10 @@
 // once, keeps its part of the spectrum (32 values per thread) in an
 // L2-resident scratch, and then, for each segment, the product with that
 // segment's coefficients, the inverse transform, sigma and the tails, with
-// exactly the single-segment kernel's arithmetic.
+// exactly the single-segment kernel's arithmetic.  Bound by latency beside the
+// single kernel's FP32 work: a segment begins with 64 KB of spectrum and 48 KB
+// of coefficients per unit from L2, as 16-byte loads (as 8-byte ones 199 ns per
+// correlation at N = 2^16 and M = 8, now 149; the single kernel 171).
 #include "bege_unit.cuh"
 
 namespace bege {
@@ -17,6 +20,7 @@ template <int S, int U>
 __global__ void __launch_bounds__(256 * U, U == 1 ? 2 : 1) correlate_multi_kernel(PlanDev p, MultiArgs a) {
   constexpr int C = S / 2 / U;
   constexpr int kT = Geo<kF>::T;
+  constexpr int kAhead = S <= 4 ? 3 : S == 8 ? 2 : 1;  // the reload has nothing to hide behind
   using SM = Sm<kF, U>;
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = C == 1 ? 0 : (int)cluster.block_rank();
@@ -35,7 +39,7 @@ __global__ void __launch_bounds__(256 * U, U == 1 ? 2 : 1) correlate_multi_kerne
   const int cid = blockIdx.x / C;
   const int ncl = gridDim.x / C;
   const int nz = (int)(a.Lp / 2);
-  float2* const scratch = a.scratch + ((size_t)blockIdx.x * U + ui) * 32 * kT;
+  float4* const scratch = a.scratch + ((size_t)blockIdx.x * U + ui) * 16 * kT;
 
   for (int64_t k = a.k0 + cid; k < a.k1; k += ncl) {
     // S2: forward stages 1-2 (stage 3 runs inside the middle for m = 0)
@@ -47,9 +51,9 @@ __global__ void __launch_bounds__(256 * U, U == 1 ? 2 : 1) correlate_multi_kerne
     for (int m = 0; m < a.M; ++m) {
       // S3-S5 for segment m: product, sigma share, inverse transform
       if (m == 0)
-        middle<SM, 1, true, false>(ui, ug, a.AB[0], a.M > 1 ? scratch : nullptr, false);
+        middle<SM, kAhead, true, false>(ui, ug, a.AB[0], a.M > 1 ? scratch : nullptr, false);
       else  // the rows are rewritten after the cluster's reads
-        middle<SM, 1, true, (C > 1)>(ui, ug, a.AB[m], scratch, true);
+        middle<SM, kAhead, true, (C > 1)>(ui, ug, a.AB[m], scratch, true);
       mid_leave<SM, U>(ui, ug);
       stage2i<SM>(ui);
       SM::sync(ui);
@@ -138,16 +142,19 @@ cudaError_t launch_multi_t(const PlanDev& p, const MultiArgs& a, cudaStream_t s)
 
 }  // namespace
 
-size_t multi_scratch_bytes(int sms) { return (size_t)sms * 2 * 256 * 32 * sizeof(float2); }
+size_t multi_scratch_bytes(int sms) { return (size_t)sms * 2 * 256 * 16 * sizeof(float4); }
 
 cudaError_t launch_correlate_multi(const PlanDev& p, const MultiArgs& a, cudaStream_t s) {
   if (a.k1 <= a.k0 || a.M < 1) return cudaSuccess;
   if (p.g.F != kF || p.g.S < 2 || a.Lp > kF || a.M > kMaxMulti) return cudaErrorInvalidValue;
+  // Units per CTA: one where the reload of the spectrum, not the cluster, is
+  // waited for (8 segments, ns per correlation, one / two units: N = 2^15 64.4 /
+  // 58.5, 2^16 148.6 / 150.5, 2^17 333 / 351).
   switch (p.g.S) {
     case 2: return launch_multi_t<2, 1>(p, a, s);
     case 4: return launch_multi_t<4, 2>(p, a, s);
-    case 8: return launch_multi_t<8, 2>(p, a, s);
-    case 16: return launch_multi_t<16, 2>(p, a, s);
+    case 8: return launch_multi_t<8, 1>(p, a, s);
+    case 16: return launch_multi_t<16, 1>(p, a, s);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -203,7 +203,7 @@ struct MultiArgs {
   bege_tail* recs[kMaxMulti];
   uint64_t cap[kMaxMulti];
   unsigned long long* counter[kMaxMulti];
-  float2* scratch;  // multi_scratch_bytes(): the template spectrum of each CTA
+  float4* scratch;  // multi_scratch_bytes(): the template spectrum of each CTA
 };
 size_t multi_scratch_bytes(int sms);
 cudaError_t launch_correlate_multi(const PlanDev& p, const MultiArgs& a, cudaStream_t s);

@@ -464,12 +464,12 @@ __device__ __forceinline__ void stage3(int ui, const MidItem& m, bool self, floa
 }
 
 // Stage 3, the product with sum |Y|^2, stage 3' of thread t's two
-// butterflies, in place.  MULTI: the spectrum is kept in `scratch` (32 values a
-// thread, stride kT) for the block's other segments, or with `reload` read
+// butterflies, in place.  MULTI: the spectrum is kept in `scratch` (16 float4 a
+// thread, stride T) for the block's other segments, or with `reload` read
 // from there.  AHEAD: pairs of rows whose coefficients are loaded ahead.
 template <class SM, int AHEAD, bool MULTI = false, bool WAIT = false>
 __device__ __forceinline__ void middle(int ui, int ug, const float4* __restrict__ coef,
-                                       float2* __restrict__ scratch = nullptr,
+                                       float4* __restrict__ scratch = nullptr,
                                        bool reload = false) {
   constexpr int kT = SM::G::T;
   const int t = SM::tid();
@@ -491,17 +491,16 @@ __device__ __forceinline__ void middle(int ui, int ug, const float4* __restrict_
   if (MULTI && reload) {
 #pragma unroll
     for (int r = 0; r < 16; ++r) {
-      za[r] = __ldcg(scratch + r * kT + t);
-      zb[r] = __ldcg(scratch + (16 + r) * kT + t);
+      const float4 v = __ldcg(scratch + r * kT + t);
+      za[r] = make_float2(v.x, v.y);
+      zb[r] = make_float2(v.z, v.w);
     }
   } else {
     stage3<SM>(ui, m, self, za, zb);
     if (MULTI && scratch) {
 #pragma unroll
-      for (int r = 0; r < 16; ++r) {
-        __stcg(scratch + r * kT + t, za[r]);
-        __stcg(scratch + (16 + r) * kT + t, zb[r]);
-      }
+      for (int r = 0; r < 16; ++r)
+        __stcg(scratch + r * kT + t, make_float4(za[r].x, za[r].y, zb[r].x, zb[r].y));
     }
   }
   float acc = 0.f;
