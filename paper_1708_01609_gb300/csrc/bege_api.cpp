@@ -79,6 +79,7 @@ struct Bank {
 // jobs (events included: creating three costs more than a small launch).
 struct JobBuffers {
   DevBuf sigma, recs, counter;
+  DevBuf exch;  // exchange buffer of the correlate kernel (may be absent)
   int64_t sigma_cap = 0;
   uint64_t rec_cap = 0;
   cudaEvent_t done = nullptr;
@@ -123,6 +124,7 @@ struct Batch {
 
 struct bege_ctx {
   int device = 0;
+  int sms = 0;
   bege_config cfg{};
   std::mutex mu;
   uint64_t bytes = 0;
@@ -151,7 +153,7 @@ struct bege_ctx {
                                     " bytes exceeds the HBM budget");
     void* p = nullptr;
     cudaError_t e = cudaMalloc(&p, bytes ? bytes : 16);
-    if (e != cudaSuccess && !spare.empty()) {
+    if (e != cudaSuccess) {
       cudaGetLastError();
       drop_spare();
       e = cudaMalloc(&p, bytes ? bytes : 16);
@@ -196,7 +198,26 @@ struct bege_ctx {
     spare.push_back(*b);
     *b = DevBuf{};
   }
+  // Exchange buffers of the correlate kernel (at most 40 MB each) stay with
+  // their job buffers, at most kExchangeBytes in all; idle ones are given back
+  // with the spare buffers.
+  static constexpr uint64_t kExchangeBytes = 160u << 20;
+  uint64_t exchange_bytes = 0;
+  void drop_exchange(JobBuffers* b) {
+    exchange_bytes -= b->exch.bytes;
+    release(&b->exch);
+  }
+  float4* take_exchange(JobBuffers* b, size_t need) {  // b: of a job not launched yet
+    if (need == 0 || cfg.hbm_budget_bytes) return nullptr;
+    if (need > b->exch.bytes) {
+      drop_exchange(b);
+      if (exchange_bytes + need > kExchangeBytes || alloc(&b->exch, need) != BEGE_OK) return nullptr;
+      exchange_bytes += need;
+    }
+    return static_cast<float4*>(b->exch.ptr);
+  }
   void drop_spare() {
+    for (auto& b : pool) drop_exchange(b.get());
     for (DevBuf& b : spare) release(&b);
     spare.clear();
     spare_bytes = 0;
@@ -205,6 +226,7 @@ struct bege_ctx {
     release(&b->sigma);
     release(&b->recs);
     release(&b->counter);
+    drop_exchange(b);
     for (cudaEvent_t e : {b->done, b->k_start, b->k_stop})
       if (e) cudaEventDestroy(e);
     b->done = b->k_start = b->k_stop = nullptr;
@@ -530,6 +552,7 @@ int bege_create(bege_ctx** out, int device, const bege_config* cfg) {
   if (prop.major < 10) return fail(BEGE_ECUDA, "libbege needs an sm_103a (Blackwell) GPU");
   auto* ctx = new bege_ctx();
   ctx->device = device;
+  ctx->sms = prop.multiProcessorCount;
   ctx->cfg = c;
   *out = ctx;
   return BEGE_OK;
@@ -757,6 +780,9 @@ static int correlate_impl(bege_ctx* ctx, int32_t seg_id, int32_t bank_id, int64_
       auto ci = ctx->configs.find(seg->n);
       const bege::CorrConfig cc =
           ci != ctx->configs.end() ? ci->second : bege::default_config(seg->plan->g);
+      // a context with a budget, or a full device, does without
+      a.exch = ctx->take_exchange(job->buf.get(),
+                                  bege::exchange_bytes(seg->plan->g, cc, nsig, ctx->sms));
       e = bege::launch_correlate(seg->plan->dev, a, cc, s);
     }
   }
@@ -1164,6 +1190,11 @@ int64_t bege_segment_length(bege_ctx* ctx, int32_t seg_id) {
 
 namespace bege {
 int ctx_device(const bege_ctx* ctx) { return ctx->device; }
+void ctx_drop_spare(bege_ctx* ctx) {
+  DeviceGuard dg(ctx->device);
+  std::lock_guard<std::mutex> lk(ctx->mu);
+  ctx->drop_spare();
+}
 int64_t bank_count(bege_ctx* ctx, int32_t bank_id) {
   std::lock_guard<std::mutex> lk(ctx->mu);
   auto bi = ctx->banks.find(bank_id);

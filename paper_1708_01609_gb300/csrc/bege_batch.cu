@@ -40,7 +40,7 @@ __device__ __forceinline__ void combine_group(const float2* uc, int grank, float
                                               int64_t krow, const TailOut& out) {
   Combine<S, 1> cb;
   cb.twiddles(uc, grank);
-  cb.template emit<false>(Sm<kF, 1>::rowptr(), uc, grank, thr, tmpl, krow, out, 0.f);
+  cb.template emit<false>(typename Combine<S, 1>::Shared{Sm<kF, 1>::rowptr()}, uc, grank, thr, tmpl, krow, out, 0.f);
 }
 
 // One work item.  The stages do not depend on the column count S = N/8192, so

@@ -90,7 +90,7 @@ __global__ void __launch_bounds__(256 * U, U == 1 ? 2 : 1) correlate_multi_kerne
           __syncthreads();
         const float sigma = sigma_of(SM::sigall(), S / 2, S * 2 * kF);
         if (rank == 0 && threadIdx.x == 0) a.sigma[m][krow] = sigma;
-        cb.template emit<false>(SM::rowptr(), p.uc, rank, a.kappa * sigma, (uint32_t)k, krow, out,
+        cb.template emit<false>(typename Combine<S, U>::Shared{SM::rowptr()}, p.uc, rank, a.kappa * sigma, (uint32_t)k, krow, out,
                                 sigma);
         if constexpr (C > 1) {
           __syncwarp();

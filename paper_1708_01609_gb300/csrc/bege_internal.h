@@ -147,6 +147,8 @@ int set_last_error(int code, const std::string& msg);
 // CUDA device of a context, and the row count of one of its banks (0 if the
 // handle is unknown).
 int ctx_device(const bege_ctx* ctx);
+// Frees the idle buffers that the context keeps for later calls.
+void ctx_drop_spare(bege_ctx* ctx);
 int64_t bank_count(bege_ctx* ctx, int32_t bank_id);
 
 // Stop every serving-form server of a context.
@@ -182,7 +184,12 @@ struct CorrelateArgs {
   unsigned long long* proj = nullptr;  // optional: per-lag maximum over the bank (Eq. Ak)
   float kappa_hi = 0.f;                // optional: tails only below kappa_hi sigma (0 = none)
   uint32_t lag_end = 0xffffffffu;      // optional: tails only at lags < lag_end (overlap-save)
+  float4* exch = nullptr;              // optional: exchange_bytes, for this launch alone
 };
+// Bytes of the buffer through which a correlation of `count` templates in
+// launch shape cfg can exchange its columns on a GPU of `sms` SMs (two
+// templates per resident cluster); 0 where it has no use for one.
+size_t exchange_bytes(const Geometry& g, CorrConfig cfg, int64_t count, int sms);
 cudaError_t launch_correlate(const PlanDev& p, const CorrelateArgs& a, CorrConfig cfg,
                              cudaStream_t s);
 

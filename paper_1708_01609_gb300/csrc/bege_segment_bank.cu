@@ -1,5 +1,7 @@
 // Geometry, plan tables, launch shapes, the segment-spectrum launcher and
 // chirp-bank synthesis.
+#include <algorithm>
+
 #include "bege_unit.cuh"
 
 namespace bege {
@@ -85,6 +87,13 @@ CorrConfig default_config(const Geometry& g) {
   if (g.S == 1) return {1, 256};
   if (g.S == 2) return {2, 256};
   return {4, 512};
+}
+
+size_t exchange_bytes(const Geometry& g, CorrConfig cfg, int64_t count, int sms) {
+  if (g.S < 8 || cfg.nc != 4) return 0;
+  // one CTA of 4 columns per SM: no more than sms / (S / 4) clusters are resident
+  const int64_t clusters = std::min<int64_t>(count, sms / (g.S / 4));
+  return (size_t)clusters * g.S * 4096 * sizeof(float4);
 }
 
 cudaError_t launch_segment(const PlanDev& p, const float* y, float2* D, float4* AB, bool natural,

@@ -466,6 +466,7 @@ int bege_serve_destroy(bege_ctx* ctx, int32_t server_id) {
   // requests still admitted after the last slice (none: the loop drains them)
   for (cudaStream_t st : sv->streams) cudaStreamDestroy(st);
   if (sv->load_stream) cudaStreamDestroy(sv->load_stream);
+  bege::ctx_drop_spare(ctx);
   return BEGE_OK;
 }
 

@@ -84,8 +84,8 @@ struct Lay {
   static constexpr size_t u2 = u1 + G::P * 256 * 8;      // [8][16] float2: stage 2'
   static constexpr size_t ws = u2 + 8 * 16 * 8;          // [16] float2: w_S^q (folded templates)
   static constexpr size_t rowptr = ws + 16 * 8;          // [8] the units' rows in the cluster
-  static constexpr size_t sigall = rowptr + 8 * 8;       // [8] units' shares of sum |Y|^2
-  static constexpr size_t red = sigall + 8 * 4;          // [U][W] warp sums
+  static constexpr size_t sigall = rowptr + 8 * 8;       // [2][8] units' shares of sum |Y|^2
+  static constexpr size_t red = sigall + 2 * 8 * 4;          // [U][W] warp sums
   static constexpr size_t one = align16(red + U * G::W * 4);
   static constexpr size_t units = one + (ONE ? n3 + n2 + n1 : 0);
   // within a unit
@@ -294,10 +294,11 @@ __device__ __forceinline__ void store_blocks(int ui, const float2 (&va)[16 / SM:
 // the columns is zero (nz <= F / 2).  ONE: two columns (S = 2) and nz <= 2 F.
 // Otherwise folded over nfold multiples of F.  WAIT: the cluster's reads of the
 // previous contents of the rows are awaited after the loads and the
-// arithmetic, before the stores.
+// arithmetic, before the stores.  arrive: the cluster's barrier is arrived at
+// there.
 template <class SM, bool HALFZ, bool ONE, bool WAIT>
 __device__ __forceinline__ void stage1(int ui, int S, int ug, const float* __restrict__ src,
-                                       int nz, int nfold) {
+                                       int nz, int nfold, bool arrive = false) {
   constexpr int R = SM::G::R, T = SM::G::T, F = 256 * R;
   const float2* z = reinterpret_cast<const float2*>(src);
   const int t = SM::tid();
@@ -344,6 +345,7 @@ __device__ __forceinline__ void stage1(int ui, int S, int ug, const float* __res
     }
   }
   if constexpr (WAIT) cluster_wait();
+  if (arrive) cluster_arrive();
   store_blocks<SM>(ui, va, vb);
 }
 
@@ -843,11 +845,25 @@ struct Combine {
   static __device__ __forceinline__ int row(int rank, int r) {
     return rank * per + r * (kT * U) + (int)threadIdx.x;
   }
-  static __device__ __forceinline__ int slot(int n1) { return (n1 >> 8) * kBlk + (n1 & 255); }
-  static __device__ __forceinline__ void load(float4* const* rowptr, int at, float2 (&t)[S]) {
+  // Rows of unit u in the cluster's shared memory ...
+  struct Shared {
+    float4* const* rowptr;
+    __device__ __forceinline__ float4 operator()(int u, int n1) const {
+      return rowptr[u][(n1 >> 8) * kBlk + (n1 & 255)];
+    }
+  };
+  // ... or in the exchange buffer.
+  struct Global {
+    const float4* x;
+    __device__ __forceinline__ float4 operator()(int u, int n1) const {
+      return __ldcg(x + u * kF + n1);
+    }
+  };
+  template <class X>
+  static __device__ __forceinline__ void load(const X& x, int n1, float2 (&t)[S]) {
 #pragma unroll
     for (int u = 0; u < S / 2; ++u) {
-      const float4 v = rowptr[u][at];
+      const float4 v = x(u, n1);
       t[u] = make_float2(v.x, v.y);
       t[u == 0 ? S / 2 : S - u] = make_float2(v.z, v.w);
     }
@@ -858,13 +874,13 @@ struct Combine {
 #pragma unroll
       for (int q = 0; q < S / 2; ++q) w[r][q] = __ldg(uc + q * kF + row(rank, r));
   }
-  template <bool EXT>
-  __device__ __forceinline__ void emit(float4* const* rowptr, const float2* __restrict__ uc,
-                                       int rank, float thr, uint32_t tmpl, int64_t krow,
+  template <bool EXT, class X>
+  __device__ __forceinline__ void emit(const X& x, const float2* __restrict__ uc, int rank,
+                                       float thr, uint32_t tmpl, int64_t krow,
                                        const TailOut& a, float sigma) {
     float2 t[R][S];
 #pragma unroll
-    for (int r = 0; r < R; ++r) load(rowptr, slot(row(rank, r)), t[r]);
+    for (int r = 0; r < R; ++r) load(x, row(rank, r), t[r]);
     float big = 0.f;
 #pragma unroll
     for (int r = 0; r < R; ++r) {
@@ -876,11 +892,11 @@ struct Combine {
 #pragma unroll 1
       for (int r = 0; r < R; ++r) {
         const int n1 = row(rank, r);
-        float2 x[S], o[S];
-        load(rowptr, slot(n1), x);
-        dft_row<S, true>(x, [&](int q) { return __ldg(uc + q * kF + n1); });
+        float2 y[S], o[S];
+        load(x, n1, y);
+        dft_row<S, true>(y, [&](int q) { return __ldg(uc + q * kF + n1); });
 #pragma unroll
-        for (int k = 0; k < S; ++k) o[k] = x[rev<S>(k)];
+        for (int k = 0; k < S; ++k) o[k] = y[rev<S>(k)];
         emit_row<S, kF, EXT>(o, n1, S * kF, thr, tmpl, krow, a, sigma);
       }
     }
@@ -979,7 +995,7 @@ __global__ void __launch_bounds__(256 * U, U == 1 ? 2 : 1) unit_kernel(PlanDev p
       __syncthreads();
     const float sigma = sigma_of(SM::sigall(), S / 2, S * 2 * kF);
     if (rank == 0 && threadIdx.x == 0) a.sigma[krow] = sigma;
-    cb.template emit<EXT>(SM::rowptr(), p.uc, rank, a.kappa * sigma, (uint32_t)k, krow, out, sigma);
+    cb.template emit<EXT>(typename Combine<S, U>::Shared{SM::rowptr()}, p.uc, rank, a.kappa * sigma, (uint32_t)k, krow, out, sigma);
     if constexpr (C > 1) {
       __syncwarp();
       cluster_arrive_relaxed();  // every remote value has fed a vote: the reads are done
@@ -988,6 +1004,81 @@ __global__ void __launch_bounds__(256 * U, U == 1 ? 2 : 1) unit_kernel(PlanDev p
     }
   }
   if constexpr (C > 1) cluster_wait();  // the cluster's last reads of this CTA's rows
+}
+
+// The same for S >= 8 with the columns exchanged through the buffer a.exch
+// (L2) and the combine one template behind: a CTA writes its units' outputs
+// of template k, goes on with template k + 1 and combines k just before it
+// writes k + 1, so the cluster's barrier (arrive in stage 1, wait before the
+// combine) has most of a template's time to complete and nothing waits for a
+// neighbour's pace or for distributed shared memory.  The buffer holds two
+// templates of every unit: outputs of template k overwrite those of k - 2,
+// which every CTA combined before it arrived for k - 1.  Per template, this /
+// unit_kernel: N = 2^16 166 / 171 ns, 2^17 351 / 405 (at N = 2^15, one CTA a
+// template, 82 / 76).
+template <int S, int U, bool HALFZ, bool EXT>
+__global__ void __launch_bounds__(256 * U, U == 1 ? 2 : 1)
+unit_exchange_kernel(PlanDev p, CorrelateArgs a) {
+  constexpr int C = S / 2 / U;
+  static_assert(C > 1, "a cluster shares the template");
+  using SM = Sm<kF, U>;
+  using CB = Combine<S, U>;
+  cg::cluster_group cluster = cg::this_cluster();
+  const int rank = (int)cluster.block_rank();
+  const int ui = U == 1 ? 0 : (int)threadIdx.x / SM::G::T;
+  const int ug = rank * U + ui;
+  setup_common<SM, 256 * U>(p);
+  setup_unit<SM>(p, S, ug, ui);
+  __syncthreads();
+
+  const int cid = blockIdx.x / C, ncl = gridDim.x / C;
+  const int nz = (int)(a.Lp / 2), nfold = (nz + kF - 1) / kF;
+  const TailOut out{a.recs, a.cap, a.counter, a.dump, a.proj, a.kappa_hi, a.lag_end};
+  float4* const exch = a.exch + (size_t)cid * (S * kF);
+  int par = 0;
+  auto combine = [&](int64_t k) {  // of the template before, which is in buffer par ^ 1
+    CB cb;
+    cb.twiddles(p.uc, rank);
+    cluster_wait();  // every row and share of the cluster is there
+    const float sigma = sigma_of(SM::sigall() + 8 * (par ^ 1), S / 2, S * 2 * kF);
+    const int64_t krow = k - a.k0;
+    if (rank == 0 && threadIdx.x == 0) a.sigma[krow] = sigma;
+    cb.template emit<EXT>(typename CB::Global{exch + (par ^ 1) * (S / 2 * kF)}, p.uc, rank,
+                          a.kappa * sigma, (uint32_t)k, krow, out, sigma);
+  };
+  const int64_t first = a.k0 + cid;
+  int64_t k = first;
+  for (; k < a.k1; k += ncl) {
+    stage1<SM, HALFZ, false, false>(ui, S, ug, a.bank + k * a.Lp, nz, nfold, k != first);
+    SM::sync(ui);
+    stage2<SM>(ui);
+    mid_enter<SM, U>(ui, ug);
+    middle<SM, 1>(ui, ug, a.AB);
+    mid_leave<SM, U>(ui, ug);
+    stage2i<SM>(ui);
+    SM::sync(ui);
+    if (k != first) combine(k - ncl);
+    {
+      float2 va[1][16], vb[1][16];
+      stage1i<SM>(ui, va, vb);
+      float4* x = exch + (par * (S / 2) + ug) * kF + SM::tid();
+#pragma unroll
+      for (int q = 0; q < 16; ++q)
+        __stcg(x + 256 * q, make_float4(va[0][rev<16>(q)].x, va[0][rev<16>(q)].y,
+                                        vb[0][rev<16>(q)].x, vb[0][rev<16>(q)].y));
+    }
+    if (SM::tid() == 0) {
+      const float share = unit_power<SM>(ui);
+#pragma unroll
+      for (int q = 0; q < C; ++q)
+        *cluster.map_shared_rank(SM::sigall() + 8 * par + ug, (unsigned)q) = share;
+    }
+    par ^= 1;
+  }
+  if (k != first) {
+    cluster_arrive();
+    combine(k - ncl);
+  }
 }
 
 // S = 2: the units of a CTA (256 threads) take templates of their own and wait
@@ -1032,6 +1123,11 @@ __global__ void __launch_bounds__(256, 2) short_kernel(PlanDev p, CorrelateArgs 
 template <int S, int U, bool HALFZ, bool EXT>
 static cudaError_t launch_unit_t(const PlanDev& p, const CorrelateArgs& a, cudaStream_t s) {
   constexpr int C = S / 2 / U;
+  if constexpr (S >= 8 && U == 2) {
+    if (a.exch)
+      return launch_clusters<unit_exchange_kernel<S, U, HALFZ, EXT>>(
+          C, 256 * U, Lay<kF, U, false>::total, 1, 1, p, a, s);
+  }
   return launch_clusters<unit_kernel<S, U, HALFZ, EXT>>(C, 256 * U, Lay<kF, U, false>::total,
                                                         U == 1 ? 2 : 1, 1, p, a, s);
 }

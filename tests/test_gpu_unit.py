@@ -81,3 +81,32 @@ def test_coefficients_and_tables_at_a_quarter_turn(ctx):
         ctx.bege_release(seg)
         assert np.abs(dump - y).max() <= 2e-6, j
     ctx.bege_release(bid)
+
+
+@pytest.mark.parametrize("n,length", [(1 << 16, 4096), (1 << 17, 4096), (1 << 17, 5000)])
+def test_exchange_through_l2_equals_shared_memory(ctx, n, length):
+    """N >= 2^16 exchanges columns through a buffer one template behind; a
+    context with a budget does without it.  Same bits, over several templates
+    per cluster and a last round that not every cluster takes part in."""
+    count = 401
+    bank = S.random_samples_bank(count, length, n + length)
+    y = S.band_limited_noise(n, 5)
+    got = []
+    small = make_ctx(hbm_budget_bytes=1 << 30)
+    for c in (ctx, small):
+        seg, bid = c.bege_load_segment(y), c.bege_define_bank_samples(bank)
+        c.bege_set_config(n, 4, 512)
+        for k0, k1 in ((0, count), (7, 8)):
+            job = c.bege_correlate(seg, bid, k0, k1, 3.5)
+            recs, total = c.bege_fetch_tails(job, sort=True)
+            assert total == len(recs) > 0
+            got.append((recs.copy(), c.bege_get_sigma(job, k1 - k0)))
+            c.bege_release(job)
+        c.bege_release(seg)
+        c.bege_release(bid)
+    small.close()
+    for a, b in zip(got[:2], got[2:]):
+        assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
+    all_, one = got[0], got[1]
+    assert one[1][0] == all_[1][7]
+    assert np.array_equal(one[0], all_[0][all_[0]["tmpl"] == 7])
