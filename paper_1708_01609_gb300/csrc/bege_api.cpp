@@ -207,9 +207,17 @@ struct bege_ctx {
     exchange_bytes -= b->exch.bytes;
     release(&b->exch);
   }
-  float4* take_exchange(JobBuffers* b, size_t need) {  // b: of a job not launched yet
+  // b: of a job not launched yet, on stream s (whose capture, if one is going
+  // on, an allocation would end)
+  float4* take_exchange(JobBuffers* b, size_t need, cudaStream_t s) {
     if (need == 0 || cfg.hbm_budget_bytes) return nullptr;
     if (need > b->exch.bytes) {
+      cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+      if (cudaStreamIsCapturing(s, &capture) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+      }
+      if (capture != cudaStreamCaptureStatusNone) return nullptr;
       drop_exchange(b);
       if (exchange_bytes + need > kExchangeBytes || alloc(&b->exch, need) != BEGE_OK) return nullptr;
       exchange_bytes += need;
@@ -782,7 +790,7 @@ static int correlate_impl(bege_ctx* ctx, int32_t seg_id, int32_t bank_id, int64_
           ci != ctx->configs.end() ? ci->second : bege::default_config(seg->plan->g);
       // a context with a budget, or a full device, does without
       a.exch = ctx->take_exchange(job->buf.get(),
-                                  bege::exchange_bytes(seg->plan->g, cc, nsig, ctx->sms));
+                                  bege::exchange_bytes(seg->plan->g, cc, nsig, ctx->sms), s);
       e = bege::launch_correlate(seg->plan->dev, a, cc, s);
     }
   }

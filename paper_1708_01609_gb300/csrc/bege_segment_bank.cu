@@ -82,7 +82,8 @@ bool config_valid(const Geometry& g, CorrConfig c) {
 // SM, so half as many CTAs meet in a cluster and a unit's neighbour in the
 // CTA needs no distributed shared memory; S = 2 has one unit a template and
 // two CTAs per SM.  Per template (65536 chirps, GB300), 4 x 512 against 2 x
-// 256: N = 2^15 75.7 / 81.9 ns, 2^16 170.7 / 188.8, 2^17 405 / 411.
+// 256: N = 2^15 75.7 / 81.9 ns, 2^16 170.7 / 188.8, 2^17 405 / 411 (and 165 and
+// 354 with the exchange through L2, which takes this shape).
 CorrConfig default_config(const Geometry& g) {
   if (g.S == 1) return {1, 256};
   if (g.S == 2) return {2, 256};
@@ -185,7 +186,7 @@ __device__ __forceinline__ void chirp_samples(unsigned long long alpha, unsigned
 // up to 4096 samples are evaluated once and kept in registers between the
 // norm and the store; a sample costs two complex products and its share of
 // the start values, about 14 FP64 instructions, where two evaluations of sinpi
-// took about 60.
+// took about 60 (2^20 rows of 4096 samples: 415 -> 148 ms).
 __global__ void __launch_bounds__(kChirpThreads)
 bank_chirp_kernel(const unsigned long long* __restrict__ ab, int64_t L, int64_t Lp, double frac,
                   bool symmetric, float* __restrict__ bank) {

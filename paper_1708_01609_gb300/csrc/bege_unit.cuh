@@ -42,19 +42,19 @@
 // writes 16 consecutive values of one column as 8 16-byte accesses, free of
 // bank conflicts, and its mirror butterfly in the other column likewise.
 //
-// Bound: FP32 issue and shared-memory bandwidth (FFT butterflies), not HBM:
-// at N = 2^16 a correlation issues 110e3 warp instructions (91e3 of them on
-// the FMA pipe) and moves 23.5e3 shared-memory wavefronts, 50% and 39% of
-// what its time allows; what is left is latency (L2 coefficients, the
-// cluster's barrier) with 16 warps per SM, all that 128 registers a thread
-// allow.  Per template of 1 s, against Stockham passes with plain twiddle
-// products and ten CTA barriers a template (65536 chirps, GB300): N = 2^14
-// 49.6 -> 35.2 ns, 2^15 102 -> 75.7, 2^16 216 -> 171, 2^17 473 -> 405.
+// Bound: FP32 issue and shared-memory bandwidth (FFT butterflies), not HBM: at
+// N = 2^16 a correlation issues 108.6e3 warp instructions (91e3 of them on the
+// FMA pipe) and moves 20e3 shared-memory wavefronts, 52% and 37% of what its
+// time allows (at N = 2^14 59% and 42%); what is left is latency (barriers, L2
+// coefficients) with 16 warps per SM, all that 128 registers a thread allow.
+// Per template of 1 s, against Stockham passes with plain twiddle products and
+// ten CTA barriers a template (65536 chirps, GB300): N = 2^14 49.6 -> 35.0 ns,
+// 2^15 102 -> 78, 2^16 216 -> 165, 2^17 472 -> 354.
 // Measured beside it and not kept: packed FP32 pairs (an FFMA2 takes the FMA
 // pipe 2.2 to 2.5 cycles, no less than two FFMAs); columns of 2048 points with
 // 128-thread units (183 ns at 2^16, 41 at 2^14); stage 1' storing straight
 // into the CTA that combines (209 ns against 191 for reading there, with
-// clusters of four).
+// clusters of four); one column's butterflies after the other's (level).
 #pragma once
 
 #include "bege_corr.cuh"
