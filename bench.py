@@ -243,7 +243,8 @@ def run_reference(args):
 # our arm
 # ---------------------------------------------------------------------------
 # the sources the N = 2^16 FP32 correlate kernel is compiled from
-CORRELATE_SOURCES = ("bege_corr.cuh", "bege_fft.cuh", "bege_corr_s8.cu", "bege_internal.h")
+CORRELATE_SOURCES = ("bege_corr.cuh", "bege_fft.cuh", "bege_unit.cuh", "bege_corr_s8.cu",
+                     "bege_internal.h")
 
 
 def correlate_source_hash() -> str:
@@ -389,7 +390,7 @@ def run_ours(args):
         "roofline": {
             "bound": "alu", "achieved": achieved / 1e12, "peak": peak / 1e12, "unit": "TFLOP/s",
             "frac": achieved / peak, "traffic": traffic,
-            "kernel": "correlate_kernel<4096,8,2,256>", "kernel_ms": kernel_ms,
+            "kernel": "unit_exchange_kernel<8,2>", "kernel_ms": kernel_ms,
             "flops_per_launch": flops_launch,
             "peak_basis": (f"FP32 ALU: {props.multi_processor_count} SMs x 128 lanes x 2 flops x "
                            f"{sm_max:.0f} MHz (max SM clock of MEASURED_PEAKS.json)"),
