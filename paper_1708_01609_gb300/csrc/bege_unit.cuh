@@ -1029,6 +1029,10 @@ unit_exchange_kernel(PlanDev p, CorrelateArgs a) {
   const int ug = rank * U + ui;
   setup_common<SM, 256 * U>(p);
   setup_unit<SM>(p, S, ug, ui);
+  // the first template's share goes into the other CTAs' shared memory: all of
+  // them have started once the wait that pairs with this (before the first
+  // store) returns
+  cluster_arrive();
   __syncthreads();
 
   const int cid = blockIdx.x / C, ncl = gridDim.x / C;
@@ -1057,7 +1061,10 @@ unit_exchange_kernel(PlanDev p, CorrelateArgs a) {
     mid_leave<SM, U>(ui, ug);
     stage2i<SM>(ui);
     SM::sync(ui);
-    if (k != first) combine(k - ncl);
+    if (k != first)
+      combine(k - ncl);
+    else
+      cluster_wait();
     {
       float2 va[1][16], vb[1][16];
       stage1i<SM>(ui, va, vb);
