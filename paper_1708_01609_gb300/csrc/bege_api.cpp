@@ -6,6 +6,7 @@
 #include <algorithm>
 #include <atomic>
 #include <cmath>
+#include <cstdint>
 #include <cstdio>
 #include <cstring>
 #include <map>
@@ -79,7 +80,7 @@ struct Bank {
 // jobs (events included: creating three costs more than a small launch).
 struct JobBuffers {
   DevBuf sigma, recs, counter;
-  DevBuf exch;  // exchange buffer of the correlate kernel (may be absent)
+  DevBuf exch;  // exchange buffer of the job's correlate kernel (may be absent)
   int64_t sigma_cap = 0;
   uint64_t rec_cap = 0;
   cudaEvent_t done = nullptr;
@@ -169,6 +170,7 @@ struct bege_ctx {
   }
   void release(DevBuf* b) {
     if (b->ptr) {
+      exchange_refused = SIZE_MAX;
       cudaFree(b->ptr);
       bytes -= b->bytes;
     }
@@ -198,34 +200,66 @@ struct bege_ctx {
     spare.push_back(*b);
     *b = DevBuf{};
   }
-  // Exchange buffers of the correlate kernel (at most 40 MB each) stay with
-  // their job buffers, at most kExchangeBytes in all; idle ones are given back
-  // with the spare buffers.
+  // Exchange buffers of the correlate kernel (at most 40 MB each) belong to a
+  // job from its launch to its release and are idle between jobs, for
+  // whichever comes next: as many exist as jobs were ever held at once, at
+  // most kExchangeBytes in all, and idle ones are given back with the spare
+  // buffers.  A size that the device refused is not asked for again before
+  // the context has given memory back.
   static constexpr uint64_t kExchangeBytes = 160u << 20;
-  uint64_t exchange_bytes = 0;
-  void drop_exchange(JobBuffers* b) {
-    exchange_bytes -= b->exch.bytes;
-    release(&b->exch);
+  std::vector<DevBuf> idle_exchange;
+  uint64_t exchange_bytes = 0;  // idle and in use
+  size_t exchange_refused = SIZE_MAX;
+  void drop_exchange(DevBuf* b) {
+    exchange_bytes -= b->bytes;
+    release(b);
   }
-  // b: of a job not launched yet, on stream s (whose capture, if one is going
-  // on, an allocation would end)
+  // b: of a job not launched yet, on stream s.  Null under capture: the
+  // allocation would end it, and its graph may run after the job's release.
   float4* take_exchange(JobBuffers* b, size_t need, cudaStream_t s) {
     if (need == 0 || cfg.hbm_budget_bytes) return nullptr;
-    if (need > b->exch.bytes) {
-      cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-      if (cudaStreamIsCapturing(s, &capture) != cudaSuccess) {
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &capture) != cudaSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
+    if (capture != cudaStreamCaptureStatusNone) return nullptr;
+    auto best = idle_exchange.end();
+    uint64_t idle = 0;
+    for (auto i = idle_exchange.begin(); i != idle_exchange.end(); ++i) {
+      idle += i->bytes;
+      if (i->bytes >= need && (best == idle_exchange.end() || i->bytes < best->bytes)) best = i;
+    }
+    if (best != idle_exchange.end()) {
+      b->exch = *best;
+      idle_exchange.erase(best);
+    } else {
+      if (need >= exchange_refused || exchange_bytes - idle + need > kExchangeBytes) return nullptr;
+      while (exchange_bytes + need > kExchangeBytes) {  // the idle ones are too small
+        drop_exchange(&idle_exchange.back());
+        idle_exchange.pop_back();
+      }
+      void* p = nullptr;
+      if (cudaMalloc(&p, need) != cudaSuccess) {
         cudaGetLastError();
+        exchange_refused = need;
         return nullptr;
       }
-      if (capture != cudaStreamCaptureStatusNone) return nullptr;
-      drop_exchange(b);
-      if (exchange_bytes + need > kExchangeBytes || alloc(&b->exch, need) != BEGE_OK) return nullptr;
+      b->exch = {p, need};
+      this->bytes += need;
       exchange_bytes += need;
     }
     return static_cast<float4*>(b->exch.ptr);
   }
+  // b: of a finished job
+  void give_back(std::unique_ptr<JobBuffers> b) {
+    if (b->exch.ptr) idle_exchange.push_back(b->exch);
+    b->exch = DevBuf{};
+    pool.push_back(std::move(b));
+  }
   void drop_spare() {
-    for (auto& b : pool) drop_exchange(b.get());
+    for (DevBuf& b : idle_exchange) drop_exchange(&b);
+    idle_exchange.clear();
     for (DevBuf& b : spare) release(&b);
     spare.clear();
     spare_bytes = 0;
@@ -234,7 +268,7 @@ struct bege_ctx {
     release(&b->sigma);
     release(&b->recs);
     release(&b->counter);
-    drop_exchange(b);
+    drop_exchange(&b->exch);
     for (cudaEvent_t e : {b->done, b->k_start, b->k_stop})
       if (e) cudaEventDestroy(e);
     b->done = b->k_start = b->k_stop = nullptr;
@@ -798,6 +832,7 @@ static int correlate_impl(bege_ctx* ctx, int32_t seg_id, int32_t bank_id, int64_
   if (e == cudaSuccess) e = cudaEventRecord(job->buf->done, s);
   if (e != cudaSuccess) {
     ctx->release(&job->proj);
+    ctx->drop_exchange(&job->buf->exch);  // waits for a kernel that may use it
     ctx->pool.push_back(std::move(job->buf));
     return cuda_fail(e, "correlate");
   }
@@ -1071,7 +1106,7 @@ int bege_dump_correlation(bege_ctx* ctx, int32_t seg_id, int32_t bank_id, int64_
   ctx->release(&d);
   Job* j = find_job(ctx, job);
   if (j) {
-    ctx->pool.push_back(std::move(j->buf));
+    ctx->give_back(std::move(j->buf));
     ctx->jobs.erase(job);
   }
   if (e != cudaSuccess) return cuda_fail(e, "dump");
@@ -1138,7 +1173,7 @@ int bege_autotune(bege_ctx* ctx, int32_t seg_id, int32_t bank_id, int64_t k_begi
       float ms = 0.f;
       cudaError_t e = cudaEventSynchronize(j->buf->done);
       if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, j->buf->k_start, j->buf->k_stop);
-        ctx->pool.push_back(std::move(j->buf));
+      ctx->give_back(std::move(j->buf));
       ctx->jobs.erase(job);
       if (e != cudaSuccess) return cuda_fail(e, "autotune");
       if (r > 0) t.push_back(ms);
@@ -1488,7 +1523,7 @@ int bege_release(bege_ctx* ctx, int32_t handle) {
     cudaEventSynchronize(ji->second->buf->done);
     ctx->release(&ji->second->proj);
     ctx->release(&ji->second->scratch);
-    ctx->pool.push_back(std::move(ji->second->buf));
+    ctx->give_back(std::move(ji->second->buf));
     ctx->jobs.erase(ji);
     return BEGE_OK;
   }
