@@ -395,6 +395,12 @@ int wait_counted(Job* j) {
   return BEGE_OK;
 }
 
+// Waits for a job that is let go.  The event of one enqueued under capture
+// cannot be waited for, and that refusal is no error of the launches to come.
+void wait_done(Job* j) {
+  if (cudaEventSynchronize(j->buf->done) != cudaSuccess) cudaGetLastError();
+}
+
 Job* find_job(bege_ctx* ctx, int32_t id) {
   auto it = ctx->jobs.find(id);
   return it == ctx->jobs.end() ? nullptr : it->second.get();
@@ -607,7 +613,7 @@ int bege_destroy(bege_ctx* ctx) {
     DeviceGuard dg(ctx->device);
     std::lock_guard<std::mutex> lk(ctx->mu);
     for (auto& kv : ctx->jobs) {
-      cudaEventSynchronize(kv.second->buf->done);
+      wait_done(kv.second.get());
       ctx->release(&kv.second->proj);
       ctx->release(&kv.second->scratch);
       ctx->free_buffers(kv.second->buf.get());
@@ -1520,7 +1526,7 @@ int bege_release(bege_ctx* ctx, int32_t handle) {
   std::lock_guard<std::mutex> lk(ctx->mu);
   auto ji = ctx->jobs.find(handle);
   if (ji != ctx->jobs.end()) {
-    cudaEventSynchronize(ji->second->buf->done);
+    wait_done(ji->second.get());
     ctx->release(&ji->second->proj);
     ctx->release(&ji->second->scratch);
     ctx->give_back(std::move(ji->second->buf));
@@ -1538,7 +1544,7 @@ int bege_release(bege_ctx* ctx, int32_t handle) {
     // what may still use the segment: its own kernel, jobs not released yet
     if (!si->second->loaded) cudaDeviceSynchronize();
     for (auto& kv : ctx->jobs)
-      if (kv.second->seg == handle) cudaEventSynchronize(kv.second->buf->done);
+      if (kv.second->seg == handle) wait_done(kv.second.get());
     ctx->keep(&si->second->D);
     ctx->keep(&si->second->AB);
     ctx->segs.erase(si);

@@ -1,4 +1,5 @@
 """What a context keeps between calls."""
+import numpy as np
 import pytest
 
 import synthetic as S
@@ -25,3 +26,34 @@ def test_sequential_searches_share_one_exchange_buffer():
             held.append(ctx.bege_device_bytes() - before)
         assert 0 < held[0] <= 40 << 20
         assert held == held[:1] * 8
+
+
+@pytest.mark.parametrize("idle_buffer", [False, True])
+def test_capture_of_a_search_allocates_nothing(idle_buffer):
+    """A search enqueued on a stream under capture takes no exchange buffer,
+    new or idle, and leaves the capture valid; the graph runs, and later
+    searches are as ever."""
+    torch = pytest.importorskip("torch")
+    n = 1 << 16
+    with make_ctx(tail_capacity=1 << 12) as ctx:
+        bank = ctx.bege_define_bank_samples(S.random_samples_bank(20, 64, 1))
+        seg = ctx.bege_load_segment(S.band_limited_noise(n, 1))
+        if not idle_buffer:
+            ctx.bege_set_config(n, 2, 256)      # this shape has no use for one
+        job = ctx.bege_correlate(seg, bank, 0, 20, 5.0)
+        want = ctx.bege_get_sigma(job, 20)
+        ctx.bege_release(job)
+        ctx.bege_set_config(n, 4, 512)
+        held = ctx.bege_device_bytes()
+        graph, stream = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+        with torch.cuda.graph(graph, stream=stream):
+            job = ctx.bege_correlate(seg, bank, 0, 20, 5.0, stream.cuda_stream)
+        assert ctx.bege_device_bytes() == held
+        for _ in range(2):
+            graph.replay()
+        torch.cuda.synchronize()
+        second = ctx.bege_correlate(seg, bank, 0, 20, 5.0)
+        assert np.array_equal(ctx.bege_get_sigma(second, 20), want)
+        del graph
+        for h in (second, job, seg, bank):
+            ctx.bege_release(h)
