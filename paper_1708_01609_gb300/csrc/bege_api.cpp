@@ -801,6 +801,15 @@ static int correlate_impl(bege_ctx* ctx, int32_t seg_id, int32_t bank_id, int64_
   cudaError_t e = cudaSuccess;
   if (project) e = cudaMemsetAsync(job->proj.ptr, 0, job->proj.bytes, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(job->buf->counter.ptr, 0, 16, s);
+  auto ci = ctx->configs.find(seg->n);
+  const bege::CorrConfig cc =
+      ci != ctx->configs.end() ? ci->second : bege::default_config(seg->plan->g);
+  // a context with a budget, or a full device, does without; ahead of the
+  // event, for an idle stream passes it while the call still allocates
+  float4* exch = nullptr;
+  if (e == cudaSuccess && ctx->cfg.precision == 0)
+    exch = ctx->take_exchange(job->buf.get(),
+                              bege::exchange_bytes(seg->plan->g, cc, nsig, ctx->sms), s);
   if (e == cudaSuccess) e = cudaEventRecord(job->buf->k_start, s);
   if (e == cudaSuccess) {
     bege::CorrelateArgs a{};
@@ -819,18 +828,13 @@ static int correlate_impl(bege_ctx* ctx, int32_t seg_id, int32_t bank_id, int64_
     a.status = reinterpret_cast<unsigned int*>(static_cast<char*>(job->buf->counter.ptr) + 8);
     a.proj = static_cast<unsigned long long*>(job->proj.ptr);
     a.kappa_hi = kappa_hi;
+    a.exch = exch;
     // overlap-save: the window y[n .. n+L-1] of a length-L template stays
     // inside the segment for n <= N - L
     if (linear) a.lag_end = (uint32_t)(seg->n - bank->L + 1);
     if (ctx->cfg.precision != 0) {
       e = bege::launch_correlate_tc(seg->plan->dev, a, ctx->cfg.precision, s);
     } else {
-      auto ci = ctx->configs.find(seg->n);
-      const bege::CorrConfig cc =
-          ci != ctx->configs.end() ? ci->second : bege::default_config(seg->plan->g);
-      // a context with a budget, or a full device, does without
-      a.exch = ctx->take_exchange(job->buf.get(),
-                                  bege::exchange_bytes(seg->plan->g, cc, nsig, ctx->sms), s);
       e = bege::launch_correlate(seg->plan->dev, a, cc, s);
     }
   }
