@@ -425,12 +425,13 @@ BEGE_API int bege_serve_destroy(bege_ctx* ctx, int32_t server_id);
  *                   the first tail_capacity records are stored)
  *   stream          cudaStream_t as void*; the call only enqueues work
  *
- * The first call on a device looks up the scratch array's device address
- * (with that device current), so the first call on each device should come
- * before any stream capture.  Every call recomputes the twiddle tables for
- * its n in the scratch array on `stream`, ahead of its other kernels.  The scratch array keeps the last
- * call's contents and is shared by all calls on a device: calls whose work
- * overlaps on the GPU race and must be serialised by the caller.  Errors:
+ * The call uses the scratch array of the current CUDA context.  The first call
+ * in a context loads the library's code there, so it should come before any
+ * stream capture.  Every call recomputes the twiddle tables for its n in the
+ * scratch array on `stream`, ahead of its other kernels.  The scratch array
+ * keeps the last call's contents and is shared by all calls in a context:
+ * calls whose work overlaps on the GPU race and must be serialised by the
+ * caller.  Errors:
  * EINVAL (sizes, alignment, NULL), ECUDA. */
 BEGE_API int bege_search_noalloc(const float* strain_dev, int64_t n, const float* bank_dev,
                                  int64_t ld, int64_t k_begin, int64_t k_end, float kappa,

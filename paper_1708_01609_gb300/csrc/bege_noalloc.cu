@@ -13,8 +13,8 @@
 //   - the FP32 twiddle tables for that N (computed on the device in FP64
 //     by every call, ahead of the call's own kernels on its stream, so no
 //     call depends on what an earlier call left in the array).
-// The array lives on every GPU that loads the library until the process
-// exits (about 1.2 MiB).  All calls on a device share it and it keeps the
+// Every CUDA context that loads the library has such an array until it ends
+// (about 1.2 MiB).  All calls in a context share it and it keeps the
 // contents of the last call, so two calls whose work overlaps on the GPU
 // (for example on two streams) corrupt each other; callers serialise them.
 #include <mutex>
@@ -40,11 +40,8 @@ constexpr size_t kScratchBytes = kOffTables + al256(plan_floats2(kMaxGeometry) *
 
 static __device__ __align__(256) unsigned char g_search_scratch[kScratchBytes];
 
-// Per-device set-up: the device address of the scratch array, looked up once
-// per device with that device current.
-constexpr int kMaxDevices = 64;
+// Held while one call enqueues its kernels.
 std::mutex g_mu;
-unsigned char* g_addr[kMaxDevices] = {};
 
 }  // namespace
 
@@ -74,25 +71,16 @@ extern "C" int bege_search_noalloc(const float* strain_dev, int64_t n, const flo
       reinterpret_cast<uintptr_t>(sigma_dev) % 4 || reinterpret_cast<uintptr_t>(tails_dev) % 4)
     return set_last_error(BEGE_EINVAL, "bege_search_noalloc: misaligned buffer");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return set_last_error(BEGE_ECUDA, cudaGetErrorString(e));
-  if (dev < 0 || dev >= kMaxDevices)
-    return set_last_error(BEGE_EINVAL, "bege_search_noalloc: device index too large");
-
   const Geometry g = make_geometry(n);
-  unsigned char* base = nullptr;
   {
     std::lock_guard<std::mutex> lk(g_mu);
-    if (!g_addr[dev]) {
-      void* p = nullptr;
-      e = cudaGetSymbolAddress(&p, g_search_scratch);
-      if (e != cudaSuccess)
-        return set_last_error(BEGE_ECUDA, std::string("cudaGetSymbolAddress: ") +
-                                              cudaGetErrorString(e));
-      g_addr[dev] = static_cast<unsigned char*>(p);
-    }
-    base = g_addr[dev];
+    // every CUDA context has a scratch array of its own: the current one's
+    void* scratch = nullptr;
+    cudaError_t e = cudaGetSymbolAddress(&scratch, g_search_scratch);
+    if (e != cudaSuccess)
+      return set_last_error(BEGE_ECUDA,
+                            std::string("cudaGetSymbolAddress: ") + cudaGetErrorString(e));
+    unsigned char* const base = static_cast<unsigned char*>(scratch);
     // The tables are rebuilt on every call, in stream order before this
     // call's kernels: the host keeps no record of which n the array holds,
     // which could disagree with the device's order of work.
