@@ -22,6 +22,10 @@
  *     that return results to host memory synchronise on the job themselves.
  *   - Lags are circular indices 0..N-1.  Template indices are bank rows.
  *   - Sizes: N is a power of two in [2^10, 2^17]; 1 <= L <= min(N, 2^16).
+ *   - Range: FP32.  A template whose sigma_k is finite has the results of its
+ *     exact spectra rounded, whatever the scale of strain and template; one
+ *     whose sum of squares leaves the FP32 range (|rho_k| beyond about 1e19)
+ *     has no finite sigma, no tails, and no defined bege_dump_correlation.
  *   - Device: one context drives one GPU (sm_103a).  No CPU fallback exists:
  *     if no usable GPU is present bege_create fails with BEGE_ECUDA.
  */

@@ -74,6 +74,7 @@ struct Segment {
 struct Bank {
   int64_t count = 0, L = 0, Lp = 0;
   DevBuf w;
+  bool large = false;  // holds a sample above bege::kLargeSample
 };
 
 // What a job needs beside its segment and bank; kept by the context between
@@ -104,6 +105,7 @@ struct BatchEntryHost {
   int32_t bank = -1;
   int64_t k0 = 0, k1 = 0;
   float kappa = 0.f;
+  bool large = false;  // of its bank
 };
 
 struct Batch {
@@ -505,31 +507,29 @@ static int batch_build(bege_ctx* ctx, Batch* b) {
     e = bege::launch_segment_batch(b->args, static_cast<const bege::SegJob*>(b->jobs.ptr),
                                    b->n_jobs, b->cs);
   if (e == cudaSuccess) {
-    if (b->plan == 0) {
-      e = bege::launch_batch(b->args, std::min(clusters, b->n_items), b->cs);
-    } else {
-      for (size_t i = 0; i < b->entries.size() && e == cudaSuccess; ++i) {
-        const auto& en = b->entries[i];
-        const auto& sg = b->segs_host[i];
-        auto pl = ctx->plans[en.n];
-        auto ci = ctx->configs.find(en.n);
-        const bege::CorrConfig cc =
-            ci != ctx->configs.end() ? ci->second : bege::default_config(pl->g);
-        bege::CorrelateArgs a{};
-        a.AB = sg.AB;
-        a.bank = sg.bank;
-        a.Lp = sg.Lp;
-        a.k0 = sg.k0;
-        a.k1 = sg.k1;
-        a.kappa = sg.kappa;
-        a.sigma = sg.sigma;
-        a.recs = sg.recs;
-        a.cap = sg.cap;
-        a.counter = sg.counter;
-        a.dump = nullptr;
-        a.max_clusters = 0;
-        e = bege::launch_correlate(pl->dev, a, cc, b->cs);
-      }
+    if (b->plan == 0) e = bege::launch_batch(b->args, std::min(clusters, b->n_items), b->cs);
+    for (size_t i = 0; i < b->entries.size() && e == cudaSuccess; ++i) {
+      const auto& en = b->entries[i];
+      const auto& sg = b->segs_host[i];
+      auto pl = ctx->plans[en.n];
+      auto ci = ctx->configs.find(en.n);
+      const bege::CorrConfig cc =
+          ci != ctx->configs.end() ? ci->second : bege::default_config(pl->g);
+      bege::CorrelateArgs a{};
+      a.AB = sg.AB;
+      a.bank = sg.bank;
+      a.Lp = sg.Lp;
+      a.k0 = sg.k0;
+      a.k1 = sg.k1;
+      a.kappa = sg.kappa;
+      a.sigma = sg.sigma;
+      a.recs = sg.recs;
+      a.cap = sg.cap;
+      a.counter = sg.counter;
+      a.dump = nullptr;
+      a.max_clusters = 0;
+      if (b->plan == 1) e = bege::launch_correlate(pl->dev, a, cc, b->cs);
+      if (e == cudaSuccess && en.large) e = bege::launch_range(pl->dev, a, b->cs);
     }
   }
   cudaGraph_t g = nullptr;
@@ -750,11 +750,22 @@ int bege_define_bank_samples(bege_ctx* ctx, const float* samples, int64_t count,
   if (e == cudaSuccess)
     e = cudaMemcpy2DAsync(bank->w.ptr, bank->Lp * sizeof(float), samples, length * sizeof(float),
                           length * sizeof(float), (size_t)count, cudaMemcpyHostToDevice, s);
+  DevBuf flag;  // without room for it the bank counts as large
+  int large = 1;
+  if (e == cudaSuccess && ctx->take(&flag, 16) == BEGE_OK) {
+    e = bege::launch_bank_large(static_cast<float*>(bank->w.ptr), count * bank->Lp,
+                                static_cast<int*>(flag.ptr), s);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(&large, flag.ptr, sizeof(int), cudaMemcpyDeviceToHost, s);
+  }
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) {
+    ctx->release(&flag);
     ctx->release(&bank->w);
     return cuda_fail(e, "bank upload");
   }
+  ctx->keep(&flag);
+  bank->large = large != 0;
   const int32_t id = ctx->next_id++;
   ctx->banks[id] = std::move(bank);
   *bank_id = id;
@@ -836,6 +847,7 @@ static int correlate_impl(bege_ctx* ctx, int32_t seg_id, int32_t bank_id, int64_
       e = bege::launch_correlate_tc(seg->plan->dev, a, ctx->cfg.precision, s);
     } else {
       e = bege::launch_correlate(seg->plan->dev, a, cc, s);
+      if (e == cudaSuccess && bank->large) e = bege::launch_range(seg->plan->dev, a, s);
     }
   }
   if (e == cudaSuccess) e = cudaEventRecord(job->buf->k_stop, s);
@@ -935,6 +947,20 @@ int bege_correlate_multi(bege_ctx* ctx, const int32_t* seg_ids, int32_t n_seg, i
   for (auto& j : jobs)
     if (e == cudaSuccess) e = cudaEventRecord(j->buf->k_start, s);
   if (e == cudaSuccess) e = bege::launch_correlate_multi(segs[0]->plan->dev, a, s);
+  for (int32_t i = 0; i < n_seg && bank->large && e == cudaSuccess; ++i) {
+    bege::CorrelateArgs one{};
+    one.AB = a.AB[i];
+    one.bank = a.bank;
+    one.Lp = a.Lp;
+    one.k0 = a.k0;
+    one.k1 = a.k1;
+    one.kappa = a.kappa;
+    one.sigma = a.sigma[i];
+    one.recs = a.recs[i];
+    one.cap = a.cap[i];
+    one.counter = a.counter[i];
+    e = bege::launch_range(segs[i]->plan->dev, one, s);
+  }
   for (auto& j : jobs) {
     if (e == cudaSuccess) e = cudaEventRecord(j->buf->k_stop, s);
     if (e == cudaSuccess) e = cudaEventRecord(j->buf->done, s);
@@ -1289,7 +1315,7 @@ int bege_batch_create(bege_ctx* ctx, const bege_batch_entry* entries, int32_t co
       return fail(BEGE_EINVAL, "batch entry: template range outside the bank or empty");
     if (!std::isfinite(en.kappa) || en.kappa < 0.f)
       return fail(BEGE_EINVAL, "batch entry: kappa must be finite and >= 0");
-    b->entries.push_back({en.n, en.bank_id, en.k_begin, en.k_end, en.kappa});
+    b->entries.push_back({en.n, en.bank_id, en.k_begin, en.k_end, en.kappa, bi->second->large});
     b->sigma_off.push_back(nsig);
     ny += en.n;
     nD += en.n / 2 + 1;

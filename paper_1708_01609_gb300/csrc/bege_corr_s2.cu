@@ -8,4 +8,9 @@ cudaError_t launch_correlate_s2(const PlanDev& p, const CorrelateArgs& a, cudaSt
                           : unit::launch_short<unit::kF, false>(p, a, s);
 }
 
+cudaError_t launch_range_s2(const PlanDev& p, const CorrelateArgs& a, cudaStream_t s) {
+  return a.Lp <= unit::kF ? unit::launch_range_short<unit::kF, true>(p, a, s)
+                          : unit::launch_range_short<unit::kF, false>(p, a, s);
+}
+
 }  // namespace bege

@@ -192,6 +192,14 @@ struct CorrelateArgs {
 size_t exchange_bytes(const Geometry& g, CorrConfig cfg, int64_t count, int sms);
 cudaError_t launch_correlate(const PlanDev& p, const CorrelateArgs& a, CorrConfig cfg,
                              cudaStream_t s);
+// Behind the FP32 correlation of one segment in any form (single, block,
+// batch): the templates whose sigma came out not finite once more in a wider
+// range, where that gives another result.  Of use only for a bank that holds
+// a sample above kLargeSample (or none that is known).
+constexpr float kLargeSample = 0x1p64f;
+cudaError_t launch_range(const PlanDev& p, const CorrelateArgs& a, cudaStream_t s);
+// *flag = 1 if one of the n samples (a multiple of 8) is above kLargeSample, else 0.
+cudaError_t launch_bank_large(const float* samples, int64_t n, int* flag, cudaStream_t s);
 
 // Several segments of one length against the same templates (Sec. 3.2: a
 // template's transform serves a block of segments): per template the
@@ -224,6 +232,11 @@ cudaError_t launch_correlate_s8(const PlanDev& p, const CorrelateArgs& a, CorrCo
                                 cudaStream_t s);
 cudaError_t launch_correlate_s16(const PlanDev& p, const CorrelateArgs& a, CorrConfig c,
                                  cudaStream_t s);
+cudaError_t launch_range_s1(const PlanDev& p, const CorrelateArgs& a, cudaStream_t s);
+cudaError_t launch_range_s2(const PlanDev& p, const CorrelateArgs& a, cudaStream_t s);
+cudaError_t launch_range_s4(const PlanDev& p, const CorrelateArgs& a, cudaStream_t s);
+cudaError_t launch_range_s8(const PlanDev& p, const CorrelateArgs& a, cudaStream_t s);
+cudaError_t launch_range_s16(const PlanDev& p, const CorrelateArgs& a, cudaStream_t s);
 
 // Precision form: S2-S6 with the column FFTs on tcgen05 tensor cores.
 // precision 1 = BF16x3, 2 = FP16x3.  Needs F = 4096 (N >= 2^14) and

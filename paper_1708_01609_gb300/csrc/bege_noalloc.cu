@@ -107,6 +107,7 @@ extern "C" int bege_search_noalloc(const float* strain_dev, int64_t n, const flo
       a.dump = nullptr;
       a.max_clusters = 0;
       e = launch_correlate(p, a, default_config(g), s);
+      if (e == cudaSuccess) e = launch_range(p, a, s);
     }
     if (e != cudaSuccess) return set_last_error(BEGE_ECUDA, cudaGetErrorString(e));
   }

@@ -124,6 +124,38 @@ cudaError_t launch_correlate(const PlanDev& p, const CorrelateArgs& a, CorrConfi
   }
 }
 
+cudaError_t launch_range(const PlanDev& p, const CorrelateArgs& a, cudaStream_t s) {
+  if (a.k1 <= a.k0) return cudaSuccess;
+  switch (p.g.S) {
+    case 1: return launch_range_s1(p, a, s);
+    case 2: return launch_range_s2(p, a, s);
+    case 4: return launch_range_s4(p, a, s);
+    case 8: return launch_range_s8(p, a, s);
+    case 16: return launch_range_s16(p, a, s);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+// Bound by the read of the bank from HBM, once after its upload.
+__global__ void __launch_bounds__(256)
+bank_large_kernel(const float4* __restrict__ w, int64_t n, int* __restrict__ flag) {
+  bool large = false;
+  for (int64_t i = blockIdx.x * 256ll + threadIdx.x; i < n; i += gridDim.x * 256ll) {
+    const float4 v = __ldg(w + i);
+    large |= !(fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))) <= kLargeSample);
+  }
+  if (large) *flag = 1;
+}
+
+cudaError_t launch_bank_large(const float* samples, int64_t n, int* flag, cudaStream_t s) {
+  cudaError_t e = cudaMemsetAsync(flag, 0, sizeof(int), s);
+  if (e != cudaSuccess) return e;
+  const int64_t blocks = std::min<int64_t>((n / 4 + 255) / 256, 152 * 8);
+  bank_large_kernel<<<(unsigned)blocks, 256, 0, s>>>(reinterpret_cast<const float4*>(samples), n / 4,
+                                                     flag);
+  return cudaGetLastError();
+}
+
 // ---------------------------------------------------------------------------
 // Bank synthesis: w[m] = T(m) sin(2 pi phase(m)), unit L2 norm; time-
 // symmetric banks (Fig. 2 caption): w[m] = T(m) (sin(2 pi phase(m)) +

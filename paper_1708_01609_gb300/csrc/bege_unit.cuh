@@ -64,6 +64,8 @@ namespace unit {
 
 constexpr int kF = 4096;        // column length of N >= 2^14
 constexpr int kBlk = 288;       // 16-byte slots of a block of 256 rows
+constexpr float kMaxFinite = 3.402823466e38f;
+constexpr float kScaleDown = 0x1p-64f, kScaleUp = kLargeSample;  // see "Range"
 
 template <int F>
 struct Geo {
@@ -295,14 +297,17 @@ __device__ __forceinline__ void store_blocks(int ui, const float2 (&va)[16 / SM:
 // Otherwise folded over nfold multiples of F.  WAIT: the cluster's reads of the
 // previous contents of the rows are awaited after the loads and the
 // arithmetic, before the stores.  arrive: the cluster's barrier is arrived at
-// there.
-template <class SM, bool HALFZ, bool ONE, bool WAIT>
+// there.  SCALED: z times `scale`.
+template <class SM, bool HALFZ, bool ONE, bool WAIT, bool SCALED = false>
 __device__ __forceinline__ void stage1(int ui, int S, int ug, const float* __restrict__ src,
-                                       int nz, int nfold, bool arrive = false) {
+                                       int nz, int nfold, bool arrive = false, float scale = 1.f) {
   constexpr int R = SM::G::R, T = SM::G::T, F = 256 * R;
   const float2* z = reinterpret_cast<const float2*>(src);
   const int t = SM::tid();
-  auto load = [&](int m) { return m < nz ? __ldg(z + m) : make_float2(0.f, 0.f); };
+  auto load = [&](int m) {
+    const float2 x = m < nz ? __ldg(z + m) : make_float2(0.f, 0.f);
+    return SCALED ? cscale(x, scale) : x;
+  };
   float2 va[16 / R][R], vb[16 / R][R];
 #pragma unroll
   for (int i = 0; i < 16 / R; ++i)
@@ -469,10 +474,11 @@ __device__ __forceinline__ void stage3(int ui, const MidItem& m, bool self, floa
 // butterflies, in place.  MULTI: the spectrum is kept in `scratch` (16 float4 a
 // thread, stride T) for the block's other segments, or with `reload` read
 // from there.  AHEAD: pairs of rows whose coefficients are loaded ahead.
-template <class SM, int AHEAD, bool MULTI = false, bool WAIT = false>
+// SCALED: the spectrum times `scale`.
+template <class SM, int AHEAD, bool MULTI = false, bool WAIT = false, bool SCALED = false>
 __device__ __forceinline__ void middle(int ui, int ug, const float4* __restrict__ coef,
                                        float4* __restrict__ scratch = nullptr,
-                                       bool reload = false) {
+                                       bool reload = false, float scale = 1.f) {
   constexpr int kT = SM::G::T;
   const int t = SM::tid();
   const bool unit0 = ug == 0, self = unit0 && t == 0;
@@ -499,6 +505,13 @@ __device__ __forceinline__ void middle(int ui, int ug, const float4* __restrict_
     }
   } else {
     stage3<SM>(ui, m, self, za, zb);
+    if constexpr (SCALED) {
+#pragma unroll
+      for (int r = 0; r < 16; ++r) {
+        za[r] = cscale(za[r], scale);
+        zb[r] = cscale(zb[r], scale);
+      }
+    }
     if (MULTI && scratch) {
 #pragma unroll
       for (int r = 0; r < 16; ++r)
@@ -714,24 +727,33 @@ __device__ __forceinline__ void segment_unit(const PlanDev& p, int S, int ug,
   const int ui = T < 32 ? ((int)threadIdx.x / T) & 1 : 0;
   if ((int)threadIdx.x < T) setup_unit<SM>(p, S, ug, 0);
   __syncthreads();
-  if (fft) stage1<SM, false, ONE, false>(ui, S, ug, y, p.g.H, S);
-  __syncthreads();
-  if (fft) stage2<SM>(ui);
-  __syncthreads();
   float2* const z = reinterpret_cast<float2*>(SM::rows(ui));
-  {
-    const int t = SM::tid();
+  const int t = SM::tid();
+  const bool self = ug == 0 && t == 0;
+  // once more from y / 2^64 if some value is not finite, see "Range"
+  for (float down = 1.f, up = 1.f;; down = kScaleDown, up = kScaleUp) {
+    if (fft) stage1<SM, false, ONE, false, true>(ui, S, ug, y, p.g.H, S, false, down);
+    __syncthreads();
+    if (fft) stage2<SM>(ui);
+    __syncthreads();
     float2 za[16], zb[16];
-    const bool self = ug == 0 && t == 0;
-    if (fft) stage3<SM>(ui, mid_item<R>(ug == 0, t), self, za, zb);
-    __syncthreads();  // the rows have been read
+    float nonfinite = 0.f;
+    if (fft) {
+      stage3<SM>(ui, mid_item<R>(ug == 0, t), self, za, zb);
+#pragma unroll
+      for (int r = 0; r < 16; ++r)
+        nonfinite += (za[r].x - za[r].x) + (za[r].y - za[r].y) + (zb[r].x - zb[r].x) + (zb[r].y - zb[r].y);
+    }
+    // the rows have been read
+    if (__syncthreads_or(nonfinite != 0.f) && down == 1.f) continue;
     if (fft) {
 #pragma unroll
       for (int r = 0; r < 16; ++r) {
-        z[2 * r * T + t] = za[r];
-        z[(2 * r + 1) * T + t] = self ? zb[r] : cconj(zb[r]);
+        z[2 * r * T + t] = cscale(za[r], up);
+        z[(2 * r + 1) * T + t] = cscale(self ? zb[r] : cconj(zb[r]), up);
       }
     }
+    break;
   }
   __syncthreads();
   const float2* const zs = reinterpret_cast<const float2*>(SM::rows(0));
@@ -1127,6 +1149,144 @@ __global__ void __launch_bounds__(256, 2) short_kernel(PlanDev p, CorrelateArgs 
   }
 }
 
+// ---------------------------------------------------------------------------
+// Range
+// ---------------------------------------------------------------------------
+// At a quarter turn the tangent form holds (1 -/+ 2^30 i) b between its two
+// products, so values beyond 2^97 overflow there although the spectrum is
+// finite.  Nothing that overflowed leaves a template's sum |Y|^2 finite, and
+// one whose sigma is not finite has no tails.  These kernels, launched behind
+// a search whose bank holds samples above 2^64 (or is not known), do the
+// templates without finite sigma again: from z / 2^64, with the spectrum
+// brought back before the product.  Both factors are exact but for values
+// 2^126 times smaller than the largest.  A template without a sample above
+// 2^64 (its product has overflowed) stays as it is.  With a finite sigma the
+// inverse stages stay below 2^81.  They are kernels of their own because any
+// of it in the searching kernels, a call behind their loops included, changed
+// their registers: 0.97 to 1.03 times their time, batch 1.05.
+//
+// The factor of unit ui, 1 where it is not (wanted) or of no use.
+template <class SM>
+__device__ __forceinline__ float range_scale(int* over, int ui, const float* __restrict__ src,
+                                             int nz, bool wanted) {
+  SM::sync(ui);  // over[ui] has been read
+  if (SM::tid() == 0) over[ui] = 0;
+  SM::sync(ui);
+  bool large = false;
+  for (int m = SM::tid(); m < nz; m += SM::G::T) {
+    const float2 x = __ldg(reinterpret_cast<const float2*>(src) + m);
+    large |= !(fmaxf(fabsf(x.x), fabsf(x.y)) <= kScaleUp);
+  }
+  if (wanted && large) over[ui] = 1;
+  SM::sync(ui);
+  return over[ui] ? kScaleDown : 1.f;
+}
+
+// Stages 1 to 2' with the factor.
+template <class SM, int U, bool HALFZ, bool ONE>
+__device__ __forceinline__ void scaled_rows(int ui, int S, int ug, const float* __restrict__ src,
+                                            int nz, int nfold, const float4* __restrict__ coef,
+                                            float down) {
+  stage1<SM, HALFZ, ONE, false, true>(ui, S, ug, src, nz, nfold, false, down);
+  SM::sync(ui);
+  stage2<SM>(ui);
+  mid_enter<SM, U>(ui, ug);
+  middle<SM, 1, false, false, true>(ui, ug, coef, nullptr, false, 1.f / down);
+  mid_leave<SM, U>(ui, ug);
+  stage2i<SM>(ui);
+  SM::sync(ui);
+}
+
+// The rows [r0, r1) of group g of n groups, and whether one of them has no
+// finite sigma (which all CTAs of a group see alike; a barrier of the CTA).
+__device__ __forceinline__ bool range_rows(const CorrelateArgs& a, int64_t g, int64_t n,
+                                           int64_t* r0, int64_t* r1) {
+  const int64_t count = a.k1 - a.k0, per = (count + n - 1) / n;
+  *r0 = g * per;
+  *r1 = *r0 + per < count ? *r0 + per : count;
+  bool bad = false;
+  for (int64_t r = *r0 + threadIdx.x; r < *r1; r += blockDim.x)
+    bad |= !(__ldcg(a.sigma + r) <= kMaxFinite);
+  return __syncthreads_or(bad);
+}
+
+// N >= 2^15: clusters of S / 4 CTAs of two units, as unit_kernel.
+template <int S, bool HALFZ, bool EXT>
+__global__ void __launch_bounds__(512, 1) range_kernel(PlanDev p, CorrelateArgs a) {
+  constexpr int U = 2, C = S / 2 / U;
+  using SM = Sm<kF, U>;
+  __shared__ int over[U];
+  cg::cluster_group cluster = cg::this_cluster();
+  const int rank = C == 1 ? 0 : (int)cluster.block_rank();
+  const int ui = (int)threadIdx.x / SM::G::T, ug = rank * U + ui;
+  int64_t r0, r1;
+  if (!range_rows(a, blockIdx.x / C, gridDim.x / C, &r0, &r1)) return;
+  setup_common<SM, 256 * U>(p);
+  setup_unit<SM>(p, S, ug, ui);
+  if (threadIdx.x < S / 2) {
+    const int c = (int)threadIdx.x / U, u = (int)threadIdx.x % U;
+    float4* const rows = C == 1 ? SM::rows(0) : cluster.map_shared_rank(SM::rows(0), (unsigned)c);
+    SM::rowptr()[threadIdx.x] = rows + u * (SM::L::unit_bytes / 16);
+  }
+  cluster.sync();
+  const int nz = (int)(a.Lp / 2), nfold = (nz + kF - 1) / kF;
+  const TailOut out{a.recs, a.cap, a.counter, a.dump, a.proj, a.kappa_hi, a.lag_end};
+  for (int64_t r = r0; r < r1; ++r) {
+    if (__ldcg(a.sigma + r) <= kMaxFinite) continue;
+    const int64_t k = a.k0 + r;
+    const float* const src = a.bank + k * a.Lp;
+    const float down = range_scale<SM>(over, ui, src, nz, true);
+    if (down == 1.f) continue;
+    scaled_rows<SM, U, HALFZ, false>(ui, S, ug, src, nz, nfold, a.AB, down);
+    float2 va[1][16], vb[1][16];
+    stage1i<SM>(ui, va, vb);
+    store_blocks<SM>(ui, va, vb);
+    if (SM::tid() == 0) {
+      const float share = unit_power<SM>(ui);
+      for (int q = 0; q < C; ++q) *cluster.map_shared_rank(SM::sigall() + ug, (unsigned)q) = share;
+    }
+    cluster.sync();  // and every CTA has read this sigma
+    const float sigma = sigma_of(SM::sigall(), S / 2, S * 2 * kF);
+    if (rank == 0 && threadIdx.x == 0) a.sigma[r] = sigma;
+    Combine<S, U> cb;
+    cb.twiddles(p.uc, rank);
+    cb.template emit<EXT>(typename Combine<S, U>::Shared{SM::rowptr()}, p.uc, rank,
+                          a.kappa * sigma, (uint32_t)k, r, out, sigma);
+    cluster.sync();
+  }
+}
+
+// N <= 2^14, as short_kernel.
+template <int F, bool HALFZ, bool EXT>
+__global__ void __launch_bounds__(256, 2) range_short_kernel(PlanDev p, CorrelateArgs a) {
+  constexpr int U = 4096 / F;
+  using SM = Sm<F, U, true>;
+  __shared__ int over[U];
+  const int ui = U == 1 ? 0 : (int)threadIdx.x / SM::G::T;
+  int64_t r0, r1;
+  if (!range_rows(a, blockIdx.x, gridDim.x, &r0, &r1)) return;
+  setup_common<SM, 256>(p);
+  if (ui == 0) setup_unit<SM>(p, 2, 0, 0);
+  __syncthreads();
+  const int nz = (int)(a.Lp / 2);
+  for (; r0 < r1; r0 += U) {  // a unit's barriers are its own; units of a warp go together
+    const int64_t r = r0 + ui < r1 ? r0 + ui : r0, k = a.k0 + r;
+    const bool wanted = r0 + ui < r1 && !(__ldcg(a.sigma + r) <= kMaxFinite);
+    if (!__any_sync(0xffffffffu, wanted)) continue;
+    const float* const src = a.bank + k * a.Lp;
+    const float down = range_scale<SM>(over, ui, src, nz, wanted);
+    const bool active = down != 1.f;
+    if (!__any_sync(0xffffffffu, active)) continue;
+    scaled_rows<SM, U, HALFZ, true>(ui, 2, 0, src, nz, 0, a.AB, down);
+    const float share = unit_power<SM>(ui);
+    const float sigma = sigma_of(&share, 1, 4 * F);
+    if (active && SM::tid() == 0) a.sigma[r] = sigma;
+    const TailOut out{a.recs, a.cap, a.counter, active ? a.dump : nullptr, a.proj, a.kappa_hi,
+                      a.lag_end};
+    finish_s2<SM, EXT>(ui, p.uc, active ? a.kappa * sigma : INFINITY, (uint32_t)k, r, out, sigma);
+  }
+}
+
 template <int S, int U, bool HALFZ, bool EXT>
 static cudaError_t launch_unit_t(const PlanDev& p, const CorrelateArgs& a, cudaStream_t s) {
   constexpr int C = S / 2 / U;
@@ -1161,6 +1321,27 @@ static cudaError_t launch_short(const PlanDev& p, const CorrelateArgs& a, cudaSt
   return extended(p, a)
              ? launch_clusters<short_kernel<F, HALFZ, true>>(1, 256, smem, 2, U, p, a, s)
              : launch_clusters<short_kernel<F, HALFZ, false>>(1, 256, smem, 2, U, p, a, s);
+}
+
+template <int S>
+static cudaError_t launch_range(const PlanDev& p, const CorrelateArgs& a, cudaStream_t s) {
+  constexpr int C = S / 4;
+  constexpr size_t smem = Lay<kF, 2, false>::total;
+  const bool ext = extended(p, a);
+  if (a.Lp <= kF)
+    return ext ? launch_clusters<range_kernel<S, true, true>>(C, 512, smem, 1, 1, p, a, s)
+               : launch_clusters<range_kernel<S, true, false>>(C, 512, smem, 1, 1, p, a, s);
+  return ext ? launch_clusters<range_kernel<S, false, true>>(C, 512, smem, 1, 1, p, a, s)
+             : launch_clusters<range_kernel<S, false, false>>(C, 512, smem, 1, 1, p, a, s);
+}
+
+template <int F, bool HALFZ>
+static cudaError_t launch_range_short(const PlanDev& p, const CorrelateArgs& a, cudaStream_t s) {
+  constexpr int U = 4096 / F;
+  constexpr size_t smem = Lay<F, U, true>::total;
+  return extended(p, a)
+             ? launch_clusters<range_short_kernel<F, HALFZ, true>>(1, 256, smem, 2, U, p, a, s)
+             : launch_clusters<range_short_kernel<F, HALFZ, false>>(1, 256, smem, 2, U, p, a, s);
 }
 
 }  // namespace unit
