@@ -133,7 +133,7 @@ __global__ void __launch_bounds__(kT, 2) batch_kernel(BatchArgs b) {
 
 // S1 for every segment of the batch: block i computes rank jobs[i].rank of
 // segment jobs[i] (S/2 blocks per segment).
-__global__ void __launch_bounds__(kT, 1) segment_batch_kernel(BatchArgs b,
+__global__ void __launch_bounds__(2 * kT, 1) segment_batch_kernel(BatchArgs b,
                                                              const SegJob* __restrict__ jobs) {
   const SegJob j = jobs[blockIdx.x];
   segment_unit<Sm<kF, 1>, false>(b.plans[plan_index(j.S)], j.S, j.rank, j.y, j.D, j.AB, false);
@@ -195,7 +195,7 @@ cudaError_t launch_segment_batch(const BatchArgs& b, const SegJob* jobs, int njo
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   if (njobs <= 0) return cudaSuccess;
-  segment_batch_kernel<<<njobs, kT, smem, s>>>(b, jobs);
+  segment_batch_kernel<<<njobs, 2 * kT, smem, s>>>(b, jobs);
   return cudaGetLastError();
 }
 

@@ -427,6 +427,23 @@ template <class SM>
 __device__ __forceinline__ const float4* mid_row(int ui, int slot, int k0, int k1) {
   return SM::rows(ui) + k0 * kBlk + (slot * 144 + k1 * 9);
 }
+// The conjugated inputs of butterfly (0, 8), which has its own base, 1/32 turn,
+// and no mirror: conjugated back and turned.
+__device__ __forceinline__ void self_turn(float2 (&x)[16]) {
+  constexpr float c[16] = {1.f, 0.98078528040323044913f, 0.92387953251128675613f,
+                           0.83146961230254523708f, 0.70710678118654752440f,
+                           0.55557023301960222474f, 0.38268343236508977173f,
+                           0.19509032201612826785f, 0.f, -0.19509032201612826785f,
+                           -0.38268343236508977173f, -0.55557023301960222474f,
+                           -0.70710678118654752440f, -0.83146961230254523708f,
+                           -0.92387953251128675613f, -0.98078528040323044913f};
+#pragma unroll
+  for (int r = 1; r < 16; ++r) {
+    const float s = r < 8 ? c[8 - r] : c[r - 8];  // sin(2 pi r / 32)
+    x[r] = cmul(cconj(x[r]), make_float2(c[r], -s));
+  }
+  x[0] = cconj(x[0]);
+}
 template <class SM>
 __device__ __forceinline__ void stage3(int ui, const MidItem& m, bool self, float2 (&za)[16],
                                        float2 (&zb)[16]) {
@@ -443,21 +460,7 @@ __device__ __forceinline__ void stage3(int ui, const MidItem& m, bool self, floa
     xb[2 * r] = make_float2(u.x, -u.y);
     xb[2 * r + 1] = make_float2(u.z, -u.w);
   }
-  if (self) {  // butterfly (0, 8) has its own base, 1/32 turn, and no mirror
-    constexpr float c[16] = {1.f, 0.98078528040323044913f, 0.92387953251128675613f,
-                             0.83146961230254523708f, 0.70710678118654752440f,
-                             0.55557023301960222474f, 0.38268343236508977173f,
-                             0.19509032201612826785f, 0.f, -0.19509032201612826785f,
-                             -0.38268343236508977173f, -0.55557023301960222474f,
-                             -0.70710678118654752440f, -0.83146961230254523708f,
-                             -0.92387953251128675613f, -0.98078528040323044913f};
-#pragma unroll
-    for (int r = 1; r < 16; ++r) {
-      const float s = r < 8 ? c[8 - r] : c[r - 8];  // sin(2 pi r / 32)
-      xb[r] = cmul(cconj(xb[r]), make_float2(c[r], -s));
-    }
-    xb[0] = cconj(xb[0]);
-  }
+  if (self) self_turn(xb);
   const float2* w = SM::t3(ui) + t;
   dft16x2<false, false>(xa, xb, [&](int q) {
     const float2 s = w[kT * q];
@@ -676,14 +679,22 @@ __device__ __forceinline__ void stage1i(int ui, float2 (&va)[16 / SM::G::R][SM::
 // S1: segment spectrum D and product coefficients A, B of a unit
 // ---------------------------------------------------------------------------
 // The strain takes the template's stages 1 to 3 (folded over the S multiples
-// of F), so a thread ends with the bins of a butterfly and its mirror: D, A
-// and B of both follow in registers.
+// of F).  Then D, A and B of a bin and its mirror follow from their two values.
+// Bound: latency, of few warps that depend on one another, so the work is
+// spread: a thread takes one column's butterfly, not two, and several CTAs run
+// the stages of a unit, each to form its share of the pairs.  One launch behind
+// the other from device memory (GB300), against one CTA a unit with both
+// columns in a thread (and the Stockham kernel before that): N = 2^10 6.4 us
+// (7.8, 6.9), 2^12 6.6 (10.5, 7.7), 2^13 8.5 (16.5, 11.0), 2^14 13.0 (23.1,
+// 18.0); a load and its wait at 2^15 23 (37, 46), 2^16 25 (41, 71), where loads
+// in a row wait for the allocation.
 struct BinPair {
   float2 A, B, Am, Bm;  // of bin j and of bin H - j
 };
-// Bins j and jm = H - j (j = 0: jm = 0 stands for the Nyquist bin's partner).
-__device__ __forceinline__ BinPair bin_pair(const PlanDev& p, int j, int jm, float2 zj, float2 zm,
-                                            float2* __restrict__ D) {
+// Bins j and jm = H - j (j = 0: jm = 0 stands for the Nyquist bin's partner)
+// with their factors wN^j, wN^jm.
+__device__ __forceinline__ BinPair bin_pair(const PlanDev& p, int j, int jm, float2 wj, float2 wm,
+                                            float2 zj, float2 zm, float2* __restrict__ D) {
   const int H = p.g.H;
   // D_j = (Zj + conj Zm)/2 - (i/2) wN^j (Zj - conj Zm)
   auto spectrum = [](float2 w, float2 x, float2 y) {
@@ -698,7 +709,6 @@ __device__ __forceinline__ BinPair bin_pair(const PlanDev& p, int j, int jm, flo
     A = cadd(cmul(cmul(g, g), Dx), cmul(cmul(d, d), cH));
     B = cmul(cmul(g, d), cadd(Dx, cH));
   };
-  const float2 wj = p.wN[j], wm = p.wN[jm];
   const float2 Dj = spectrum(wj, zj, zm);
   const float2 Dm = j == jm ? Dj : spectrum(wm, zm, zj);
   const float2 DH = make_float2(zj.x - zj.y, 0.f);  // D_{N/2}, used when j == 0
@@ -712,45 +722,133 @@ __device__ __forceinline__ BinPair bin_pair(const PlanDev& p, int j, int jm, flo
 }
 
 // natural: {A, B} of bin j at (j mod S) F + j / S (the tensor-core kernel);
-// otherwise where middle reads them.  The first T threads of the CTA run the
+// otherwise where middle reads them.  The first 2 T threads of the CTA run the
 // stages and leave the spectrum in shared memory by thread and row (Z of row r
 // at 2 r T + t, of its mirror at (2 r + 1) T + t; thread 0 of unit 0: rows r
-// of its two butterflies), and all of them form the pairs: a loop over 16 T
-// items keeps the code short (unrolled over the 16 rows of a butterfly it took
-// 25 us for N = 2^12, mostly instruction fetches) and every thread at work.
+// of its two butterflies).  Of the 16 T pairs the CTA forms those of its part
+// (of parts): a loop keeps the code short (unrolled over the 16 rows of a
+// butterfly it took 25 us for N = 2^12, mostly instruction fetches).
 template <class SM, bool ONE>
 __device__ __forceinline__ void segment_unit(const PlanDev& p, int S, int ug,
                                              const float* __restrict__ y, float2* __restrict__ D,
-                                             float4* __restrict__ AB, bool natural) {
+                                             float4* __restrict__ AB, bool natural, int part = 0,
+                                             int parts = 1) {
   constexpr int R = SM::G::R, T = SM::G::T, F = 256 * R;
-  const bool fft = threadIdx.x < (T < 32 ? 32 : T);  // F = 256: a second unit repeats the first
-  const int ui = T < 32 ? ((int)threadIdx.x / T) & 1 : 0;
-  if ((int)threadIdx.x < T) setup_unit<SM>(p, S, ug, 0);
-  __syncthreads();
-  float2* const z = reinterpret_cast<float2*>(SM::rows(ui));
-  const int t = SM::tid();
+  const int H = S * F;
+  auto bin = [&](int b, int k0, int k1, int k2) { return S * (k0 + R * k1 + 16 * R * k2) + b; };
+  // thread t of slot h (column h of the unit, in the middle za or zb)
+  const int t = SM::tid(), h = ((int)threadIdx.x / T) & 1;
+  const bool fft = (int)threadIdx.x < 2 * T;
   const bool self = ug == 0 && t == 0;
+  // the tables by the CTA's last T threads, the samples under way meanwhile
+  if ((int)(blockDim.x - threadIdx.x) <= T) setup_unit<SM>(p, S, ug, 0);
+  // the bins of this thread's next pair and their factors, loaded ahead
+  int it = part * blockDim.x + threadIdx.x, j = 0, jm = 0;
+  float2 wj, wm;
+  auto next_pair = [&] {
+    const int u = it & (T - 1), r = it / T;
+    const MidItem m = mid_item<R>(ug == 0, u);
+    const int ba = ug == 0 ? m.sa * (S / 2) : ug, bb = ug == 0 ? ba : S - ug;
+    j = bin(ba, m.k0, m.k1, r);
+    jm = bin(bb, m.k0b, m.k1b, 15 - r);
+    if (it < 16 * T && (ug != 0 || u != 0)) {
+      wj = p.wN[j];
+      wm = p.wN[jm];
+    }
+  };
+  next_pair();
+  float2* const rows = reinterpret_cast<float2*>(SM::rows(0));
   // once more from y / 2^64 if some value is not finite, see "Range"
-  for (float down = 1.f, up = 1.f;; down = kScaleDown, up = kScaleUp) {
-    if (fft) stage1<SM, false, ONE, false, true>(ui, S, ug, y, p.g.H, S, false, down);
-    __syncthreads();
-    if (fft) stage2<SM>(ui);
-    __syncthreads();
-    float2 za[16], zb[16];
-    float nonfinite = 0.f;
-    if (fft) {
-      stage3<SM>(ui, mid_item<R>(ug == 0, t), self, za, zb);
+  float up = 1.f;
+  for (float down = 1.f;; down = kScaleDown, up = kScaleUp) {
+    {  // stage 1
+      auto load = [&](int m) {
+        return cscale(__ldg(reinterpret_cast<const float2*>(y) + m), down);
+      };
+      float2 v[16 / R][R];
+      if (fft) {
 #pragma unroll
-      for (int r = 0; r < 16; ++r)
-        nonfinite += (za[r].x - za[r].x) + (za[r].y - za[r].y) + (zb[r].x - zb[r].x) + (zb[r].y - zb[r].y);
+        for (int i = 0; i < 16 / R; ++i)
+#pragma unroll
+          for (int r = 0; r < R; ++r) {
+            const int m = t + T * i + 256 * r;
+            v[i][r] = load(m);
+            if constexpr (ONE) {
+              const float2 x = load(m + F);
+              v[i][r] = h ? csub(v[i][r], x) : cadd(v[i][r], x);
+            }
+          }
+      }
+      __syncthreads();  // the tables
+      if (fft) {
+        if constexpr (!ONE) {
+          const int b = h == 0 ? ug : ug == 0 ? S / 2 : S - ug;
+#pragma unroll 1
+          for (int f = 1; f < S; ++f) {
+            const float2 w = SM::ws()[(b * f) & (S - 1)];
+#pragma unroll
+            for (int i = 0; i < 16 / R; ++i)
+#pragma unroll
+              for (int r = 0; r < R; ++r)
+                v[i][r] = cadd(v[i][r], cmul(load(t + T * i + 256 * r + F * f), w));
+          }
+        }
+        const float2* const w = reinterpret_cast<const float2*>(SM::t1(0)) + h;
+#pragma unroll
+        for (int i = 0; i < 16 / R; ++i) {
+          dft_row<R, false>(v[i], [&](int q) { return w[2 * q]; });
+#pragma unroll
+          for (int k = 0; k < R; ++k)
+            rows[2 * (k * kBlk + t + T * i) + h] = v[i][rev<R>(k)];
+        }
+      }
+    }
+    __syncthreads();
+    float2 v[16];
+    {  // stage 2
+      const int k0 = R == 1 ? 0 : (t & 16) ? R - 1 - (t >> 5) : t >> 5, n0 = t & 15;
+      float2* const blk = rows + 2 * k0 * kBlk;
+      if (fft) {
+#pragma unroll
+        for (int r = 0; r < 16; ++r) v[r] = blk[2 * (n0 + 16 * r) + h];
+        const float2* const w = reinterpret_cast<const float2*>(SM::t2(0)) + 2 * k0 + h;
+        dft_row<16, false>(v, [&](int q) { return w[2 * R * q]; });
+      }
+      __syncthreads();
+      if (fft) {
+#pragma unroll
+        for (int k = 0; k < 16; ++k) blk[288 * h + n0 + 18 * k] = v[rev<16>(k)];
+      }
+    }
+    __syncthreads();
+    float bad[4] = {0.f, 0.f, 0.f, 0.f};
+    if (fft) {  // stage 3: the butterfly, or its mirror conjugated
+      const MidItem m = mid_item<R>(ug == 0, t);
+      const float4* const x =
+          h ? mid_row<SM>(0, m.sb, m.k0b, m.k1b) : mid_row<SM>(0, m.sa, m.k0, m.k1);
+      const float sign = h ? -1.f : 1.f;
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        const float4 u = x[r];
+        v[2 * r] = make_float2(u.x, sign * u.y);
+        v[2 * r + 1] = make_float2(u.z, sign * u.w);
+      }
+      if (self && h) self_turn(v);
+      const float2* const w = SM::t3(0) + t;
+      dft_row<16, false>(v, [&](int q) { return w[T * q]; });
+#pragma unroll
+      for (int r = 0; r < 16; ++r) {
+        bad[r & 1] = fmaf(v[r].x, 0.f, bad[r & 1]);
+        bad[2 + (r & 1)] = fmaf(v[r].y, 0.f, bad[2 + (r & 1)]);
+      }
     }
     // the rows have been read
-    if (__syncthreads_or(nonfinite != 0.f) && down == 1.f) continue;
+    if (__syncthreads_or((bad[0] + bad[1]) + (bad[2] + bad[3]) != 0.f) && down == 1.f) continue;
     if (fft) {
 #pragma unroll
       for (int r = 0; r < 16; ++r) {
-        z[2 * r * T + t] = cscale(za[r], up);
-        z[(2 * r + 1) * T + t] = cscale(self ? zb[r] : cconj(zb[r]), up);
+        const float2 z = v[rev<16>(r)];
+        rows[(2 * r + h) * T + t] = h && !self ? cconj(z) : z;
       }
     }
     break;
@@ -760,18 +858,19 @@ __device__ __forceinline__ void segment_unit(const PlanDev& p, int S, int ug,
   auto place = [&](int j, float2 A, float2 B) {
     AB[(j % S) * F + j / S] = make_float4(A.x, A.y, B.x, B.y);
   };
-  auto bin = [&](int b, int k0, int k1, int k2) { return S * (k0 + R * k1 + 16 * R * k2) + b; };
   float2* const af = reinterpret_cast<float2*>(AB + (size_t)ug * (24 * T));
   // third q of the pair of rows that holds `row`: {A, A'} of either row, {B, B}
   auto third = [&](int row, int q, int t) { return 2 * ((3 * (row >> 1) + q) * T + t); };
 #pragma unroll 2
-  for (int it = threadIdx.x; it < 16 * T; it += blockDim.x) {
-    const int t = it & (T - 1), r = it / T;
+  while (it < 16 * T) {
+    const int t = it & (T - 1), r = it / T, j0 = j, jm0 = jm;
+    const float2 wj0 = wj, wm0 = wm;
+    it += parts * blockDim.x;
+    next_pair();
     if (ug != 0 || t != 0) {
-      const MidItem m = mid_item<R>(ug == 0, t);
-      const int ba = ug == 0 ? m.sa * (S / 2) : ug, bb = ug == 0 ? ba : S - ug;
-      const int j = bin(ba, m.k0, m.k1, r), jm = bin(bb, m.k0b, m.k1b, 15 - r);
-      const BinPair o = bin_pair(p, j, jm, zs[2 * r * T + t], zs[(2 * r + 1) * T + t], D);
+      const int j = j0, jm = jm0;
+      const BinPair o = bin_pair(p, j, jm, wj0, wm0, cscale(zs[2 * r * T + t], up),
+                                 cscale(zs[(2 * r + 1) * T + t], up), D);
       if (natural) {
         place(j, o.A, o.B);
         place(jm, o.Am, o.Bm);
@@ -786,7 +885,8 @@ __device__ __forceinline__ void segment_unit(const PlanDev& p, int S, int ug,
     // where the product's thread 0 looks for them, see middle
     if (r <= 8) {
       const int rm = (16 - r) & 15, j = bin(0, 0, 0, r), jm = bin(0, 0, 0, rm);
-      const BinPair o = bin_pair(p, j, jm, zs[2 * r * T], zs[2 * rm * T], D);
+      const BinPair o =
+          bin_pair(p, j, jm, p.wN[j], p.wN[jm], cscale(zs[2 * r * T], up), cscale(zs[2 * rm * T], up), D);
       if (natural) {
         place(j, o.A, o.B);
         if (jm != j) place(jm, o.Am, o.Bm);
@@ -804,7 +904,8 @@ __device__ __forceinline__ void segment_unit(const PlanDev& p, int S, int ug,
     }
     if (r < 8) {
       const int j = bin(0, 0, 8, r), jm = bin(0, 0, 8, 15 - r);
-      const BinPair o = bin_pair(p, j, jm, zs[(2 * r + 1) * T], zs[(2 * (15 - r) + 1) * T], D);
+      const BinPair o = bin_pair(p, j, jm, p.wN[j], p.wN[jm], cscale(zs[(2 * r + 1) * T], up),
+                                 cscale(zs[(2 * (15 - r) + 1) * T], up), D);
       if (natural) {
         place(j, o.A, o.B);
         place(jm, o.Am, o.Bm);
@@ -817,22 +918,33 @@ __device__ __forceinline__ void segment_unit(const PlanDev& p, int S, int ug,
   }
 }
 
-// One CTA of 256 threads per unit.
+// CTAs per unit: each runs the stages and forms its share of the pairs, one a
+// thread.
+template <int F>
+__host__ __device__ constexpr int segment_threads() {
+  return F / 8 < 256 ? 256 : F / 8;
+}
+template <int F>
+__host__ __device__ constexpr int segment_parts() {
+  return F / segment_threads<F>();
+}
 template <int F, bool ONE>
-__global__ void __launch_bounds__(256, 1)
+__global__ void __launch_bounds__(segment_threads<F>(), 1)
 segment_kernel(PlanDev p, const float* __restrict__ y, float2* __restrict__ D,
                float4* __restrict__ AB, bool natural) {
-  segment_unit<Sm<F, F == 256 ? 2 : 1, ONE>, ONE>(p, unit_geo(p.g).S, blockIdx.x, y, D, AB, natural);
+  constexpr int P = segment_parts<F>();
+  segment_unit<Sm<F, 1, ONE>, ONE>(p, unit_geo(p.g).S, blockIdx.x / P, y, D, AB,
+                                                  natural, blockIdx.x % P, P);
 }
 
 template <int F, bool ONE>
 static cudaError_t launch_segment_t(const PlanDev& p, const float* y, float2* D, float4* AB,
                                     bool natural, cudaStream_t s) {
-  constexpr size_t smem = Lay<F, F == 256 ? 2 : 1, ONE>::total;
+  constexpr size_t smem = Lay<F, 1, ONE>::total;
   auto kern = segment_kernel<F, ONE>;
   cudaError_t e = ensure_smem(kern, smem);
   if (e != cudaSuccess) return e;
-  kern<<<unit_geo(p.g).S / 2, 256, smem, s>>>(p, y, D, AB, natural);
+  kern<<<unit_geo(p.g).S / 2 * segment_parts<F>(), segment_threads<F>(), smem, s>>>(p, y, D, AB, natural);
   return cudaGetLastError();
 }
 
