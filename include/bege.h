@@ -251,7 +251,8 @@ BEGE_API int bege_get_bank_samples(bege_ctx* ctx, int32_t bank_id, int64_t k_beg
 BEGE_API int64_t bege_segment_length(bege_ctx* ctx, int32_t seg_id);
 BEGE_API int64_t bege_bank_length(bege_ctx* ctx, int32_t bank_id);
 
-/* Device bytes currently owned by the context. */
+/* Device bytes currently owned by the context, with what it keeps between
+ * calls (see bege_release). */
 BEGE_API uint64_t bege_device_bytes(const bege_ctx* ctx);
 
 /* Launch shapes of the correlate kernel for segment length n.  A shape is
@@ -443,8 +444,14 @@ BEGE_API int bege_search_noalloc(const float* strain_dev, int64_t n, const float
                                  uint64_t tail_capacity, unsigned long long* tail_count_dev,
                                  void* stream);
 
-/* Release a segment, bank, job or batch handle and its device memory (job
- * buffers return to the context's pool).  Errors: EINVAL for an unknown
+/* Release a segment, bank, job or batch handle and its device memory.  The
+ * context keeps for later calls: the buffers of a job (sigma, records), of
+ * released segments up to 4 MB in all, and, unless it has a budget, the buffers
+ * through which the search of N >= 2^16 exchanges columns, at most 40 MB each,
+ * as many as jobs were held at once, 160 MB in all.  Segment and exchange
+ * buffers go back to the device when an allocation of the context does not fit,
+ * with bege_serve_destroy and with bege_destroy; a context with
+ * hbm_budget_bytes has no exchange buffers.  Errors: EINVAL for an unknown
  * handle. */
 BEGE_API int bege_release(bege_ctx* ctx, int32_t handle);
 
