@@ -23,7 +23,7 @@ def mctx():
     c.close()
 
 
-@pytest.mark.parametrize("lg,m", [(16, 1), (16, 3), (16, 8), (14, 2), (17, 2)])
+@pytest.mark.parametrize("lg,m", [(16, 1), (16, 3), (16, 8), (14, 2), (15, 3), (17, 2)])
 def test_multi_equals_single_searches(mctx, lg, m):
     ctx, bank, params = mctx
     n = 1 << lg

@@ -87,11 +87,12 @@ def test_coefficients_and_tables_at_a_quarter_turn(ctx):
 def test_exchange_through_l2_equals_shared_memory(ctx, n, length):
     """N >= 2^16 exchanges columns through a buffer one template behind; a
     context with a budget does without it.  Same bits, over several templates
-    per cluster and a last round that not every cluster takes part in."""
+    per cluster and a last round that not every cluster takes part in, in both
+    epilogues."""
     count = 401
     bank = S.random_samples_bank(count, length, n + length)
     y = S.band_limited_noise(n, 5)
-    got = []
+    got, extended = [], []
     small = make_ctx(hbm_budget_bytes=1 << 30)
     for c in (ctx, small):
         seg, bid = c.bege_load_segment(y), c.bege_define_bank_samples(bank)
@@ -102,11 +103,48 @@ def test_exchange_through_l2_equals_shared_memory(ctx, n, length):
             assert total == len(recs) > 0
             got.append((recs.copy(), c.bege_get_sigma(job, k1 - k0)))
             c.bege_release(job)
+        job = c.bege_correlate_ex(seg, bid, 0, count, 3.5, kappa_hi=4.5, linear=True, project=True)
+        recs, total = c.bege_fetch_tails(job, sort=True)
+        assert total == len(recs) > 0
+        extended.append((recs.copy(), *c.bege_fetch_max(job, n)))
+        c.bege_release(job)
         c.bege_release(seg)
         c.bege_release(bid)
     small.close()
     for a, b in zip(got[:2], got[2:]):
         assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
+    for a, b in zip(*extended):
+        assert np.array_equal(a, b)
     all_, one = got[0], got[1]
     assert one[1][0] == all_[1][7]
     assert np.array_equal(one[0], all_[0][all_[0]["tmpl"] == 7])
+
+
+@pytest.mark.parametrize("lg", [10, 11, 12, 13, 14])
+def test_rounds_of_the_short_kernels(ctx, lg):
+    """More templates than the GPU holds at once: rows of the first round, the
+    second and a last one that ends within a CTA, against the oracle, and the
+    same bits as a search of that row alone."""
+    torch = pytest.importorskip("torch")
+    n, length = 1 << lg, 300
+    units = 2 * torch.cuda.get_device_properties(0).multi_processor_count * (1 << (14 - lg))
+    count = 2 * units + 3
+    bank = S.random_samples_bank(count, length, lg)
+    y = S.band_limited_noise(n, 9)
+    seg, bid = ctx.bege_load_segment(y), ctx.bege_define_bank_samples(bank)
+    job = ctx.bege_correlate(seg, bid, 0, count, 4.0)
+    recs, total = ctx.bege_fetch_tails(job, sort=True)
+    assert total == len(recs)
+    sigma = ctx.bege_get_sigma(job, count)
+    ctx.bege_release(job)
+    rows = [0, 1, units - 1, units, units + 17, 2 * units - 1, 2 * units, count - 2, count - 1]
+    _, want = oracle_rho(y, bank[rows])
+    for k, ref in zip(rows, want):
+        assert abs(sigma[k] / ref - 1) <= 1e-6
+        job = ctx.bege_correlate(seg, bid, k, k + 1, 4.0)
+        one, _ = ctx.bege_fetch_tails(job, sort=True)
+        assert ctx.bege_get_sigma(job, 1)[0] == sigma[k]
+        assert np.array_equal(one, recs[recs["tmpl"] == k])
+        ctx.bege_release(job)
+    ctx.bege_release(seg)
+    ctx.bege_release(bid)
