@@ -257,7 +257,8 @@ BEGE_API uint64_t bege_device_bytes(const bege_ctx* ctx);
 
 /* Launch shapes of the correlate kernel for segment length n.  A shape is
  * (columns per CTA, threads per CTA); the cluster holds (n / 8192) / columns
- * CTAs.  bege_list_configs writes up to `max` pairs into `out` as
+ * CTAs.  n <= 2^13 has one shape, listed as (1, 256): CTAs of 256 threads with
+ * several templates each.  bege_list_configs writes up to `max` pairs into `out` as
  * {nc0, threads0, nc1, threads1, ...} and the number available into *count. */
 BEGE_API int bege_list_configs(bege_ctx* ctx, int64_t n, int32_t* out, int32_t max, int32_t* count);
 

@@ -1,5 +1,5 @@
 // libbege C ABI: contexts, handles, memory accounting and job bookkeeping.
-// The arithmetic of the search lives in bege_kernels.cu; this file validates
+// The arithmetic of the search lives in the .cu files; this file validates
 // arguments, owns device memory and enqueues the kernels.
 #include <cuda_runtime.h>
 
@@ -528,6 +528,7 @@ static int batch_build(bege_ctx* ctx, Batch* b) {
       a.counter = sg.counter;
       a.dump = nullptr;
       a.max_clusters = 0;
+      // no exchange buffer: up to 40 MB would be the batch's as long as it lives
       if (b->plan == 1) e = bege::launch_correlate(pl->dev, a, cc, b->cs);
       if (e == cudaSuccess && en.large) e = bege::launch_range(pl->dev, a, b->cs);
     }

@@ -8,7 +8,7 @@ namespace bege {
 
 // One segment of a batch and the bank range it is correlated with.
 struct BatchSeg {
-  const float4* AB;            // product coefficients of the segment (residue-major)
+  const float4* AB;            // product coefficients, in the order the product reads them
   const float* bank;           // bank rows of Lp floats
   int64_t Lp;
   int64_t k0, k1;              // bank rows [k0, k1)

@@ -33,8 +33,9 @@
 //     T_b[n1] = wH^(-b n1) IFFT_F(Y_{S.+b})[n1].
 // Column b pairs with column S-b (bins j and H-j); columns {0, S/2} and
 // {i, S-i} form units.  A CTA owns whole units; the CTAs of a thread-block
-// cluster hold all S columns and read each other's columns through
-// distributed shared memory only in the final S-point combine.
+// cluster hold all S columns and exchange them only for the final S-point
+// combine, through distributed shared memory or, by default for N >= 2^16,
+// through a buffer in L2.
 //
 // This file: column maps, the tail epilogue and the launch; bege_unit.cuh has
 // the segment and correlate kernels, bege_corr_tc.cu the tensor-core form.
@@ -58,16 +59,16 @@ __host__ __device__ constexpr size_t align16(size_t x) { return (x + 15) & ~size
 
 extern __shared__ __align__(16) unsigned char smem_raw[];
 
-// Column ownership for S columns split over C = S/NC CTAs.
+// Column ownership for S >= 2 columns split over C = S/NC CTAs (this and the
+// pair items: the tensor-core form).
 template <int S, int NC>
 struct ColMap {
-  static_assert(S == 1 ? NC == 1 : (NC % 2 == 0 && S % NC == 0), "column split");
-  static constexpr int C = S == 1 ? 1 : S / NC;
-  static constexpr int UPC = S == 1 ? 1 : NC / 2;
+  static_assert(NC % 2 == 0 && S % NC == 0, "column split");
+  static constexpr int C = S / NC;
+  static constexpr int UPC = NC / 2;
   // column held by local slot c of CTA `rank`: unit u (u < S/2) holds columns
   // u and S-u, unit 0 columns 0 and S/2; a CTA holds NC/2 consecutive units
   static __device__ __forceinline__ int slot_column(int rank, int c) {
-    if constexpr (S == 1) return 0;
     const int ug = rank * (NC / 2) + (c >> 1);
     const int second = c & 1;
     if (ug == 0) return second ? S / 2 : 0;
@@ -76,16 +77,16 @@ struct ColMap {
   // owner rank and local slot of column b
   static __device__ __forceinline__ void home(int b, int* owner, int* slot) {
     int unit = 0, second = 0;
-    if (S > 1 && b == S / 2)
+    if (b == S / 2)
       second = 1;
     else if (b < S / 2)
       unit = b;
-    else if (S > 1) {
+    else {
       unit = S - b;
       second = 1;
     }
-    *owner = S == 1 ? 0 : unit / UPC;
-    *slot = S == 1 ? 0 : 2 * (unit % UPC) + second;
+    *owner = unit / UPC;
+    *slot = 2 * (unit % UPC) + second;
   }
 };
 
@@ -99,7 +100,7 @@ struct PairItem {
 
 template <int F, int S>
 __device__ __forceinline__ int unit_items(int ug) {
-  return ug == 0 ? (S >= 2 ? F + 1 : F / 2 + 1) : F;
+  return ug == 0 ? F + 1 : F;
 }
 
 template <int F, int S>
@@ -238,9 +239,9 @@ __device__ __forceinline__ void emit_row(const float2 (&t)[S], int n1, int H, fl
   }
 }
 
-// The S-point DFT across columns (column b at colptr[b], padded rows) and the
-// tails of CTA `rank`'s rows, thread `tix` of T.
-template <int F, int S, int NC, int T, bool EXT = false>
+// The tensor-core form's S-point DFT across columns (column b at colptr[b],
+// padded rows) and the tails, in the extended epilogue, of CTA `rank`'s rows, thread `tix` of T.
+template <int F, int S, int NC, int T>
 __device__ __forceinline__ void combine_and_emit(float2* const* colptr, int H, int rank, float thr,
                                                  uint32_t tmpl, int64_t krow, const TailOut& a,
                                                  float sigma, int tix = threadIdx.x) {
@@ -255,7 +256,7 @@ __device__ __forceinline__ void combine_and_emit(float2* const* colptr, int H, i
 #pragma unroll
     for (int b = 0; b < S; ++b) t[b] = colptr[b][pn1];
     dft<S, true>(t);
-    emit_row<S, F, EXT>(t, n1, H, thr, tmpl, krow, a, sigma);
+    emit_row<S, F, true>(t, n1, H, thr, tmpl, krow, a, sigma);
   }
 }
 

@@ -6,8 +6,8 @@
 
 namespace bege {
 
-// Shared-memory index with one padding slot every 16 complex values: keeps
-// the strided Stockham stores (stride 16 and 17*16) free of bank conflicts.
+// Shared-memory index with one padding slot every 16 complex values, for the
+// columns of the tensor-core form (rows 16 apart in different banks).
 __device__ __forceinline__ int pad(int i) { return i + (i >> 4); }
 
 template <int F>
@@ -160,8 +160,7 @@ __device__ __forceinline__ void dft16(float2 (&x)[16]) {
 
 template <int R, bool INV>
 __device__ __forceinline__ void dft(float2 (&x)[R]) {
-  if constexpr (R == 1) {
-  } else if constexpr (R == 2) {
+  if constexpr (R == 2) {
     dft2<INV>(x[0], x[1]);
   } else if constexpr (R == 4) {
     dft4<INV>(x[0], x[1], x[2], x[3]);

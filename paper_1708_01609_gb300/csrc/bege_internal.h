@@ -1,5 +1,5 @@
 // Internal interface between the C-ABI host layer (bege_api.cpp) and the
-// CUDA kernels (bege_kernels.cu).  Not part of the public ABI.
+// CUDA kernels (the .cu files).  Not part of the public ABI.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -19,19 +19,21 @@ namespace bege {
 // "column" b, an F-point FFT of a twiddled, folded input (a four-step whose
 // first step is pruned by the template's support).  Columns b and S-b hold
 // the bins j and H-j that the real-FFT unpacking couples, so they form a
-// "unit" processed by one CTA; the CTAs of a thread-block cluster share the
-// S columns and exchange them through distributed shared memory only for
-// the final S-point combine.
+// "unit" of one CTA; the CTAs of a thread-block cluster share the S columns and
+// exchange them only for the final S-point combine, through distributed shared
+// memory or (exchange_bytes) through L2.  H <= 4096 counts as one column here;
+// the FP32 kernels then work on two of half the length (UnitGeo).
 struct Geometry {
   int N;    // real samples
   int H;    // N / 2 complex samples
-  int F;    // column FFT length (512..4096)
-  int S;    // columns = H / F (1..16)
+  int F;    // min(H, 4096): the column length for N >= 2^14
+  int S;    // H / F (1..16)
 };
 
 // Launch shape of the correlate kernel: columns per CTA (the cluster has
 // S / nc CTAs) and threads per CTA.  Chosen per N by default or by the
-// autotuner.
+// autotuner.  S = 1 has one shape, listed as {1, 256}: 256 threads, as many
+// templates as they have units for.
 struct CorrConfig {
   int nc;
   int threads;

@@ -82,8 +82,8 @@ bool config_valid(const Geometry& g, CorrConfig c) {
 // SM, so half as many CTAs meet in a cluster and a unit's neighbour in the
 // CTA needs no distributed shared memory; S = 2 has one unit a template and
 // two CTAs per SM.  Per template (65536 chirps, GB300), 4 x 512 against 2 x
-// 256: N = 2^15 75.7 / 81.9 ns, 2^16 170.7 / 188.8, 2^17 405 / 411 (and 165 and
-// 354 with the exchange through L2, which takes this shape).
+// 256: N = 2^15 78 / 83 ns, 2^16 171 / 189, 2^17 405 / 420 (and 165 and 354 with
+// the exchange through L2, which takes this shape).
 CorrConfig default_config(const Geometry& g) {
   if (g.S == 1) return {1, 256};
   if (g.S == 2) return {2, 256};
@@ -164,8 +164,11 @@ cudaError_t launch_bank_large(const float* samples, int64_t n, int* flag, cudaSt
 // sin(2 pi phase / 2^64) at kKeep samples m0, m0 + d, m0 + 2 d, ...: the phase
 // alpha m + beta m^2 (cycles * 2^64, exact modulo one cycle) is quadratic in m,
 // so the unit phasor advances by a factor that itself advances by the constant
-// factor `turn` = exp(2 pi i 2 beta d^2); the two start values are exact
-// phases, and kKeep steps of FP64 products leave errors below 1e-14.
+// factor `turn` = exp(2 pi i 2 beta d^2).  The start values have exact phases.
+// After i <= 15 steps a sample holds i (i - 1) / 2 times the error of `turn`, i
+// times that of the first step and i (i + 1) / 2 roundings of a product, below
+// 1e-13 in all (1.2e-14 is the largest of 200000 random chirps): far below half
+// an FP32 ulp of a unit sine, so only rounding ties can differ.
 constexpr int kChirpThreads = 256;
 constexpr int kKeep = 16;
 

@@ -27,7 +27,7 @@
 //
 // Every stage works in place: a butterfly writes the 16 rows it read, so the
 // spectrum sits digit-reversed in shared memory, the product reads its
-// coefficients in the same order (coef_pos), and one ordering point between
+// coefficients in the same order (segment_unit), and one ordering point between
 // stages is enough.  Stages 2, 3, 3', 2' exchange values only between
 // threads of the same k0; warp w of a unit holds k0 = w and R - 1 - w (a column
 // bin's mirror has every digit complemented), so between them a warp waits
@@ -1148,8 +1148,8 @@ __global__ void __launch_bounds__(256 * U, U == 1 ? 2 : 1) unit_kernel(PlanDev p
 // neighbour's pace or for distributed shared memory.  The buffer holds two
 // templates of every unit: outputs of template k overwrite those of k - 2,
 // which every CTA combined before it arrived for k - 1.  Per template, this /
-// unit_kernel: N = 2^16 166 / 171 ns, 2^17 351 / 405 (at N = 2^15, one CTA a
-// template, 82 / 76).
+// unit_kernel: N = 2^16 165 / 171 ns, 2^17 354 / 405 (at N = 2^15, where one CTA
+// holds a template, it took 8% longer).
 template <int S, int U, bool HALFZ, bool EXT>
 __global__ void __launch_bounds__(256 * U, U == 1 ? 2 : 1)
 unit_exchange_kernel(PlanDev p, CorrelateArgs a) {
@@ -1228,8 +1228,8 @@ unit_exchange_kernel(PlanDev p, CorrelateArgs a) {
 // at work, where one column of N / 2 points per CTA of 256 threads left seven
 // eighths of them idle in the passes at N = 2^10; two units of 16 threads share
 // a warp there.  Per template (2^18 chirps of N samples at most, GB300),
-// against that kernel: N = 2^10 13.5 -> 2.3 ns, 2^11 16.5 -> 4.5, 2^12 23.6 ->
-// 9.2, 2^13 29.4 -> 19.0.
+// against that kernel: N = 2^10 13.5 -> 2.1 ns, 2^11 16.5 -> 4.5, 2^12 23.6 ->
+// 9.2, 2^13 29.4 -> 18.7.
 template <int F, bool HALFZ, bool EXT>
 __global__ void __launch_bounds__(256, 2) short_kernel(PlanDev p, CorrelateArgs a) {
   constexpr int U = 4096 / F;
