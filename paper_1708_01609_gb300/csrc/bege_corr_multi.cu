@@ -7,7 +7,7 @@
 // exactly the single-segment kernel's arithmetic.  Bound by latency beside the
 // single kernel's FP32 work: a segment begins with 64 KB of spectrum and 96 KB
 // of coefficients per unit from L2, as 16-byte loads (as 8-byte ones 199 ns per
-// correlation at N = 2^16 and M = 8, now 150; the single kernel 165).
+// correlation at N = 2^16 and M = 8, now 151; the single kernel 165).
 #include "bege_unit.cuh"
 
 namespace bege {
