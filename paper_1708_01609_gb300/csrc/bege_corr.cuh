@@ -303,15 +303,17 @@ static cudaError_t resident_clusters(int C, int threads, size_t smem, int minb, 
 }
 
 // Launches `kern` with clusters of C CTAs (minb CTAs per SM), as many as fit
-// and are needed for the templates of a, `each` at a time per cluster.
-template <auto kern>
+// and are needed for the templates of a, `each` at a time per cluster.  BEHIND:
+// the kernel is made ready while the one before it runs, for which it waits
+// itself (cudaGridDependencySynchronize): 2 to 3 us less for a range kernel.
+template <auto kern, bool BEHIND = false>
 static cudaError_t launch_clusters(int C, int threads, size_t smem, int minb, int each,
                                    const PlanDev& p, const CorrelateArgs& a, cudaStream_t s) {
   int clusters = 0;
   cudaError_t e = resident_clusters<kern>(C, threads, smem, minb, &clusters);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = (unsigned)C;
   attr[0].val.clusterDim.y = 1;
@@ -325,6 +327,11 @@ static cudaError_t launch_clusters(int C, int threads, size_t smem, int minb, in
   if (a.max_clusters > 0 && want > a.max_clusters) want = a.max_clusters;
   if (want > clusters) want = clusters;
   cfg.gridDim = dim3((unsigned)(want * C), 1, 1);
+  if (BEHIND) {
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.numAttrs = 2;
+  }
   return cudaLaunchKernelEx(&cfg, kern, p, a);
 }
 

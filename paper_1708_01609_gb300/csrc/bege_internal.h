@@ -132,7 +132,7 @@ inline __host__ __device__ float2 rot_entry(double c, double s) {
 Geometry make_geometry(int64_t n);
 
 // The tables of geometry g in an array of plan_floats2(g) float2 at `base`,
-// and the kernel that writes them there.
+// and the kernel that writes them there, and 0 to *zero if given.
 constexpr __host__ __device__ int plan_floats2(const Geometry& g) {
   const UnitGeo u = unit_geo(g);
   int n = u.S + g.H;
@@ -140,7 +140,8 @@ constexpr __host__ __device__ int plan_floats2(const Geometry& g) {
   return n;
 }
 PlanDev plan_at(const Geometry& g, float2* base);
-cudaError_t launch_plan_tables(const Geometry& g, float2* base, cudaStream_t s);
+cudaError_t launch_plan_tables(const Geometry& g, float2* base, cudaStream_t s,
+                               unsigned long long* zero = nullptr);
 
 // Record `msg` as the calling thread's last error (bege_last_error) and
 // return `code`.

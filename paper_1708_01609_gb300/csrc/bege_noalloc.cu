@@ -85,13 +85,12 @@ extern "C" int bege_search_noalloc(const float* strain_dev, int64_t n, const flo
     // call's kernels: the host keeps no record of which n the array holds,
     // which could disagree with the device's order of work.
     float2* const tables = reinterpret_cast<float2*>(base + kOffTables);
-    e = launch_plan_tables(g, tables, s);
+    e = launch_plan_tables(g, tables, s, tail_count_dev);
     if (e != cudaSuccess) return set_last_error(BEGE_ECUDA, cudaGetErrorString(e));
     const PlanDev p = plan_at(g, tables);
     float4* AB = reinterpret_cast<float4*>(base + kOffAB);
     float2* D = reinterpret_cast<float2*>(base + kOffD);
     e = launch_segment(p, strain_dev, D, AB, false, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(tail_count_dev, 0, sizeof(unsigned long long), s);
     if (e == cudaSuccess) {
       CorrelateArgs a{};
       a.AB = AB;

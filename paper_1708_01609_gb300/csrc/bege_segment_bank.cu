@@ -30,8 +30,10 @@ PlanDev plan_at(const Geometry& g, float2* base) {
 }
 
 // One table entry per thread (plan_at's order).
-__global__ void __launch_bounds__(256) plan_tables_kernel(Geometry g, float2* __restrict__ base) {
+__global__ void __launch_bounds__(256)
+plan_tables_kernel(Geometry g, float2* __restrict__ base, unsigned long long* zero) {
   int i = blockIdx.x * 256 + threadIdx.x;
+  if (i == 0 && zero) *zero = 0;
   if (i >= plan_floats2(g)) return;
   float2* const out = base + i;
   const UnitGeo u = unit_geo(g);
@@ -50,8 +52,9 @@ __global__ void __launch_bounds__(256) plan_tables_kernel(Geometry g, float2* __
   *out = make_float2((float)c, (float)s);
 }
 
-cudaError_t launch_plan_tables(const Geometry& g, float2* base, cudaStream_t s) {
-  plan_tables_kernel<<<(plan_floats2(g) + 255) / 256, 256, 0, s>>>(g, base);
+cudaError_t launch_plan_tables(const Geometry& g, float2* base, cudaStream_t s,
+                               unsigned long long* zero) {
+  plan_tables_kernel<<<(plan_floats2(g) + 255) / 256, 256, 0, s>>>(g, base, zero);
   return cudaGetLastError();
 }
 

@@ -1317,6 +1317,7 @@ __device__ __forceinline__ bool range_rows(const CorrelateArgs& a, int64_t g, in
   *r0 = g * per;
   *r1 = *r0 + per < count ? *r0 + per : count;
   bool bad = false;
+  cudaGridDependencySynchronize();  // the search
   for (int64_t r = *r0 + threadIdx.x; r < *r1; r += blockDim.x)
     bad |= !(__ldcg(a.sigma + r) <= kMaxFinite);
   return __syncthreads_or(bad);
@@ -1441,10 +1442,10 @@ static cudaError_t launch_range(const PlanDev& p, const CorrelateArgs& a, cudaSt
   constexpr size_t smem = Lay<kF, 2, false>::total;
   const bool ext = extended(p, a);
   if (a.Lp <= kF)
-    return ext ? launch_clusters<range_kernel<S, true, true>>(C, 512, smem, 1, 1, p, a, s)
-               : launch_clusters<range_kernel<S, true, false>>(C, 512, smem, 1, 1, p, a, s);
-  return ext ? launch_clusters<range_kernel<S, false, true>>(C, 512, smem, 1, 1, p, a, s)
-             : launch_clusters<range_kernel<S, false, false>>(C, 512, smem, 1, 1, p, a, s);
+    return ext ? launch_clusters<range_kernel<S, true, true>, true>(C, 512, smem, 1, 1, p, a, s)
+               : launch_clusters<range_kernel<S, true, false>, true>(C, 512, smem, 1, 1, p, a, s);
+  return ext ? launch_clusters<range_kernel<S, false, true>, true>(C, 512, smem, 1, 1, p, a, s)
+             : launch_clusters<range_kernel<S, false, false>, true>(C, 512, smem, 1, 1, p, a, s);
 }
 
 template <int F, bool HALFZ>
@@ -1452,8 +1453,8 @@ static cudaError_t launch_range_short(const PlanDev& p, const CorrelateArgs& a, 
   constexpr int U = 4096 / F;
   constexpr size_t smem = Lay<F, U, true>::total;
   return extended(p, a)
-             ? launch_clusters<range_short_kernel<F, HALFZ, true>>(1, 256, smem, 2, U, p, a, s)
-             : launch_clusters<range_short_kernel<F, HALFZ, false>>(1, 256, smem, 2, U, p, a, s);
+             ? launch_clusters<range_short_kernel<F, HALFZ, true>, true>(1, 256, smem, 2, U, p, a, s)
+             : launch_clusters<range_short_kernel<F, HALFZ, false>, true>(1, 256, smem, 2, U, p, a, s);
 }
 
 }  // namespace unit
