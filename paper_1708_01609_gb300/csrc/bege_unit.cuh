@@ -734,7 +734,6 @@ __device__ __forceinline__ void segment_unit(const PlanDev& p, int S, int ug,
                                              float4* __restrict__ AB, bool natural, int part = 0,
                                              int parts = 1) {
   constexpr int R = SM::G::R, T = SM::G::T, F = 256 * R;
-  const int H = S * F;
   auto bin = [&](int b, int k0, int k1, int k2) { return S * (k0 + R * k1 + 16 * R * k2) + b; };
   // thread t of slot h (column h of the unit, in the middle za or zb)
   const int t = SM::tid(), h = ((int)threadIdx.x / T) & 1;
